@@ -208,6 +208,14 @@ cudaError_t launch_map_pass(const DevCtx& c, const PrefillArgs& a, cudaStream_t 
 cudaError_t launch_decode_attn(const DevCtx& c, const DecBatch& b, int layer_begin, int layer_count, int n_seqs_total,
                                const __nv_bfloat16* q, __nv_bfloat16* out, int nsplit, cudaStream_t s);
 
+// a whole decode step in one launch, clusters of `cluster` CTAs (a power of two up to 16) per (sequence, layer, KV head);
+// contexts without collaborative voting.  indexed_end: end of the indexed prefix (the largest of the batch).
+int dec_step_capacity(const DevCtx& c, int cluster);  // CTAs that run at once (0: this cluster size is not available)
+bool dec_step_fits(const DevCtx& c, int span_bound, int indexed_end, int cluster);
+cudaError_t launch_dec_step(const DevCtx& c, const DecBatch& b, int layer_begin, int layer_count, const __nv_bfloat16* q,
+                            const __nv_bfloat16* k, const __nv_bfloat16* v, __nv_bfloat16* out, int span_bound,
+                            int indexed_end, int cluster, cudaStream_t s);
+
 // test kernel for the bounded waits: one wait with `short_limit` cycles on a barrier nothing completes (kernels_probe.cu)
 cudaError_t launch_wait_probe(const DevCtx& c, long long short_limit, cudaStream_t s);
 

@@ -2,22 +2,11 @@
 // token ranges [sink | selected spans | tokens since the last eviction].  Every K/V row is read once with 16-byte
 // loads and shared by the G query heads of its KV group; softmax reductions use warp shuffles.
 #include "common.cuh"
-#include "mma_util.cuh"
+#include "decode_util.cuh"
 
 namespace ltri {
 
-constexpr float kLog2eD = 1.4426950408889634f;
 constexpr int kDecThreads = 128;  // 4 warps = 8 half-warps, each half-warp owns one token at a time
-
-__device__ __forceinline__ void unpack8(const uint4& raw, float (&f)[8]) {
-  const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 t = __bfloat1622float2(p[i]);
-    f[2 * i] = t.x;
-    f[2 * i + 1] = t.y;
-  }
-}
 
 // grid (nsplit, Hkv, b.n*layer_count), 4 warps.  Each warp walks 16-token tiles of the CTA's slice of the virtual
 // token list (sink | selected spans | recent tokens): the tile's K and V rows (two contiguous 256-byte rows per
@@ -25,7 +14,6 @@ __device__ __forceinline__ void unpack8(const uint4& raw, float (&f)[8]) {
 // m16n8k16 tensor-core MMAs with the G query heads of the group in the first rows of the 16-row operand, so the
 // per-token ALU cost is a handful of instructions and the kernel stays bound by the K/V stream.
 // Partial results (m, l, O[128]) per (unit, head, split) go to dec_part.
-constexpr int kDTile = 16;
 constexpr int kDStages = 2;     // two stages of 8 KB per warp: three CTAs (12 warps) fit an SM, which hides more latency
 constexpr int kDecCtasPerSm = 3;  // than a deeper ring at two CTAs per SM
 constexpr int kDWarpBytes = kDStages * 2 * kDTile * 256;  // K and V rows of every stage
@@ -109,10 +97,8 @@ __global__ void __launch_bounds__(kDecThreads, kDecCtasPerSm) k_decode_attn(DevC
     }
   };
 
-  float O[16][4];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) O[i][0] = O[i][1] = O[i][2] = O[i][3] = 0.f;
-  float m = -INFINITY, lsum = 0.f;
+  DecAcc acc;
+  acc.clear();
 
   // tiles of this warp: warp, warp + 4, ...
   const int my_tiles = ntiles > warp ? (ntiles - warp + 3) / 4 : 0;
@@ -129,65 +115,21 @@ __global__ void __launch_bounds__(kDecThreads, kDecCtasPerSm) k_decode_attn(DevC
     __syncwarp();
     const uint32_t sk = wbase + stage * (2 * kDTile * 256), sv = sk + kDTile * 256;
     const int vb = v0 + (warp + 4 * it) * kDTile;
-    float S[2][4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) S[i][0] = S[i][1] = S[i][2] = S[i][3] = 0.f;
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-      uint32_t bf[4];
-      ldsm_x4(bf, sk + tile_off((lane & 7) + ((lane >> 4) << 3), ks * 2 + ((lane >> 3) & 1)));
-      const uint32_t a[4] = {qa[ks][0], 0u, qa[ks][1], 0u};
-      mma_bf16(S[0], a, bf[0], bf[1]);
-      mma_bf16(S[1], a, bf[2], bf[3]);
-    }
-    // row r of this lane: tokens nt*8 + 2*qd + e
-    float tmax = -INFINITY;
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        if (vb + nt * 8 + 2 * qd + e >= v1) S[nt][e] = -INFINITY;
-        tmax = fmaxf(tmax, S[nt][e]);
-      }
-    tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
-    tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
-    const float mnew = fmaxf(m, tmax * c2);
-    const float mu = mnew == -INFINITY ? 0.f : mnew;
-    const float alpha = exp2f(m - mu);
-    m = mnew;
-    float p[2][2];
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) p[nt][e] = exp2f(fmaf(S[nt][e], c2, -mu));
-    lsum = lsum * alpha + (p[0][0] + p[0][1] + p[1][0] + p[1][1]);
-#pragma unroll
-    for (int nt = 0; nt < 16; ++nt) {
-      O[nt][0] *= alpha;
-      O[nt][1] *= alpha;
-    }
-    const uint32_t pa[4] = {pack_bf16(p[0][0], p[0][1]), 0u, pack_bf16(p[1][0], p[1][1]), 0u};
-#pragma unroll
-    for (int dp = 0; dp < 8; ++dp) {
-      uint32_t bf[4];
-      ldsm_x4_t(bf, sv + tile_off((lane & 7) + (((lane >> 3) & 1) << 3), dp * 2 + (lane >> 4)));
-      mma_bf16(O[2 * dp], pa, bf[0], bf[1]);
-      mma_bf16(O[2 * dp + 1], pa, bf[2], bf[3]);
-    }
+    dec_tile_16(acc, qa, sk, sv, v1 - vb, c2, lane);
     __syncwarp();
   }
   cp_async_wait<0>();
-  lsum += __shfl_xor_sync(0xffffffffu, lsum, 1);
-  lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
+  acc.lsum += __shfl_xor_sync(0xffffffffu, acc.lsum, 1);
+  acc.lsum += __shfl_xor_sync(0xffffffffu, acc.lsum, 2);
   if (r < G) {
     if (qd == 0) {
-      sm_m[warp][r] = m;
-      sm_l[warp][r] = lsum;
+      sm_m[warp][r] = acc.m;
+      sm_l[warp][r] = acc.lsum;
     }
 #pragma unroll
     for (int nt = 0; nt < 16; ++nt) {
-      sm_o[warp][r][nt * 8 + 2 * qd] = O[nt][0];
-      sm_o[warp][r][nt * 8 + 2 * qd + 1] = O[nt][1];
+      sm_o[warp][r][nt * 8 + 2 * qd] = acc.O[nt][0];
+      sm_o[warp][r][nt * 8 + 2 * qd + 1] = acc.O[nt][1];
     }
   }
   __syncthreads();

@@ -241,6 +241,8 @@ struct ltri_ctx {
   int sm_count = 148;
   bool use_tc = false;     // tcgen05/TMEM/TMA attention kernels (default when available)
   int dec_fused = -1;      // decode retrieval in one launch: -1 auto, 0 never, 1 whenever the index fits, 2 cluster kernel
+  int step_cap[5] = {0, 0, 0, 0, 0};  // one-launch decode step: CTAs that run at once as clusters of 1 << i
+  int step_cluster = 0;    // testing aid (LTRI_DEC_CLUSTER): 0 auto, otherwise the cluster size of the one-launch step
   // host-buffer entry (LTRI_FLAG_HOST_STAGING): two staging sets in the arena, a copy-up and a copy-down stream, and
   // events that order every reuse of a set's layer-group slices
   static constexpr int kHostGroups = 4;
@@ -418,8 +420,12 @@ int ltri_create(const ltri_params* p, void* cuda_stream, ltri_ctx** out) {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) ctx->sm_count = sms;
   }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  // testing aid: 0 two launches, 1 one launch, 2 one launch with the cluster kernel whatever the index size
+  // testing aid for the retrieval of a decode step: 0 two launches, 1 one launch, 2 one launch with the cluster kernel
+  // whatever the index size (any of them keeps the one-launch step out)
   if (const char* f = std::getenv("LTRI_DEC_FUSED")) ctx->dec_fused = std::max(0, std::min(2, std::atoi(f)));
+  if (const char* f = std::getenv("LTRI_DEC_CLUSTER")) ctx->step_cluster = std::atoi(f);
+  if (ctx->dec_fused < 0 && !ctx->d.vote)
+    for (int i = 1; i < 5; ++i) ctx->step_cap[i] = dec_step_capacity(ctx->d, 1 << i);
   const char* impl = std::getenv("LTRI_ATTN_IMPL");  // "mma" selects the warp-MMA kernels (debugging aid)
   ctx->use_tc = tc_attention_supported(ctx->d) && !(impl && std::strcmp(impl, "mma") == 0) &&
                 tc_encode_kv_maps(ctx->d, ctx->kv_maps);
@@ -838,6 +844,29 @@ int ltri_host_outputs_ready(ltri_ctx* ctx, void* cuda_stream) {
   return LTRI_OK;
 }
 
+// Cluster size of the one-launch decode step, 0 when the step runs as separate launches: the largest power of two
+// whose clusters all run at once and that leaves a CTA at least 64 of the tokens known on the host.  A CTA scans at
+// most kStepSpans spans of the index: a longer scan is bound by the memory, and the separate launches, whose retriever
+// holds no shared memory for tiles and leaves more CTAs per SM to hide the latency, stream it faster (33K spans, 32
+// units: 92 against 103 us a step).
+constexpr int kStepSpans = 2560;
+static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, long long ub) {
+  const DevCtx& d = ctx->d;
+  int e_max = 0;
+  long long known = 1;
+  for (int i = 0; i < b.n; ++i) {
+    e_max = std::max(e_max, b.loc_begin[i]);
+    known = std::max(known, (long long)d.Ls + b.pos[i] + 1 - b.loc_begin[i]);
+  }
+  for (int i = 4; i >= 1; --i) {
+    const int cl = 1 << i;
+    if (ctx->step_cluster > 0 ? cl != ctx->step_cluster : known / cl < 64 && cl > 2) continue;
+    if (ctx->step_cluster == 0 && d.unit == 0 && ub > (long long)kStepSpans * cl) continue;
+    if ((long long)units * cl <= ctx->step_cap[i] && dec_step_fits(d, (int)ub, e_max, cl)) return cl;
+  }
+  return 0;
+}
+
 int ltri_decode_step(ltri_ctx* ctx, const int32_t* seq_ids, int n_seqs, int layer_begin, int layer_count,
                      const void* q, const void* k, const void* v, void* out, void* cuda_stream) {
   if (!ctx || !seq_ids) return LTRI_EINVAL;
@@ -896,6 +925,13 @@ int ltri_decode_step(ltri_ctx* ctx, const int32_t* seq_ids, int n_seqs, int laye
       b.shift[i] = d.paged ? s.base - d.Lsp : 0;
     }
     const int units = b.n * layer_count * d.Hkv;
+    if (const int cl = step_cluster_size(ctx, b, units, ub)) {
+      int e_max = 0;
+      for (int i = 0; i < b.n; ++i) e_max = std::max(e_max, b.loc_begin[i]);
+      Scope sc(ctx, st, LTRI_K_DEC_ATTN, 1);
+      LTRI_CUDA(ctx, launch_dec_step(d, b, layer_begin, layer_count, qb, kb, vb, ob, (int)ub, e_max, cl, st));
+      continue;
+    }
     // split count of the decode attention: three CTAs fit an SM, so the grid runs in waves of 3 x SMs CTAs.  Among
     // the split counts that leave a CTA at least ~512 tokens (of the tokens known on the host: sink + everything
     // since the last eviction) take the one whose last wave is fullest; ties go to fewer, longer slices.
