@@ -235,19 +235,27 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                  Args&&... args) {
+inline cudaError_t launch_chained_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem,
+                                          cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                  Args&&... args) {
+  return launch_chained_cluster(kernel, grid, block, 1, smem, s, static_cast<Args&&>(args)...);
 }
 #endif
 
@@ -277,9 +285,26 @@ __device__ __forceinline__ long long shfl_ll(long long v, int src) {
 __device__ inline int select_reps(const long long* __restrict__ votes, int start, int len, int reps, int* toks) {
   const int lane = threadIdx.x & 31;
   int cnt = reps < len ? reps : len;
+  // spans of up to 256 tokens: every lane's votes are read once, all of them in flight, and kept for all rounds
+  constexpr int kHeld = 8;
+  const long long kNone = (long long)0x8000000000000000ull;
+  long long held[kHeld];
+  const bool inreg = len <= 32 * kHeld;
+  if (inreg) {
+#pragma unroll
+    for (int k = 0; k < kHeld; ++k) held[k] = k * 32 + lane < len ? votes[start + k * 32 + lane] : kNone;
+  }
   for (int r = 0; r < cnt; ++r) {
     long long bv = (long long)0x8000000000000000ull;
     int bi = 0x7fffffff;
+    if (inreg) {
+#pragma unroll
+      for (int k = 0; k < kHeld; ++k)
+        if (held[k] > bv) {  // (ascending tokens: an equal one does not replace)
+          bv = held[k];
+          bi = start + k * 32 + lane;
+        }
+    } else
     for (int i = lane; i < len; i += 32) {
       int tok = start + i;
       bool used = false;
@@ -301,6 +326,11 @@ __device__ inline int select_reps(const long long* __restrict__ votes, int start
       }
     }
     toks[r] = bi;
+    if (inreg) {
+#pragma unroll
+      for (int k = 0; k < kHeld; ++k)
+        if (start + k * 32 + lane == bi) held[k] = kNone;
+    }
   }
   for (int a = 1; a < cnt; ++a) {  // insertion sort, ascending token
     int x = toks[a], b = a - 1;

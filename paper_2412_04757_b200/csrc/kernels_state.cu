@@ -249,17 +249,20 @@ __device__ __forceinline__ unsigned log_bin(unsigned v) {
   return ((unsigned)e << 4) | frac;
 }
 
-constexpr int kThetaCluster = 8;   // CTAs (one thread-block cluster) per layer
 constexpr int kThetaThreads = 512;
 
-__global__ void __cluster_dims__(kThetaCluster, 1, 1) __launch_bounds__(kThetaThreads)
+// H > 0: the cluster has a warp for every pair of rows (i, m - 1 - i) of the map, m + 1 entries in all, and a lane keeps
+// its (at most H) entries in registers, so the map is read once and every pass counts from registers.  H = 0: any
+// size, every pass reads the map.
+template <int H>
+__global__ void __launch_bounds__(H > 0 ? 1024 : kThetaThreads)
     k_theta_select(DevCtx c, int layer_begin, int m, long long rank, int tables) {
   chain_wait();
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ unsigned hist[];  // [warps][kThetaBins]
-  constexpr int NW = kThetaThreads / 32;
-  const int layer = layer_begin + blockIdx.x / kThetaCluster;
+  const int CL = (int)cluster.num_blocks(), NW = blockDim.x >> 5;
+  const int layer = layer_begin + blockIdx.x / CL;
   const int part = (int)cluster.block_rank();
   if (tables && c.theta_l) {  // the layer's own quantile level: the same double arithmetic as on the host
     const long long N = (long long)m * (m + 1) / 2;
@@ -267,54 +270,76 @@ __global__ void __cluster_dims__(kThetaCluster, 1, 1) __launch_bounds__(kThetaTh
     rank = rank < 0 ? 0 : (rank > N - 1 ? N - 1 : rank);
   }
   const int* Mq = c.Mq + (size_t)layer * c.chunk * c.chunk;
-  __shared__ unsigned loc[kThetaBins + 2];  // this CTA's histogram, then its counts of negatives and zeros
-  __shared__ unsigned tot[kThetaBins];      // the cluster's histogram (every CTA builds its own copy)
-  __shared__ unsigned s_red[NW][2];
+  // this CTA's histogram, then its counts of negatives and zeros: two copies that the passes use in turn, so that one
+  // cluster barrier per pass is enough
+  __shared__ unsigned loc[2][kThetaBins + 2];
+  __shared__ unsigned tot[kThetaBins];  // the cluster's histogram (every CTA builds its own copy)
+  __shared__ unsigned s_red[32][2];
   __shared__ unsigned s_prefix, s_lo_bits;
   __shared__ long long s_rank, s_cn, s_cz;
   __shared__ int s_cls;  // 0: answer found, 1: among positives (bin chosen), -1: among negatives
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned* myhist = hist + warp * kThetaBins;
-  // sums the per-warp histograms into loc, then the cluster's loc arrays into tot.  The second cluster barrier keeps
-  // every CTA's loc intact until all have read it (and keeps a CTA from exiting while it can still be read).
+  int held[H > 0 ? H : 1];
+  const int pair = part * NW + warp;  // rows pair and m - 1 - pair
+  const int na = 2 * pair < m ? pair + 1 : 0, nb = 2 * pair < m && pair != m - 1 - pair ? m - pair : 0;
+  if (H > 0) {
+    const int* ra = Mq + (size_t)pair * c.chunk;
+    const int* rb = Mq + (size_t)(m - 1 - pair) * c.chunk - na;
+#pragma unroll
+    for (int t = 0; t < H; ++t) {
+      const int k = t * 32 + lane;
+      held[t] = k < na + nb ? (k < na ? ra[k] : rb[k]) : 0;
+    }
+  }
+  auto visit = [&](auto&& f) {
+    if (H > 0) {
+#pragma unroll
+      for (int t = 0; t < H; ++t)
+        if (t * 32 + lane < na + nb) f(held[t]);
+    } else {
+      for_each_causal(Mq, c.chunk, m, part, CL, f);
+    }
+  };
+  int pass = 0;
+  // sums the per-warp histograms into loc, then the cluster's loc arrays into tot
   auto combine = [&](bool with_counts) {
+    unsigned* mine = loc[pass & 1];
     __syncthreads();
     if (threadIdx.x < kThetaBins) {
       unsigned sum = 0;
+#pragma unroll 8
       for (int w = 0; w < NW; ++w) sum += hist[w * kThetaBins + threadIdx.x];
-      loc[threadIdx.x] = sum;
+      mine[threadIdx.x] = sum;
     }
-    if (with_counts && threadIdx.x == 0) {
-      unsigned cn = 0, cz = 0;
-      for (int w = 0; w < NW; ++w) {
-        cn += s_red[w][0];
-        cz += s_red[w][1];
-      }
-      loc[kThetaBins] = cn;
-      loc[kThetaBins + 1] = cz;
+    if (with_counts && threadIdx.x < 2) {
+      unsigned n = 0;
+      for (int w = 0; w < NW; ++w) n += s_red[w][threadIdx.x];
+      mine[kThetaBins + threadIdx.x] = n;
     }
     cluster.sync();
     if (threadIdx.x < kThetaBins) {
       unsigned sum = 0;
-      for (int r = 0; r < kThetaCluster; ++r) sum += cluster.map_shared_rank(loc, r)[threadIdx.x];
+#pragma unroll 8
+      for (int r = 0; r < CL; ++r) sum += cluster.map_shared_rank(mine, r)[threadIdx.x];
       tot[threadIdx.x] = sum;
     }
-    if (with_counts && threadIdx.x == 0) {
-      long long cn = 0, cz = 0;
-      for (int r = 0; r < kThetaCluster; ++r) {
-        const unsigned* rl = cluster.map_shared_rank(loc, r);
-        cn += rl[kThetaBins];
-        cz += rl[kThetaBins + 1];
-      }
-      s_cn = cn;
-      s_cz = cz;
+    if (with_counts && threadIdx.x < 2) {
+      long long n = 0;
+#pragma unroll 8
+      for (int r = 0; r < CL; ++r) n += cluster.map_shared_rank(mine, r)[kThetaBins + threadIdx.x];
+      if (threadIdx.x == 0)
+        s_cn = n;
+      else
+        s_cz = n;
     }
-    cluster.sync();
+    ++pass;
+    __syncthreads();
   };
   for (int t = threadIdx.x; t < NW * kThetaBins; t += blockDim.x) hist[t] = 0;
   __syncthreads();
   unsigned nneg = 0, nzero = 0;
-  for_each_causal(Mq, c.chunk, m, part, kThetaCluster, [&](int v) {
+  visit([&](int v) {
     if (v > 0)
       atomicAdd(&myhist[log_bin((unsigned)v)], 1u);
     else if (v == 0)
@@ -322,11 +347,8 @@ __global__ void __cluster_dims__(kThetaCluster, 1, 1) __launch_bounds__(kThetaTh
     else
       ++nneg;
   });
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    nneg += __shfl_xor_sync(0xffffffffu, nneg, o);
-    nzero += __shfl_xor_sync(0xffffffffu, nzero, o);
-  }
+  nneg = __reduce_add_sync(0xffffffffu, nneg);
+  nzero = __reduce_add_sync(0xffffffffu, nzero);
   if (lane == 0) {
     s_red[warp][0] = nneg;
     s_red[warp][1] = nzero;
@@ -364,18 +386,17 @@ __global__ void __cluster_dims__(kThetaCluster, 1, 1) __launch_bounds__(kThetaTh
   }
   __syncthreads();
   const int cls = s_cls;
-  if (cls == 0) return;  // the same decision in every CTA of the cluster
   // remaining bits: [0, hi).  Negatives: plain MSB radix over the sign-flipped key.
-  int hi = cls > 0 ? (int)s_lo_bits : 31;
+  int hi = cls > 0 ? (int)s_lo_bits : (cls < 0 ? 31 : 0);
   if (cls < 0 && threadIdx.x == 0) s_prefix = 0;
   __syncthreads();
-  while (hi > 0) {
+  while (hi > 0) {  // (the same decisions in every CTA of the cluster)
     const int lo = max(0, hi - kThetaBits);
     const unsigned dmask = (1u << (hi - lo)) - 1u;
     for (int t = threadIdx.x; t < NW * kThetaBins; t += blockDim.x) hist[t] = 0;
     __syncthreads();
     const unsigned prefix = s_prefix;
-    for_each_causal(Mq, c.chunk, m, part, kThetaCluster, [&](int v) {
+    visit([&](int v) {
       const bool in_cls = cls > 0 ? v > 0 : v < 0;
       const unsigned key = cls > 0 ? (unsigned)v : ((unsigned)v ^ 0x80000000u);
       if (in_cls && (key >> hi) == (prefix >> hi)) atomicAdd(&myhist[(key >> lo) & dmask], 1u);
@@ -393,8 +414,9 @@ __global__ void __cluster_dims__(kThetaCluster, 1, 1) __launch_bounds__(kThetaTh
     __syncthreads();
     hi = lo;
   }
-  if (threadIdx.x == 0 && part == 0)
+  if (cls != 0 && threadIdx.x == 0 && part == 0)
     c.thetaq[layer] = cls > 0 ? (long long)s_prefix : (long long)(int)(s_prefix ^ 0x80000000u);
+  cluster.sync();  // nobody leaves while its histogram may still be read
 }
 
 // absolute threshold: thq in units of the map summed over all heads, thq1 in units of a single (retrieval) head's map;
@@ -409,7 +431,10 @@ __global__ void k_theta_set(DevCtx c, int layer_begin, long long thq, long long 
 }
 
 // step 2: suffix sums along each row of D = Mq - theta ("sum the right elements", Fig. 2):
-// Rsuf[i][x] = sum_{j=x..i} D[i][j].  One warp per row, 32-wide shuffle scans from the diagonal leftwards.
+// Rsuf[i][x] = sum_{j=x..i} D[i][j].  One warp per row.  A lane holds four consecutive entries of every block of 128, all
+// of them requested before the first is used (one load at a time, a row of 1024 was 32 dependent round trips: 24 us for
+// one layer's map); B = blocks of 128 in a row.
+template <int B>
 __global__ void __launch_bounds__(256) k_seg_rowscan(DevCtx c, int layer_begin, int m) {
   chain_wait();
   const int layer = layer_begin + blockIdx.y;
@@ -418,96 +443,130 @@ __global__ void __launch_bounds__(256) k_seg_rowscan(DevCtx c, int layer_begin, 
   if (blockIdx.x == 0)
     for (int t = threadIdx.x; t < 2 * c.chunk; t += blockDim.x) c.best[(size_t)layer * 2 * c.chunk + t] = 0;
   if (i >= m) return;
-  const long long thq = c.thetaq[layer];
   const int* row = c.Mq + ((size_t)layer * c.chunk + i) * c.chunk;
   long long* out = c.Rsuf + ((size_t)layer * c.chunk + i) * c.chunk;
+  // 16-byte accesses need rows that start on 16 bytes and whose groups of four never leave them: always so in a context
+  // (chunk is a multiple of 16), not for a caller's dense map of any size and alignment
+  const bool vec = (c.chunk & 3) == 0 && (reinterpret_cast<uintptr_t>(c.Mq) & 15) == 0;
+  int4 v[B];
+#pragma unroll
+  for (int k = 0; k < B; ++k) {
+    const int x = k * 128 + lane * 4;
+    v[k] = make_int4(0, 0, 0, 0);
+    if (vec) {
+      if (x <= i) v[k] = *reinterpret_cast<const int4*>(row + x);
+    } else {
+      if (x <= i) v[k].x = row[x];
+      if (x + 1 <= i) v[k].y = row[x + 1];
+      if (x + 2 <= i) v[k].z = row[x + 2];
+      if (x + 3 <= i) v[k].w = row[x + 3];
+    }
+  }
+  const long long thq = c.thetaq[layer];
   long long carry = 0;
-  for (int hi = i; hi >= 0; hi -= 32) {
-    const int x = hi - lane;  // lane 0 is the rightmost element of this group
-    long long v = x >= 0 ? (long long)row[x] - thq : 0;
+#pragma unroll
+  for (int k = B - 1; k >= 0; --k) {
+    if (k * 128 > i) continue;  // (uniform over the warp)
+    const int x = k * 128 + lane * 4;
+    long long s3 = x + 3 <= i ? (long long)v[k].w - thq : 0;
+    long long s2 = s3 + (x + 2 <= i ? (long long)v[k].z - thq : 0);
+    long long s1 = s2 + (x + 1 <= i ? (long long)v[k].y - thq : 0);
+    long long s0 = s1 + (x <= i ? (long long)v[k].x - thq : 0);
+    long long inc = s0;  // sum over this lane's entries and those of the lanes to its right
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const long long t = shfl_up_ll(v, o);
-      if (lane >= o) v += t;
+      const long long t = __shfl_down_sync(0xffffffffu, inc, o);
+      if (lane + o < 32) inc += t;
     }
-    v += carry;
-    if (x >= 0) out[x] = v;
-    carry = shfl_ll(v, 31);
+    const long long right = carry + inc - s0;
+    if (vec) {
+      if (x <= i) {
+        *reinterpret_cast<longlong2*>(out + x) = make_longlong2(right + s0, right + s1);
+        *reinterpret_cast<longlong2*>(out + x + 2) = make_longlong2(right + s2, right + s3);
+      }
+    } else {
+      if (x <= i) out[x] = right + s0;
+      if (x + 1 <= i) out[x + 1] = right + s1;
+      if (x + 2 <= i) out[x + 2] = right + s2;
+      if (x + 3 <= i) out[x + 3] = right + s3;
+    }
+    carry += __shfl_sync(0xffffffffu, inc, 0);
   }
 }
 
 // step 3: prefix sums down each column ("sum the upper elements"): S(x,y) = sum_{i=x..y} Rsuf[i][x], and the
 // best point of every anti-diagonal x+y=c (max S, ties -> shorter span), kept only when S > 0.
-// A CTA owns 32 columns; thread (cx, ry) scans rows [ry*R, ry*R+R) of its column, a shared-memory scan over ry
-// supplies the offsets, and a second pass emits S.  key = (S << 10) | (1023 - (y-x)).
+// A CTA owns CX columns; thread (cx, ry) scans a group of at most 16 rows of its column, whose entries it keeps in
+// registers, a scan over the row groups supplies the offsets, and a second pass emits S.
+// key = (S << 10) | (1023 - (y-x)).  CX = 32 for regions of up to 512 tokens (32 row groups), 16 for longer ones (64).
 // seg_unit > 0 (segmentation per memory unit): only intervals inside one unit of seg_unit tokens on the absolute grid
 // are candidates; `origin` is the absolute position of the region's first token.
-// HOLD: a thread keeps its (at most 16) entries of the column in registers between the two passes (m <= 512).
-template <bool HOLD>
+template <int CX>
 __global__ void __launch_bounds__(1024) k_seg_colscan(DevCtx c, int layer_begin, int m, int seg_unit, int origin) {
   chain_wait();
+  constexpr int RY = 1024 / CX, K = RY / 32;
   extern __shared__ long long sm[];
-  long long* part = sm;             // [32 ry][32 cx]
-  long long* sbest = sm + 32 * 32;  // [m + 32]
+  long long* part = sm;                  // [RY][CX + 1]
+  long long* sbest = sm + RY * (CX + 1); // [m + CX]
   const int layer = layer_begin + blockIdx.y;
-  const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
-  const int x0 = blockIdx.x * 32, x = x0 + cx;
-  const int R = (m + 31) / 32;
+  const int cx = threadIdx.x % CX, ry = threadIdx.x / CX;
+  const int x0 = blockIdx.x * CX, x = x0 + cx;
+  const int R = (m + RY - 1) / RY;
   const long long* Rs = c.Rsuf + (size_t)layer * c.chunk * c.chunk;
-  for (int t = threadIdx.x; t < m + 32; t += blockDim.x) sbest[t] = 0;
   const int ylo = ry * R, yhi = min(m, ylo + R);
-  long long acc = 0;
-  long long cv[HOLD ? 16 : 1];
-  if (HOLD) {
+  long long cv[16];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int y = ylo + k;
-      cv[k] = (x < m && y >= x && y < yhi) ? Rs[(size_t)y * c.chunk + x] : 0;
-    }
-#pragma unroll
-    for (int k = 0; k < 16; ++k) acc += cv[k];
-  } else if (x < m) {
-    for (int y = max(ylo, x); y < yhi; ++y) acc += Rs[(size_t)y * c.chunk + x];
+  for (int k = 0; k < 16; ++k) {
+    const int y = ylo + k;
+    cv[k] = (x < m && y >= x && y < yhi) ? Rs[(size_t)y * c.chunk + x] : 0;
   }
-  part[ry * 32 + cx] = acc;
+  for (int t = threadIdx.x; t < m + CX; t += blockDim.x) sbest[t] = 0;
+  long long acc = 0;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) acc += cv[k];
+  part[ry * (CX + 1) + cx] = acc;
   __syncthreads();
-  if (ry == 0) {  // exclusive scan over ry for column cx
-    long long run = 0;
-    for (int r = 0; r < 32; ++r) {
-      const long long t = part[r * 32 + cx];
-      part[r * 32 + cx] = run;
-      run += t;
+  // exclusive scan over the row groups, a warp per column, K groups per lane
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (wid < CX) {
+    long long v[K], inc = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      v[k] = part[(lane * K + k) * (CX + 1) + wid];
+      inc += v[k];
+    }
+    const long long own = inc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    long long run = inc - own;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      part[(lane * K + k) * (CX + 1) + wid] = run;
+      run += v[k];
     }
   }
   __syncthreads();
   if (x < m) {
-    long long S = part[ry * 32 + cx];
+    long long S = part[ry * (CX + 1) + cx];
     // last token of the unit that holds x (region-relative)
     const int ymax = seg_unit > 0 ? ((origin + x) / seg_unit + 1) * seg_unit - origin - 1 : m;
-    if (HOLD) {
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const int y = ylo + k;
-        if (y < x || y >= yhi) continue;
-        S += cv[k];
-        if (S > 0 && y <= ymax) {
-          const long long key = (S << 10) | (long long)(1023 - (y - x));
-          atomicMax(&sbest[x + y - 2 * x0], key);
-        }
-      }
-    } else {
-      for (int y = max(ylo, x); y < yhi; ++y) {
-        S += Rs[(size_t)y * c.chunk + x];
-        if (S > 0 && y <= ymax) {
-          const long long key = (S << 10) | (long long)(1023 - (y - x));
-          atomicMax(&sbest[x + y - 2 * x0], key);
-        }
+    for (int k = 0; k < 16; ++k) {
+      const int y = ylo + k;
+      if (y < x || y >= yhi) continue;
+      S += cv[k];
+      if (S > 0 && y <= ymax) {
+        const long long key = (S << 10) | (long long)(1023 - (y - x));
+        atomicMax(&sbest[x + y - 2 * x0], key);
       }
     }
   }
   __syncthreads();
   long long* gbest = c.best + (size_t)layer * 2 * c.chunk;
-  for (int t = threadIdx.x; t < m + 32; t += blockDim.x) {
+  for (int t = threadIdx.x; t < m + CX; t += blockDim.x) {
     const long long key = sbest[t];
     const int cd = 2 * x0 + t;
     if (key > 0 && cd <= 2 * m - 2) atomicMax(&gbest[cd], key);
@@ -535,14 +594,20 @@ struct NmsArgs {
   int seg_unit;              // > 0: every unit of this many tokens (absolute grid) keeps max_spans spans of its own
 };
 
+// A cluster of CTAs may share a layer (its launch says how many): the first CTA runs the NMS and the gap fill, then the
+// spans are dealt to all of them for the representatives.  One layer alone took 40 us (regions of 512) to 73 us (1024) in a
+// single CTA, most of it 32 rounds of two barriers over 1024 threads and five dependent 64-bit shuffles each.
 __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   chain_wait();
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CL = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
   __shared__ long long skey[768];  // scratch of the query representatives: token lists and counts per span
   __shared__ int kx[kMaxTopK], ky[kMaxTopK];
   __shared__ int out_start[2 * kMaxTopK + 1], out_len[2 * kMaxTopK + 1];
   __shared__ int s_nout;
   __shared__ int s_ucnt[kMaxTopK + 2];  // segmentation per unit: spans kept in every unit the region touches
-  const int layer = a.layer_begin + blockIdx.x;
+  const int lidx = blockIdx.x / CL, layer = a.layer_begin + lidx;
   const size_t unit = unit_of(c, a.seq, layer);
   const int m = a.m;
   const int SU = a.seg_unit;
@@ -557,76 +622,82 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   // candidates, keeps it, and lets every thread strike out its own candidates that the new span suppresses (or whose
   // unit is full).  At most max_spans rounds of two barriers each instead of sorting up to 2047 keys.
   // Candidate of anti-diagonal cd: key = (S << 10) | (1023 - len) > 0; x = (cd - len) / 2, y = x + len.
-  __shared__ long long s_wkey[32];
-  __shared__ int s_wcd[32];
+  // The rounds run in the first 8 or 16 warps, four candidates per thread, with one barrier each: the warps' best are
+  // found with three warp-wide integer reductions and meet in one of two arrays that the rounds use in turn.
+  __shared__ uint4 s_wbest[2][16];
+  __shared__ int s_kept;
   const int tid = threadIdx.x, wlane = tid & 31, wid = tid >> 5;
-  long long ckey[2];
-  int cx[2], cy[2];
-  bool alive[2];
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int cd = tid + u * 1024;
-    ckey[u] = cd < ncand ? gbest[cd] : 0;
-    const int len = 1023 - (int)(ckey[u] & 1023);
-    cx[u] = (cd - len) >> 1;
-    cy[u] = cx[u] + len;
-    alive[u] = ckey[u] > 0;
-  }
-  for (int t = tid; t < kMaxTopK + 2; t += blockDim.x) s_ucnt[t] = 0;
-  int kept = 0;
-  auto better = [](long long ka, int ca, long long kb, int cb) { return ka > kb || (ka == kb && ca < cb); };
-  while (kept < cap_total) {
-    long long bk = 0;
-    int bc = 0x7fffffff;
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-      if (alive[u] && better(ckey[u], tid + u * 1024, bk, bc)) {
-        bk = ckey[u];
-        bc = tid + u * 1024;
-      }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const long long ok = shfl_xor_ll(bk, o);
-      const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
-      if (better(ok, oc, bk, bc)) {
-        bk = ok;
-        bc = oc;
-      }
-    }
-    if (wlane == 0) {
-      s_wkey[wid] = bk;
-      s_wcd[wid] = bc;
-    }
+  const int NT = ncand > 1024 ? 512 : 256;
+  if (SU > 0) {
+    for (int t = tid; t < kMaxTopK + 2; t += blockDim.x) s_ucnt[t] = 0;
     __syncthreads();
-    bk = s_wkey[wlane];  // every warp reduces the 32 partial results itself: all threads learn the winner
-    bc = s_wcd[wlane];
+  }
+  if (part == 0 && tid < NT) {
+    auto round_barrier = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(NT) : "memory"); };
+    const int nw = NT >> 5;
+    unsigned khi[4], klo[4];
+    int cx[4], cy[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const long long ok = shfl_xor_ll(bk, o);
-      const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
-      if (better(ok, oc, bk, bc)) {
-        bk = ok;
-        bc = oc;
+    for (int u = 0; u < 4; ++u) {
+      const int cd = tid + u * NT;
+      const long long key = cd < ncand ? gbest[cd] : 0;
+      const int len = 1023 - (int)(key & 1023);
+      cx[u] = (cd - len) >> 1;
+      cy[u] = cx[u] + len;
+      khi[u] = key > 0 ? (unsigned)(key >> 32) : 0u;  // (key 0: not alive)
+      klo[u] = key > 0 ? (unsigned)key : 0u;
+    }
+    // warp-wide best of (hi, lo) descending, then cd ascending
+    auto reduce = [&](unsigned& hi, unsigned& lo, int& cd) {
+      const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+      const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+      cd = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? cd : 0x7fffffff);
+      hi = mh;
+      lo = ml;
+    };
+    int kept = 0;
+    while (kept < cap_total) {
+      unsigned bh = 0, bl = 0;
+      int bc = 0x7fffffff;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (khi[u] > bh || (khi[u] == bh && klo[u] > bl)) {  // (ascending candidates: an equal one does not replace)
+          bh = khi[u];
+          bl = klo[u];
+          bc = tid + u * NT;
+        }
+      reduce(bh, bl, bc);
+      uint4* buf = s_wbest[kept & 1];
+      if (wlane == 0) buf[wid] = make_uint4(bh, bl, (unsigned)bc, 0u);
+      round_barrier();
+      const uint4 w = wlane < nw ? buf[wlane] : make_uint4(0u, 0u, 0x7fffffffu, 0u);
+      bh = w.x;
+      bl = w.y;
+      bc = (int)w.z;
+      reduce(bh, bl, bc);
+      if ((bh | bl) == 0u) break;  // nothing alive is left (the same decision in every thread)
+      const int wl = 1023 - (int)(bl & 1023);
+      const int wx = (bc - wl) >> 1, wy = wx + wl;
+      if (tid == 0) {
+        kx[kept] = wx;
+        ky[kept] = wy;
+        if (SU > 0) ++s_ucnt[unit_idx(wx)];
       }
-    }
-    if (bk <= 0) break;  // nothing alive is left (the same decision in every thread)
-    const int wl = 1023 - (int)(bk & 1023);
-    const int wx = (bc - wl) >> 1, wy = wx + wl;
-    if (tid == 0) {
-      kx[kept] = wx;
-      ky[kept] = wy;
-      if (SU > 0) ++s_ucnt[unit_idx(wx)];
-    }
-    ++kept;
-    __syncthreads();  // the unit counts are up to date; s_wkey may be overwritten
+      ++kept;
+      if (SU > 0) round_barrier();  // the unit counts are up to date
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
-      alive[u] = alive[u] && tid + u * 1024 != bc && !nms_suppressed(cx[u], cy[u], wx, wy, phi_milli) &&
-                 (SU == 0 || s_ucnt[unit_idx(cx[u])] < a.max_spans);
+      for (int u = 0; u < 4; ++u)
+        if ((khi[u] | klo[u]) != 0u &&
+            (tid + u * NT == bc || nms_suppressed(cx[u], cy[u], wx, wy, phi_milli) ||
+             (SU > 0 && s_ucnt[unit_idx(cx[u])] >= a.max_spans)))
+          khi[u] = klo[u] = 0u;
+      if (SU > 0) round_barrier();  // (everybody has read them)
+    }
+    if (tid == 0) s_kept = kept;
   }
   __syncthreads();
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
+  if (part == 0 && threadIdx.x < 32) {
+    const int lane = threadIdx.x, kept = s_kept;
     // order the kept spans by start (rank sort), then gap fill
     int rank0 = 0, rank1 = 0;
     const int x0 = lane < kept ? kx[lane] : 0x7fffffff;
@@ -643,7 +714,43 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
     if (lane < kept) ky[rank0] = y0;
     if (lane + 32 < kept) ky[rank1] = y1;
     __syncwarp();
-    if (lane == 0) {
+    if (SU == 0) {
+      // two entries per lane: the end of everything covered in front of a span (a prefix maximum: with phi > 0 kept spans
+      // may overlap) tells whether an uncovered run precedes it, the number of such runs where it goes
+      int covered = 0, no = 0;
+      for (int base = 0; base < kept; base += 32) {
+        const int q = base + lane;
+        const int sx = q < kept ? kx[q] : 0x7fffffff, sy = q < kept ? ky[q] + 1 : 0;
+        int inc = sy;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc = max(inc, t);
+        }
+        int before = __shfl_up_sync(0xffffffffu, inc, 1);
+        if (lane == 0) before = 0;
+        before = max(before, covered);
+        const unsigned gaps = __ballot_sync(0xffffffffu, q < kept && sx > before);
+        const int at = no + lane + __popc(gaps & ((2u << lane) - 1u));
+        if (q < kept) {
+          if (sx > before) {
+            out_start[at - 1] = before;
+            out_len[at - 1] = sx - before;
+          }
+          out_start[at] = sx;
+          out_len[at] = sy - sx;
+        }
+        covered = max(covered, __shfl_sync(0xffffffffu, inc, 31));
+        no += min(32, kept - base) + __popc(gaps);
+      }
+      if (lane == 0) {
+        if (covered < m) {
+          out_start[no] = covered;
+          out_len[no++] = m - covered;
+        }
+        s_nout = no;
+      }
+    } else if (lane == 0) {
       int pos = 0, no = 0;
       // an uncovered run [g0, g1) becomes a span; under segmentation per unit it is cut at the unit boundaries
       auto emit_gap = [&](int g0, int g1) {
@@ -666,6 +773,18 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
       s_nout = no;
     }
   }
+  if (CL > 1) {
+    cluster.sync();
+    if (part > 0) {
+      const int n = *cluster.map_shared_rank(&s_nout, 0);
+      if (threadIdx.x == 0) s_nout = n;
+      for (int t = threadIdx.x; t < min(n, 2 * kMaxTopK + 1); t += blockDim.x) {
+        out_start[t] = cluster.map_shared_rank(out_start, 0)[t];
+        out_len[t] = cluster.map_shared_rank(out_len, 0)[t];
+      }
+    }
+    cluster.sync();  // (the first CTA's shared memory is not read after this point)
+  }
   __syncthreads();
   const int nout = s_nout;
   const size_t ps = (unit * c.slots + a.slot) * c.Jmax;
@@ -673,11 +792,12 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
     if (threadIdx.x == 0) set_status(c, -5, nout);
     return;
   }
-  for (int t = threadIdx.x; t < nout; t += blockDim.x) {
-    c.pend_start[ps + t] = a.reg_start + out_start[t];
-    c.pend_len[ps + t] = out_len[t];
-  }
-  if (threadIdx.x == 0) {
+  if (part == 0)
+    for (int t = threadIdx.x; t < nout; t += blockDim.x) {
+      c.pend_start[ps + t] = a.reg_start + out_start[t];
+      c.pend_len[ps + t] = out_len[t];
+    }
+  if (part == 0 && threadIdx.x == 0) {
     c.pend_cnt[unit * c.slots + a.slot] = nout;
     c.Jcnt[layer] = a.q ? nout : 0;
   }
@@ -685,14 +805,15 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   // (span, KV head) sums their query rows with all loads of the head group in flight at once.
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   const long long* votes = c.votes + unit * c.Tpad;
-  const __nv_bfloat16* q = a.q + (size_t)blockIdx.x * a.n * c.Hq * kD;
+  const __nv_bfloat16* q = a.q + (size_t)lidx * a.n * c.Hq * kD;
   int* rep_tok = reinterpret_cast<int*>(skey);          // [Jmax][kMaxReps]
   int* rep_cnt = rep_tok + (2 * kMaxTopK + 1) * kMaxReps;
   __syncthreads();
   // representative count of every span: static, or from the area ratio of Sec. 3.3.2 on the raw region map.  The
   // row-suffix table holds sums of (Mq - theta), so a raw sum over w entries is the table value + theta * w.
   int* nrep_of = rep_cnt + (2 * kMaxTopK + 1);
-  for (int j = warp; j < nout; j += nwarps) {
+  // (the spans part, part + CL, ... are this CTA's)
+  for (int j = part + CL * warp; j < nout; j += CL * nwarps) {
     int cnt = min(c.reps, out_len[j]);
     if (c.rep_mode == 1) {
       const long long* Rs = c.Rsuf + (size_t)layer * c.chunk * c.chunk;
@@ -729,7 +850,7 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   }
   __syncthreads();
   if (!a.q) return;
-  for (int j = warp; j < nout; j += nwarps) {
+  for (int j = part + CL * warp; j < nout; j += CL * nwarps) {
     int toks[kMaxReps];
     const int nrep = select_reps(votes, a.reg_start + out_start[j], out_len[j], nrep_of[j], toks);
     if (lane == 0) {
@@ -743,8 +864,9 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   // ascending order
   const int hw = lane >> 4, hl = lane & 15;
   const int rh = ret_head_of(c, layer);
-  for (int task = 2 * warp + hw; task < nout * c.Hkv; task += 2 * nwarps) {
-    const int j = task / c.Hkv, g = task % c.Hkv;
+  const int nmine = nout > part ? (nout - part + CL - 1) / CL : 0;
+  for (int task = 2 * warp + hw; task < nmine * c.Hkv; task += 2 * nwarps) {
+    const int j = part + CL * (task / c.Hkv), g = task % c.Hkv;
     const int nrep = rep_cnt[j];
     const __nv_bfloat16* qg = q + (size_t)g * c.G * kD + hl * 8;
     // a layer with a retrieval head (Sec. 3.5) has one representative per span, that head's: the other heads add zero
@@ -802,6 +924,9 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   }
 }
 
+constexpr int kSegWideLayers = 7;    // clusters of 16 that run at once
+constexpr int kSegShareLayers = 16;  // up to here four CTAs share a layer's representatives
+
 cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start,
                              int slot, int theta_mode, float theta, long long theta_q_abs, int max_spans, int n,
                              int t0, const __nv_bfloat16* q, cudaStream_t s, bool tables, int seg_unit) {
@@ -810,23 +935,39 @@ cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_
     long long rank = (long long)floor((double)theta * (double)(N - 1));
     if (rank < 0) rank = 0;
     if (rank > N - 1) rank = N - 1;
-    const int hsmem = (kThetaThreads / 32) * kThetaBins * (int)sizeof(unsigned);
-    launch_chained(k_theta_select, dim3(layer_count * kThetaCluster), dim3(kThetaThreads), hsmem, s, c, layer_begin, m,
-                   rank, tables ? 1 : 0);
+    // Few layers: 16 CTAs of 1024 threads share one, which gives every pair of rows a warp of its own (a cluster of 16
+    // needs a GPC to itself, so seven run at once).  More: 8 CTAs of 512 threads.
+    if (layer_count <= kSegWideLayers) {
+      const int hsmem = 32 * kThetaBins * (int)sizeof(unsigned);
+      auto fn = m <= 512 ? k_theta_select<17> : k_theta_select<33>;
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, hsmem);
+      cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      launch_chained_cluster(fn, dim3(layer_count * 16), dim3(1024), 16, hsmem, s, c, layer_begin, m, rank, tables ? 1 : 0);
+    } else {
+      const int hsmem = (kThetaThreads / 32) * kThetaBins * (int)sizeof(unsigned);
+      launch_chained_cluster(k_theta_select<0>, dim3(layer_count * 8), dim3(kThetaThreads), 8, hsmem, s, c, layer_begin, m,
+                             rank, tables ? 1 : 0);
+    }
   } else {
     launch_chained(k_theta_set, dim3(layer_count), dim3(1), 0, s, c, layer_begin, theta_q_abs,
                    (long long)nearbyint((double)theta * (double)kQScale), tables ? 1 : 0);
   }
-  launch_chained(k_seg_rowscan, dim3((m + 7) / 8, layer_count), dim3(256), 0, s, c, layer_begin, m);
-  const size_t smem = (size_t)(32 * 32 + m + 32) * sizeof(long long);
-  if (m <= 512)
-    launch_chained(k_seg_colscan<true>, dim3((m + 31) / 32, layer_count), dim3(1024), smem, s, c, layer_begin, m, seg_unit,
-                   reg_start);
+  const dim3 rows((m + 7) / 8, layer_count);
+  if (m <= 256)
+    launch_chained(k_seg_rowscan<2>, rows, dim3(256), 0, s, c, layer_begin, m);
+  else if (m <= 512)
+    launch_chained(k_seg_rowscan<4>, rows, dim3(256), 0, s, c, layer_begin, m);
   else
-    launch_chained(k_seg_colscan<false>, dim3((m + 31) / 32, layer_count), dim3(1024), smem, s, c, layer_begin, m,
-                   seg_unit, reg_start);
+    launch_chained(k_seg_rowscan<8>, rows, dim3(256), 0, s, c, layer_begin, m);
+  if (m <= 512)
+    launch_chained(k_seg_colscan<32>, dim3((m + 31) / 32, layer_count), dim3(1024),
+                   (size_t)(32 * 33 + m + 32) * sizeof(long long), s, c, layer_begin, m, seg_unit, reg_start);
+  else
+    launch_chained(k_seg_colscan<16>, dim3((m + 15) / 16, layer_count), dim3(1024),
+                   (size_t)(64 * 17 + m + 16) * sizeof(long long), s, c, layer_begin, m, seg_unit, reg_start);
   NmsArgs a{seq, layer_begin, m, reg_start, slot, max_spans, n, t0, q, tables ? 1 : 0, seg_unit};
-  launch_chained(k_seg_nms, dim3(layer_count), dim3(1024), 0, s, c, a);
+  const int cl = q && layer_count <= kSegShareLayers ? 4 : 1;
+  launch_chained_cluster(k_seg_nms, dim3(layer_count * cl), dim3(1024), cl, 0, s, c, a);
   return cudaGetLastError();
 }
 

@@ -850,6 +850,9 @@ int ltri_host_outputs_ready(ltri_ctx* ctx, void* cuda_stream) {
 // holds no shared memory for tiles and leaves more CTAs per SM to hide the latency, stream it faster (33K spans, 32
 // units: 92 against 103 us a step).
 constexpr int kStepSpans = 2560;
+// The same holds for the tokens a CTA attends over, of which it keeps one 16-token tile per warp on the way (12.7K tokens
+// per unit, 64 units: 124 us a step against 130 us as clusters of four).
+constexpr int kStepTokens = 1536;
 static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, long long ub) {
   const DevCtx& d = ctx->d;
   int e_max = 0;
@@ -858,10 +861,13 @@ static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, 
     e_max = std::max(e_max, b.loc_begin[i]);
     known = std::max(known, (long long)d.Ls + b.pos[i] + 1 - b.loc_begin[i]);
   }
+  // tokens a unit attends over: known ones, and about top_k (with the persistent set twice that) units or mean spans
+  const long long item = d.unit > 0 ? d.unit : ub > 0 ? (e_max + ub - 1) / ub * 2 : 0;
+  const long long tokens = known + std::min<long long>(e_max, (long long)d.topk * item * (d.persist ? 2 : 1));
   for (int i = 4; i >= 1; --i) {
     const int cl = 1 << i;
     if (ctx->step_cluster > 0 ? cl != ctx->step_cluster : known / cl < 64 && cl > 2) continue;
-    if (ctx->step_cluster == 0 && d.unit == 0 && ub > (long long)kStepSpans * cl) continue;
+    if (ctx->step_cluster == 0 && ((d.unit == 0 && ub > (long long)kStepSpans * cl) || tokens > kStepTokens * cl)) continue;
     if ((long long)units * cl <= ctx->step_cap[i] && dec_step_fits(d, (int)ub, e_max, cl)) return cl;
   }
   return 0;
