@@ -173,7 +173,7 @@ cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_
 cudaError_t launch_score_prefill(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s);
 // tensor-core version of launch_score_prefill (split-bf16 representatives)
 cudaError_t launch_score_prefill_mma(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s);
-cudaError_t launch_topk_prefill(const DevCtx& c, const PrefillArgs& a, cudaStream_t s);
+cudaError_t launch_topk_prefill(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s);
 // host-memory pager: pulls of the missing units + gather of the selected units' rows (after launch_topk_prefill)
 cudaError_t launch_pull_pack(const DevCtx& c, const PrefillArgs& a, cudaStream_t s);
 cudaError_t launch_score_decode(const DevCtx& c, const DecBatch& b, int layer_begin, int layer_count, int n_seqs_total,

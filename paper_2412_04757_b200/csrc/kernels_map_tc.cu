@@ -51,7 +51,7 @@ constexpr int kMapKT = 4;
 
 template <int G>
 __global__ void __launch_bounds__(kMapThreads, 1)
-    k_map_tc(DevCtx c, PrefillArgs a, int n_local_groups, int n_local_tiles, int n_cur_tiles,
+    k_map_tc(DevCtx c, PrefillArgs a, int n_local_groups, int n_local_tiles, int n_cur_tiles, int group_tiles, int splits,
              const __grid_constant__ MapMaps maps) {
   extern __shared__ unsigned char smem_raw[];
   // KFULL[4] | QFULL[2] QEMPTY[2] | SFULL[4] SEMPTY[4]
@@ -69,16 +69,21 @@ __global__ void __launch_bounds__(kMapThreads, 1)
     rh = c.ret_head[layer];
     if (rh >= 0 && g != rh / G) return;
   }
-  const bool is_cur = (int)blockIdx.x >= n_local_groups;
-  const int tile0 = (is_cur ? (int)blockIdx.x - n_local_groups : (int)blockIdx.x) * kMapKT;
-  const int ntile = min(kMapKT, (is_cur ? n_cur_tiles : n_local_tiles) - tile0);
+  const int group = (int)blockIdx.x / splits, split = (int)blockIdx.x % splits;
+  const bool is_cur = group >= n_local_groups;
+  const int tile0 = (is_cur ? group - n_local_groups : group) * group_tiles;
   // first key (absolute) of key tile kt, the end of the range, and the first query block that sees the tile
   const int kbase = is_cur ? a.t0 : a.loc_begin;
   const int key_end = is_cur ? a.t0 + a.n : a.t0;
   auto key0_of = [&](int kt) { return kbase + (tile0 + kt) * 128; };
   auto blk0_of = [&](int kt) { return is_cur ? ((tile0 + kt) * 128) / TPB : 0; };
-  const int nblocks = (a.n + TPB - 1) / TPB;
-  const int bmin = blk0_of(0);
+  // the query blocks [bmin, nblocks) of this split, and the key tiles of the group that any of them sees
+  const int all_blocks = (a.n + TPB - 1) / TPB, bfirst = blk0_of(0);
+  const int per_split = (all_blocks - bfirst + splits - 1) / splits;
+  const int bmin = bfirst + split * per_split, nblocks = min(all_blocks, bmin + per_split);
+  if (bmin >= nblocks) return;
+  int ntile = min(group_tiles, (is_cur ? n_cur_tiles : n_local_tiles) - tile0);
+  while (ntile > 1 && blk0_of(ntile - 1) >= nblocks) --ntile;
 
   const uint32_t sbase = (smem_addr(smem_raw) + 1023u) & ~1023u;
   const uint32_t sK = sbase;                      // kMapKT x 32 KB: [tile][half d][128 keys][64]
@@ -374,11 +379,33 @@ static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const 
   // kernel)
   const int nloc = (a.loc_begin >= c.Ls) ? (a.t0 - a.loc_begin + 127) / 128 : 0;
   const int ncur = (a.n + 127) / 128;
-  const int gloc = (nloc + kMapKT - 1) / kMapKT, gcur = (ncur + kMapKT - 1) / kMapKT;
+  // Key tiles per CTA and splits of the query blocks.  With enough CTAs for several waves: four tiles, no split (the
+  // queries are re-read least).  Otherwise the pair that finishes first by a small model, in units of one product of a key
+  // tile with a query block (about 1.2K cycles; a CTA starts and ends in about six of them).  One layer, 36 tiles, 8 KV
+  // heads: 72 CTAs of four tiles took 57 us, 144 CTAs of two take 35.  The map and the votes are integer sums, so the
+  // results do not depend on the choice.
+  const int nblk = (a.n + 128 / G - 1) / (128 / G);
+  int kt = kMapKT, qs = 1;
+  const int heads = c.Hkv * a.layer_count;
+  auto ctas_of = [&](int k, int q) { return ((nloc + k - 1) / k + (ncur + k - 1) / k) * q * heads; };
+  if (ctas_of(kMapKT, 1) <= 3 * 148) {
+    long long best = -1;
+    for (int k = kMapKT; k >= 1; --k)
+      for (int q = 1; q <= 8 && q <= nblk; q *= 2) {
+        const long long waves = (ctas_of(k, q) + 147) / 148;
+        const long long cost = waves * (6 + k * ((nblk + q - 1) / q));
+        if (best < 0 || cost < best) {
+          best = cost;
+          kt = k;
+          qs = q;
+        }
+      }
+  }
+  const int gloc = (nloc + kt - 1) / kt, gcur = (ncur + kt - 1) / kt;
   const int smem = kMapKT * 32768 + 65536 + 3 * 4096 + 1024;  // key tiles, two query stages, the offset tiles
   cudaFuncSetAttribute(k_map_tc<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  return launch_chained(k_map_tc<G>, dim3(gloc + gcur, c.Hkv, a.layer_count), dim3(kMapThreads), smem, s, c, a, gloc, nloc,
-                        ncur, maps);
+  return launch_chained(k_map_tc<G>, dim3((gloc + gcur) * qs, c.Hkv, a.layer_count), dim3(kMapThreads), smem, s, c, a, gloc,
+                        nloc, ncur, kt, qs, maps);
 }
 
 cudaError_t launch_map_pass_tc(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, cudaStream_t s) {

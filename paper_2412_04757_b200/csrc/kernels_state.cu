@@ -143,20 +143,24 @@ cudaError_t launch_append_decode(const DevCtx& c, const DecBatch& b, int layer_b
 
 // ------------------------------------------------------------------------------------------
 // a1: regions that left the window: every span gets its index vector, the bf16 sum of the keys of
-// its most voted token(s), and is appended to the span table.  One CTA per layer, one warp per span (32 warps).
-__global__ void __launch_bounds__(1024) k_evict_index(DevCtx c, EvictArgs a) {
+// its most voted token(s), and is appended to the span table.  Eight CTAs of eight warps (a cluster, so that the span
+// count is moved on only when all have read it) share a layer, one warp per span, four key rows in flight per warp.
+// Bound: latency (votes -> token -> key rows); with one CTA of 32 warps per layer, two or three rounds of it: 12 us for
+// one region of 512 tokens, 18 us of 1024.
+constexpr int kEvictCluster = 8;
+__global__ void __cluster_dims__(kEvictCluster, 1, 1) __launch_bounds__(256) k_evict_index(DevCtx c, EvictArgs a) {
   chain_wait();
   if (a.release) chain_release();
-  const int layer = a.layer_begin + blockIdx.x;
+  const int layer = a.layer_begin + blockIdx.x / kEvictCluster, part = blockIdx.x % kEvictCluster;
   const size_t unit = unit_of(c, a.seq, layer);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = (blockDim.x >> 5) * kEvictCluster;
   const int base = c.n_spans[unit];
   const long long* votes = c.votes + unit * c.Tpad;
   int off = 0;
   for (int si = 0; si < a.nslots; ++si) {
     const size_t ps = (unit * c.slots + a.slot[si]) * c.Jmax;
     const int cnt = c.pend_cnt[unit * c.slots + a.slot[si]];
-    for (int i = warp; i < cnt; i += nwarps) {
+    for (int i = part + kEvictCluster * warp; i < cnt; i += nwarps) {
       const int start = c.pend_start[ps + i], len = c.pend_len[ps + i];
       const int dst = base + off + i;
       if (dst >= c.cap) {
@@ -169,36 +173,48 @@ __global__ void __launch_bounds__(1024) k_evict_index(DevCtx c, EvictArgs a) {
       }
       int toks[kMaxReps];
       const int nrep = select_reps(votes, start, len, c.rep_mode == 1 ? c.pend_nrep[ps + i] : c.reps, toks);
-      for (int g = 0; g < c.Hkv; ++g) {
-        const __nv_bfloat16* kslab = c.Kc + ((unit * c.Hkv + g) * c.SR) * kD;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int g0 = 0; g0 < c.Hkv; g0 += 4) {
+        float acc[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u][0] = acc[u][1] = acc[u][2] = acc[u][3] = 0.f;
         for (int r = 0; r < nrep; ++r) {
-          const uint2 raw =
-              *reinterpret_cast<const uint2*>(kslab + (size_t)slab_row(c, toks[r], a.shift) * kD + lane * 4);
-          const __nv_bfloat162 p0 = *reinterpret_cast<const __nv_bfloat162*>(&raw.x);
-          const __nv_bfloat162 p1 = *reinterpret_cast<const __nv_bfloat162*>(&raw.y);
-          acc[0] += __bfloat162float(p0.x);
-          acc[1] += __bfloat162float(p0.y);
-          acc[2] += __bfloat162float(p1.x);
-          acc[3] += __bfloat162float(p1.y);
+          const size_t row = (size_t)slab_row(c, toks[r], a.shift) * kD + lane * 4;
+          uint2 raw[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            raw[u] = g0 + u < c.Hkv
+                         ? *reinterpret_cast<const uint2*>(c.Kc + ((unit * c.Hkv + g0 + u) * c.SR) * kD + row)
+                         : make_uint2(0u, 0u);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const __nv_bfloat162 p0 = *reinterpret_cast<const __nv_bfloat162*>(&raw[u].x);
+            const __nv_bfloat162 p1 = *reinterpret_cast<const __nv_bfloat162*>(&raw[u].y);
+            acc[u][0] += __bfloat162float(p0.x);
+            acc[u][1] += __bfloat162float(p0.y);
+            acc[u][2] += __bfloat162float(p1.x);
+            acc[u][3] += __bfloat162float(p1.y);
+          }
         }
-        __nv_bfloat162 o0 = __floats2bfloat162_rn(acc[0], acc[1]);
-        __nv_bfloat162 o1 = __floats2bfloat162_rn(acc[2], acc[3]);
-        uint2 w;
-        w.x = *reinterpret_cast<uint32_t*>(&o0);
-        w.y = *reinterpret_cast<uint32_t*>(&o1);
-        *reinterpret_cast<uint2*>(c.KR + ((unit * c.Hkv + g) * c.cap + dst) * kD + lane * 4) = w;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (g0 + u >= c.Hkv) continue;
+          __nv_bfloat162 o0 = __floats2bfloat162_rn(acc[u][0], acc[u][1]);
+          __nv_bfloat162 o1 = __floats2bfloat162_rn(acc[u][2], acc[u][3]);
+          uint2 w;
+          w.x = *reinterpret_cast<uint32_t*>(&o0);
+          w.y = *reinterpret_cast<uint32_t*>(&o1);
+          *reinterpret_cast<uint2*>(c.KR + ((unit * c.Hkv + g0 + u) * c.cap + dst) * kD + lane * 4) = w;
+        }
       }
     }
     off += cnt;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) c.n_spans[unit] = min(base + off, c.cap);
+  cooperative_groups::this_cluster().sync();
+  if (part == 0 && threadIdx.x == 0) c.n_spans[unit] = min(base + off, c.cap);
 }
 
 cudaError_t launch_evict_index(const DevCtx& c, const EvictArgs& a, int layer_count, cudaStream_t s) {
-  // a warp per span: one round for a region of up to 32 spans
-  return launch_chained(k_evict_index, dim3(layer_count), dim3(1024), 0, s, c, a);
+  return launch_chained(k_evict_index, dim3(layer_count * kEvictCluster), dim3(256), 0, s, c, a);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -580,10 +596,11 @@ __global__ void __launch_bounds__(1024) k_seg_colscan(DevCtx c, int layer_begin,
 // two spans that share `inter` tokens have IoU = inter^2 / (L1^2 + L2^2 - inter^2).  Integer arithmetic; phi = 0
 // means any overlap suppresses.
 __device__ __forceinline__ bool nms_suppressed(int x, int y, int kx, int ky, int phi_milli) {
-  const long long inter = (long long)min(y, ky) - max(x, kx) + 1;
-  if (inter <= 0) return false;
-  const long long l1 = y - x + 1, l2 = ky - kx + 1, i2 = inter * inter;
-  return i2 * 1000 > (long long)phi_milli * (l1 * l1 + l2 * l2 - i2);
+  const int inter = min(y, ky) - max(x, kx) + 1;
+  if (inter <= 0 || phi_milli == 0) return inter > 0;
+  // lengths of at most 1024: every product fits 32 bits (in 64 bits the test was most of a round's instructions)
+  const unsigned l1 = y - x + 1, l2 = ky - kx + 1, i2 = (unsigned)inter * (unsigned)inter;
+  return i2 * 1000u > (unsigned)phi_milli * (l1 * l1 + l2 * l2 - i2);
 }
 
 struct NmsArgs {
@@ -1114,7 +1131,7 @@ constexpr int kTopkSelRegs = 24;  // scores of up to 12K spans (512 threads) are
 
 template <bool DECODE>
 __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin, DecBatch b, int layer_count,
-                                              int evicted_end, int mode) {
+                                              int evicted_end, int mode, int parts, int stage) {
   chain_wait();
   __shared__ unsigned hist[256];
   __shared__ unsigned s_prefix, s_need;
@@ -1127,7 +1144,8 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
   __shared__ int s_sst[2 * kMaxTopK], s_sln[2 * kMaxTopK];  // extents of the selected spans
   __shared__ int s_all[2 * kMaxTopK], s_nall;            // decode: this step's selection united with the persistent one
   __shared__ int s_ko[kMaxRanges];  // pager, decode: first K row of every range, counted from the start of the K slabs
-  const int g = blockIdx.x;
+  // `parts` CTAs make the same selection for a (layer, KV head) and share the rows to be packed; the first one stores it
+  const int g = blockIdx.x / parts, my_part = blockIdx.x % parts;
   int layer, sq, pos = 0, loc_begin = 0;
   if (DECODE) {
     const int bi = blockIdx.y / layer_count;
@@ -1180,7 +1198,20 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
       __syncthreads();
     }
   }
-  auto KEY = [&](int i) -> unsigned { return U > 0 ? ukey[i] : order_key(sc[i]); };
+  // more spans than the threads can hold in registers: the order keys are staged in shared memory (room for `stage`)
+  const bool staged = U == 0 && N > kTopkSelRegs * nt && N <= stage;
+  if (staged) {
+    for (int base = tid; base < N; base += 16 * nt) {
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = base + u * nt < N ? sc[base + u * nt] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if (base + u * nt < N) ukey[base + u * nt] = order_key(v[u]);
+    }
+    __syncthreads();
+  }
+  auto KEY = [&](int i) -> unsigned { return U > 0 || staged ? ukey[i] : order_key(sc[i]); };
   auto KEY64 = [&](int i) -> unsigned long long {
     return ((unsigned long long)order_key(utally[i]) << 32) | ukey[i];
   };
@@ -1213,7 +1244,8 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
     return;
   }
   int* sel = c.sel + (unit * c.Hkv + g) * (size_t)c.topk;
-  for (int t = tid; t < c.topk; t += nt) sel[t] = t < cnt ? s_ids[t] : -1;
+  if (my_part == 0)
+    for (int t = tid; t < c.topk; t += nt) sel[t] = t < cnt ? s_ids[t] : -1;
   // token ranges of the attention kernels: the spans' extents are fetched in parallel, merged (adjacent spans become
   // one range) by one thread in shared memory and written out in parallel
   const int* ids_all = s_ids;
@@ -1304,9 +1336,11 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
       if (tid == 0) {
         s_pre[nr] = run;
         s_nr = nr;
-        c.rng_cnt[unit * c.Hkv + g] = nr;
-        c.sel_tokens[unit * c.Hkv + g] = tokens;  // (summed over the KV heads by ltri_get_stats)
-        if (!DECODE) c.gcnt[(size_t)layer * c.Hkv + g] = run;
+        if (my_part == 0) {
+          c.rng_cnt[unit * c.Hkv + g] = nr;
+          c.sel_tokens[unit * c.Hkv + g] = tokens;  // (summed over the KV heads by ltri_get_stats)
+          if (!DECODE) c.gcnt[(size_t)layer * c.Hkv + g] = run;
+        }
       }
     }
   } else
@@ -1354,7 +1388,7 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
     if (!DECODE) c.gcnt[(size_t)layer * c.Hkv + g] = run;
   }
   __syncthreads();
-  {
+  if (my_part == 0) {
     const size_t rb = (unit * c.Hkv + g) * (size_t)c.rcap;
     for (int t = tid; t < s_nr; t += nt) {
       c.rng_start[rb + t] = s_rs[t];
@@ -1376,7 +1410,7 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
     uint4* Kdst = reinterpret_cast<uint4*>(c.Kg + gslab * kD);
     uint4* Vdst = reinterpret_cast<uint4*>(c.Vg + gslab * kD);
     const int ch = tid & 15, rpp = nt >> 4;  // 16-byte chunk of the row, rows per pass
-    for (int r0 = tid >> 4; r0 < Rz; r0 += 4 * rpp) {
+    for (int r0 = my_part * 4 * rpp + (tid >> 4); r0 < Rz; r0 += parts * 4 * rpp) {
       uint4 kv[4], vv[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -1910,28 +1944,40 @@ static int topk_unit_smem(const DevCtx& c) {
 // chunk or step).
 template <bool DECODE>
 static cudaError_t launch_topk(const DevCtx& c, int seq, int layer_begin, const DecBatch& b, int layer_count, int gy,
-                               int evicted_end, cudaStream_t s) {
-  const int smem = topk_unit_smem(c);
+                               int evicted_end, int span_bound, cudaStream_t s) {
+  int smem = topk_unit_smem(c), stage = 0, parts = 1;
+  if (!DECODE && !c.host_kv && !c.vote) {
+    // Few (layer, KV head) pairs: several CTAs repeat the selection (it costs them nothing: the GPU is idle) and share the
+    // packing, which one CTA of 512 threads alone does at some 60 GB/s (one layer, 512 tokens a KV head: 33 us).
+    parts = max(1, min(16, 148 / (c.Hkv * gy)));
+    // more spans than 512 threads hold in registers: read once into shared memory, if they fit, instead of once per pass
+    // (only with a CTA per SM to spare: the keys take an SM's shared memory)
+    if (c.unit == 0 && span_bound > kTopkSelRegs * 512 && span_bound <= 48 * 1024 && c.Hkv * gy <= 148) {
+      stage = span_bound;
+      smem = stage * (int)sizeof(unsigned);
+    }
+  }
   if (smem > 32 * 1024) {  // (static shared memory comes on top: ask for the larger limit in good time)
     cudaError_t e = cudaFuncSetAttribute(k_topk<DECODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
   if (c.vote)
     launch_chained(k_topk<DECODE>, dim3(c.Hkv, gy), dim3(512), smem, s, c, seq, layer_begin, b, layer_count, evicted_end,
-                   (int)kTopkBallot);
-  launch_chained(k_topk<DECODE>, dim3(c.Hkv, gy), dim3(512), smem, s, c, seq, layer_begin, b, layer_count, evicted_end,
-                 (int)(c.vote ? kTopkVote : kTopkSelect));
+                   (int)kTopkBallot, 1, 0);
+  launch_chained(k_topk<DECODE>, dim3(c.Hkv * parts, gy), dim3(512), smem, s, c, seq, layer_begin, b, layer_count,
+                 evicted_end, (int)(c.vote ? kTopkVote : kTopkSelect), parts, stage);
   return cudaGetLastError();
 }
 
-cudaError_t launch_topk_prefill(const DevCtx& c, const PrefillArgs& a, cudaStream_t s) {
+cudaError_t launch_topk_prefill(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s) {
   DecBatch dummy;
   dummy.n = 0;
-  return launch_topk<false>(c, a.seq, a.layer_begin, dummy, a.layer_count, a.layer_count, a.loc_begin, s);
+  return launch_topk<false>(c, a.seq, a.layer_begin, dummy, a.layer_count, a.layer_count, a.loc_begin,
+                            span_bound, s);
 }
 
 cudaError_t launch_topk_decode(const DevCtx& c, const DecBatch& b, int layer_begin, int layer_count, cudaStream_t s) {
-  return launch_topk<true>(c, 0, layer_begin, b, layer_count, b.n * layer_count, 0, s);
+  return launch_topk<true>(c, 0, layer_begin, b, layer_count, b.n * layer_count, 0, 0, s);
 }
 
 }  // namespace ltri

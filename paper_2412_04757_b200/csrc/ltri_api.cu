@@ -741,7 +741,7 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
         LTRI_CUDA(ctx, launch_score_prefill_mma(d, ag, (int)ub, st));
       else
         LTRI_CUDA(ctx, launch_score_prefill(d, ag, (int)ub, st));
-      LTRI_CUDA(ctx, launch_topk_prefill(d, ag, st));
+      LTRI_CUDA(ctx, launch_topk_prefill(d, ag, (int)ub, st));
     }
     if (d.host_kv) {
       // the group's selection is known: its units travel on the pager's stream (behind this call's spill copies, whose
