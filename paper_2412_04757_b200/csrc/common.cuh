@@ -152,6 +152,8 @@ struct PrefillArgs {
   int sink_end, loc_begin;  // sink = [0,sink_end), local = [loc_begin,t0)
   int reg_start, m;         // region [reg_start, t0+n), m tokens
   int slot;                 // pending slot of this region (-1 if the region is empty)
+  int call_layers;          // layers of the whole call (layer_count: of the group of them that a launch covers)
+  int ret_tiles;            // 128-row tiles of retrieved tokens to expect per KV head
   long long shift;          // sliding slabs: token - shift = row of the window tokens (0 in a resident context)
   const __nv_bfloat16* q;   // [layer_count][n][Hq][128]
   const __nv_bfloat16* k;

@@ -13,6 +13,7 @@
 // the other tile's softmax runs.  The running max is updated lazily (only when it grows by more than 2^8), in which
 // case the softmax thread rescales its O row in TMEM; the in-order tensor pipe guarantees the row is quiescent then.
 // Every wait is bounded; on expiry the CTA sets LTRI_ETIMEOUT in the status word, drains and frees its TMEM.
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include <cstdlib>
@@ -146,7 +147,9 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
 
 // MERGE: the launch may be asked for phase 2 (kept out of the instantiation that runs phases 0 and 1, whose inner
 // loop is sensitive to every register).
-template <int G, bool EXCH, bool MERGE>
+// SPLIT: the CTAs of a cluster share one work item, each walks every SP-th tile of its keys; the partial softmaxes are
+// merged through distributed shared memory before the epilogue (for launches with fewer items than SMs).
+template <int G, bool EXCH, bool MERGE, bool SPLIT>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_attn_tc(DevCtx c, PrefillArgs a, int phase, int final_out, int* __restrict__ redo,
               const __grid_constant__ TcMaps maps, long long v_row_offset) {
@@ -179,6 +182,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   // persistent CTA: work items (token block, KV head, layer) are dealt round-robin
   const int MB = (a.n + TOKB - 1) / TOKB;
   const int nitems = MB * c.Hkv * a.layer_count;
+  namespace cg = cooperative_groups;
+  const int SP = SPLIT ? (int)cg::this_cluster().num_blocks() : 1;
+  const int rank = SPLIT ? (int)cg::this_cluster().block_rank() : 0;
+  const int item0 = SPLIT ? (int)blockIdx.x / SP : (int)blockIdx.x;
+  const int istep = SPLIT ? nitems : (int)gridDim.x;  // (a cluster has one item)
+  __shared__ float2 s_ml[SPLIT ? 256 : 1];     // this CTA's reference maximum and row sum of every row
+  __shared__ float2 s_tot[SPLIT ? 256 : 1];    // those of the cluster
   const uint32_t sbase = (smem_addr(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = sbase;                 // 64 KB: [half d][256 rows][64]
   const uint32_t sKV = sbase + 65536;        // 2 stages x (K 32 KB | V 32 KB), each [half d][128 slots][64]
@@ -254,7 +264,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // (K low half, K high half, V low half, V high half) so that many small pieces do not serialise on one thread.
     int jt = 0, ok = 1;
     if (lane == 0) prefetch_tmap(&maps.q);
-    for (int item = blockIdx.x, wi = 0; ok && item < nitems; item += gridDim.x, ++wi) {
+    for (int item = item0, wi = 0; ok && item < nitems; item += istep, ++wi) {
       const Item w = decode(item);
       if (lane == 0) {
         // the Q buffer is free once every QK^T product of the previous item has completed
@@ -276,7 +286,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         // publish the item's tile count with a monotonic counter: a softmax thread may look for item wi only after
         // the Q tile of item wi+1 has arrived, so a parity barrier could not tell the two apart
-        s_item_tiles[wi % 3] = count_tiles(&rg, causal_ri);
+        const int all_tiles = count_tiles(&rg, causal_ri);
+        s_item_tiles[wi % 3] = SPLIT ? (all_tiles - rank + SP - 1) / SP : all_tiles;
         __threadfence_block();
         *reinterpret_cast<volatile int*>(&s_items_ready) = wi + 1;
         if (ok) {
@@ -292,7 +303,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       it.rg = &rg;
       it.causal_ri = causal_ri;
       int pslot[16], ptok[16], pbox[16];
+      int walked = 0;  // SPLIT: tiles of the item walked so far, by whichever CTA of the cluster
       while (true) {
+        if (SPLIT) {
+          const int skip = (rank + SP - walked % SP) % SP;
+          bool more = true;
+          for (int i = 0; more && i < skip; ++i, ++walked) more = it.next();
+          if (!more) break;
+          ++walked;
+        }
         int np = 0;
         // (pieces are addressed by slab row: in a sliding slab the ranges behind the sink sit at token - shift)
         if (!it.next<true>([&](int slot, int tok, int bi) {
@@ -393,7 +412,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       // own "accumulator complete" barrier for the same reason.
       bool pre = false;
       int T_pre = 0;
-      for (int item = blockIdx.x, wi = 0; ok && item < nitems; item += gridDim.x, ++wi) {
+      for (int item = item0, wi = 0; ok && item < nitems; item += istep, ++wi) {
         int T = T_pre;
         if (!pre) {
           ok = mbar_wait(bar(B_QFULL), wi & 1, abortp, c.wait_limit);
@@ -414,7 +433,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           mma_commit(bar(B_QFREE));
         }
         pre = false;
-        const bool has_next = item + (int)gridDim.x < nitems;
+        const bool has_next = item + istep < nitems;
         for (int j = 0; ok && j < T; ++j, ++jt) {
           const int st = jt & 1, nst = st ^ 1;
           const bool acc = (j > 0) || (phase == 1);
@@ -490,7 +509,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const float c2 = c.scale * kLog2eT;
     int jt = 0;
     bool ok = true;
-    for (int item = blockIdx.x, wi = 0; item < nitems; item += gridDim.x, ++wi) {
+    for (int item = item0, wi = 0; item < nitems; item += istep, ++wi) {
       const Item w = decode(item);
       const int tk = w.tok0 + rr / G;              // call-relative token
       const int h = w.g * G + rr % G;
@@ -690,6 +709,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       if (!ok) s_quit[q] = 1;
       asm volatile("bar.sync %0, 256;" ::"r"(1 + q) : "memory");  // also: s_sum is reused by the next item
       if (s_quit[q]) break;  // collective decision: all 256 threads of the tile leave after the same item
+      if (SPLIT) {  // merged with the other CTAs' parts below
+        if (half == 0) s_ml[rr] = make_float2(m_used, lsum);
+        break;
+      }
       fence_after_sync();
       if (phase == 0 && row_ok && half == 0) {
         c.rowstat[((size_t)layer * c.chunk + tk) * c.Hq + h] = make_float2(m_used, lsum);
@@ -780,13 +803,119 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
     }
   }
+  int redo_any = 0;
+  if (SPLIT) {
+    // ---------------------------------------------------------------- merge of the cluster's parts
+    // Every CTA scales its O rows to the cluster's reference maximum and pushes them to the CTA that owns the row (256 / SP
+    // rows each; the K/V ring, no longer in use, holds the SP parts as [part][4-column group][row][4]), which adds them up
+    // in rank order and runs the epilogue.  All threads of the cluster take part in the barriers, also after an expired
+    // wait.
+    cg::cluster_group cluster = cg::this_cluster();
+    __syncwarp();
+    fence_before_sync();
+    cluster.sync();  // all products of all CTAs have completed, the (m, l) of all rows are there
+    fence_after_sync();
+    const int rows = 256 / SP;
+    float* parts = reinterpret_cast<float*>(smem_raw + (sKV - smem_addr(smem_raw)));
+    const Item w = decode(item0);
+    const bool any_tile = s_item_tiles[0] > 0;
+    for (int p = 0; p < SP; ++p) redo_any |= *cluster.map_shared_rank(&s_redo, p);
+    if (warp < 16) {
+      const int q = warp >> 3, half = (warp >> 2) & 1;
+      const int rr = q * 128 + (warp & 3) * 32 + lane;
+      float M = -INFINITY, L = 0.f;
+      for (int p = 0; p < SP; ++p) M = fmaxf(M, cluster.map_shared_rank(s_ml, p)[rr].x);
+      for (int p = 0; p < SP; ++p) {
+        const float2 ml = cluster.map_shared_rank(s_ml, p)[rr];
+        if (ml.x > -INFINITY) L = fmaf(ml.y, ex2(ml.x - M), L);
+      }
+      if (half == 0) s_tot[rr] = make_float2(M, L);
+      const float mine = s_ml[rr].x;
+      const float scale = mine > -INFINITY ? ex2(mine - M) : 0.f;
+      float4* dst = reinterpret_cast<float4*>(cluster.map_shared_rank(parts, rr / rows)) +
+                    ((size_t)rank * 32 + half * 16) * rows + rr % rows;
+      const uint32_t tO = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 256 + q * 128 + half * 64;
+#pragma unroll
+      for (int ch = 0; ch < 2; ++ch) {
+        uint32_t ov[32];
+        if (any_tile) {
+          tmem_ld32(tO + ch * 32, ov);
+          tmem_ld_wait();
+        } else {
+#pragma unroll
+          for (int e = 0; e < 32; ++e) ov[e] = 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          dst[(ch * 8 + i) * rows] =
+              make_float4(__uint_as_float(ov[4 * i]) * scale, __uint_as_float(ov[4 * i + 1]) * scale,
+                          __uint_as_float(ov[4 * i + 2]) * scale, __uint_as_float(ov[4 * i + 3]) * scale);
+      }
+    }
+    cluster.sync();  // (from here on a CTA reads its own shared memory only)
+    if (warp < 16 && !s_abort) {
+      // thread = (row, block of `cols` columns); consecutive lanes take consecutive rows
+      const int rl = tid % rows, cols = rows / 4, c0 = (tid / rows) * cols;
+      const int rr = rank * rows + rl, q = rr >> 7, r = rr & 127;
+      const int tk = w.tok0 + rr / G, h = w.g * G + rr % G;
+      const bool row_ok = tk < a.n;
+      const float2 t = s_tot[rr];
+      const size_t stat_at = ((size_t)w.layer * c.chunk + tk) * c.Hq + h;
+      if (phase == 0 && row_ok && c0 == 0) {
+        c.rowstat[stat_at] = t;
+        c.rowq[stat_at] = -t.x - __log2f(t.y) + (21.0f + kMapMargin);
+      }
+      float w0 = 0.f, w1 = 1.f / t.y;  // weights of the stored local part and of the cluster's sum in the output
+      if (MERGE && phase == 2 && row_ok) {
+        const float2 stat0 = c.rowstat[stat_at];
+        const float M = fmaxf(stat0.x, t.x);
+        const float a0 = ex2(stat0.x - M), a1 = t.x == -INFINITY ? 0.f : ex2(t.x - M);
+        const float inv = 1.f / fmaf(stat0.y, a0, t.y * a1);
+        w0 = a0 * inv;
+        w1 = a1 * inv;
+      }
+      const float4* src = reinterpret_cast<const float4*>(parts) + rl;
+      float* state = c.Oacc + oacc_base(w, q) + r * 4;
+      if (row_ok)
+        for (int cg4 = c0 >> 2; cg4 < (c0 + cols) >> 2; cg4 += 2) {  // eight columns at a time
+          float4 o[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int p = 0; p < SP; ++p) {
+              const float4 v = src[((size_t)p * 32 + cg4 + u) * rows];
+              o[u].x += v.x;
+              o[u].y += v.y;
+              o[u].z += v.z;
+              o[u].w += v.w;
+            }
+          }
+          if (phase == 0 && !final_out) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) *reinterpret_cast<float4*>(state + (size_t)(cg4 + u) * 512) = o[u];
+          } else {
+            float4 o0[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+              o0[u] = MERGE && phase == 2 ? *reinterpret_cast<const float4*>(state + (size_t)(cg4 + u) * 512)
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+            uint4 wv;
+            wv.x = pack2(fmaf(o0[0].x, w0, o[0].x * w1), fmaf(o0[0].y, w0, o[0].y * w1));
+            wv.y = pack2(fmaf(o0[0].z, w0, o[0].z * w1), fmaf(o0[0].w, w0, o[0].w * w1));
+            wv.z = pack2(fmaf(o0[1].x, w0, o[1].x * w1), fmaf(o0[1].y, w0, o[1].y * w1));
+            wv.w = pack2(fmaf(o0[1].z, w0, o[1].z * w1), fmaf(o0[1].w, w0, o[1].w * w1));
+            *reinterpret_cast<uint4*>(a.out + (((size_t)w.l * a.n + tk) * c.Hq + h) * kD + cg4 * 4) = wv;
+          }
+        }
+    }
+  }
   // ------------------------------------------------------------------ teardown
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
   if (warp == 16) tmem_dealloc(tmem, 512);
   if (tid == 0 && s_abort) set_status(c, -6, (int)blockIdx.x);
-  if (tid == 0) redo[blockIdx.x] = exch ? 0 : s_redo;  // (the second launch leaves the flags clear for the next call)
+  if (tid == 0) redo[blockIdx.x] = exch ? 0 : (SPLIT ? redo_any : s_redo);  // (the second launch leaves the flags clear for the next call)
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -857,6 +986,18 @@ bool tc_attention_supported(const DevCtx& c) {
   return get_encode() != nullptr;
 }
 
+// CTAs that share a work item: a power of two up to 8 such that all clusters run at once (with one CTA per SM 74, 33 and 15
+// clusters of 2, 4 and 8 fit) and every CTA has at least three of the item's `tiles`.  The layers counted are those of the
+// whole call, so that a call issued in groups of layers gets the same sums as one issued at once.
+static int item_split(const DevCtx& c, const PrefillArgs& a, int tokb, int tiles) {
+  const int nitems = ((a.n + tokb - 1) / tokb) * c.Hkv * a.call_layers;
+  int sp = 1;
+  if (nitems <= 74 && tiles >= 6) sp = 2;
+  if (nitems <= 33 && tiles >= 12) sp = 4;
+  if (nitems <= 15 && tiles >= 24) sp = 8;
+  return sp;
+}
+
 template <int G, bool MERGE>
 static cudaError_t launch_tc_g(const DevCtx& c, const PrefillArgs& a, int phase, bool final_out, const void* kv_maps,
                                cudaStream_t s) {
@@ -876,8 +1017,6 @@ static cudaError_t launch_tc_g(const DevCtx& c, const PrefillArgs& a, int phase,
   }
   constexpr int TOKB = 256 / G;
   const int smem = 65536 + 131072 + 1024;
-  cudaFuncSetAttribute(k_attn_tc<G, false, MERGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_attn_tc<G, true, MERGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const long long v_off = phase == 0 ? (long long)c.NS * c.NL * c.Hkv * c.SR : (long long)c.NL * c.Hkv * c.Rcap;
   static int sms = 0;
   if (sms == 0) {
@@ -891,12 +1030,21 @@ static cudaError_t launch_tc_g(const DevCtx& c, const PrefillArgs& a, int phase,
   // persistent CTAs: one per SM (the kernel needs the whole TMEM and most of the shared memory of an SM)
   const int nitems = ((a.n + TOKB - 1) / TOKB) * c.Hkv * a.layer_count;
   // the regular launch, then the one that redoes the work of the CTAs that asked for it (they return at once otherwise)
-  const int grid = min(nitems, ctas);
+  const int tiles = phase == 0 ? (a.sink_end + 127) / 128 + (a.t0 - a.loc_begin + a.n + 127) / 128 : a.ret_tiles;
+  const int sp = phase == 1 || ctas < sms ? 1 : item_split(c, a, TOKB, tiles);
+  const int grid = sp > 1 ? nitems * sp : min(nitems, ctas);
   if (grid > kTcMaxCtas) return cudaErrorInvalidValue;
-  launch_chained(k_attn_tc<G, false, MERGE>, dim3(grid), dim3(kTcThreads), smem, s, c, a, phase, final_out ? 1 : 0,
-                 c.tc_redo, maps, v_off);
-  return launch_chained(k_attn_tc<G, true, MERGE>, dim3(grid), dim3(kTcThreads), smem, s, c, a, phase, final_out ? 1 : 0,
-                        c.tc_redo, maps, v_off);
+  auto launch = [&](auto fn) {
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return launch_chained_cluster(fn, dim3(grid), dim3(kTcThreads), sp, smem, s, c, a, phase, final_out ? 1 : 0, c.tc_redo,
+                                  maps, v_off);
+  };
+  if (sp > 1) {
+    launch(k_attn_tc<G, false, MERGE, true>);
+    return launch(k_attn_tc<G, true, MERGE, true>);
+  }
+  launch(k_attn_tc<G, false, MERGE, false>);
+  return launch(k_attn_tc<G, true, MERGE, false>);
 }
 
 cudaError_t launch_attn_prefill_tc(const DevCtx& c, const PrefillArgs& a, int phase, bool final_out,

@@ -259,6 +259,7 @@ struct ltri_ctx {
   char* host_kv = nullptr;   // the caller's mirror (host address)
   bool spilled = false;      // ev_spill has been recorded at least once
   cudaEvent_t ev_up[2][kHostGroups] = {}, ev_run[2][kHostGroups] = {}, ev_down[2][kHostGroups] = {};
+  int call_layers = 0;     // > 0 while the host-buffer entry issues a call of that many layers in groups
   int ret_phase = 2;       // retrieved attention: 2 merges with the stored local state, 1 continues from it (testing aid)
   bool grp_used[2][kHostGroups] = {};  // the events of (set, group) have been recorded at least once
   long long host_calls = 0;
@@ -638,6 +639,7 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
   a.seq = seq;
   a.layer_begin = layer_begin;
   a.layer_count = layer_count;
+  a.call_layers = ctx->call_layers > 0 ? ctx->call_layers : layer_count;
   a.n = n_tokens;
   a.t0 = t0;
   a.sink_end = std::min(d.Ls, t0);
@@ -645,6 +647,12 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
   a.reg_start = reg_start;
   a.m = m;
   a.slot = slot;
+  {
+    // about top_k units, or mean spans, of the indexed range
+    const long long indexed = std::max(0, E - d.Ls);
+    const long long item = d.unit > 0 ? d.unit : (ub > 0 ? indexed / ub + 1 : 0);
+    a.ret_tiles = (int)((std::min(indexed, d.topk * item) + 127) / 128);
+  }
   a.q = static_cast<const __nv_bfloat16*>(q);
   a.k = static_cast<const __nv_bfloat16*>(k);
   a.v = static_cast<const __nv_bfloat16*>(v);
@@ -821,7 +829,9 @@ int ltri_prefill_chunk_host(ltri_ctx* ctx, int seq, int layer_begin, int layer_c
     LTRI_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_up[set][g], 0));
     if (ctx->grp_used[set][g]) LTRI_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_down[set][g], 0));
     // (after the checks above this can only fail in the CUDA runtime)
+    ctx->call_layers = layer_count;
     const int rc = ltri_prefill_chunk(ctx, seq, lo, hi - lo, n_tokens, sq + qs, sk + ks, sv + ks, so + qs, st);
+    ctx->call_layers = 0;
     if (rc != LTRI_OK) return rc;
     LTRI_CUDA(ctx, cudaEventRecord(ctx->ev_run[set][g], st));
     // down

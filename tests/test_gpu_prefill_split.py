@@ -1,0 +1,44 @@
+"""Prefill attention with a work item shared by a cluster of 2, 4 or 8 CTAs, against the oracle.
+
+One or two layers of eight query heads on two KV heads are four or eight work items, so the length of the window decides
+how many CTAs share one: six tiles of 128 keys two, twelve four, twenty-four eight.
+"""
+import pytest
+import torch
+
+from paper_2412_04757_b200 import inputs
+from tests import parity_harness as ph
+from tests.test_gpu_parity import small_cfg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("window,context,extra", [
+    (700, 1500, dict()),                                                   # two CTAs
+    (1500, 2300, dict(n_q_heads=2)),                                       # four CTAs, one query head per KV head
+    (3100, 3900, dict(n_layers=1)),                                        # eight CTAs
+    (700, 3200, dict(unit_tokens=64, top_k=12, n_q_heads=16)),             # the retrieved part shared by two as well
+    (700, 4200, dict(n_layers=1, unit_tokens=128, top_k=24, n_q_heads=4)), # ... by eight
+])
+def test_shared_work_items(window, context, extra):
+    kw = dict(n_layers=2, context=context, window=window, decode_steps=1)
+    kw.update(extra)
+    rep = ph.run_stream(small_cfg(**kw), layers=list(range(kw["n_layers"])), deep=False)
+    print(rep)
+
+
+@pytest.mark.parametrize("window", [700, 1500])
+def test_a_key_of_very_large_norm_sends_the_whole_cluster_through_the_second_launch(window):
+    # the logits of one tile exceed every earlier maximum by hundreds of log2 units: the CTA that walks this tile asks for
+    # the second launch, which has to run in all CTAs that share the item
+    cfg = small_cfg(n_layers=1, context=2304, window=window, top_k=12, decode_steps=0)
+    sp = ph.StreamPair(cfg, [0], deep=False)
+    st = inputs.SyntheticStream(cfg)
+    for t0, n in st.prefill_chunks():
+        q, k, v = st.tokens(t0, n)
+        if t0 <= 700 < t0 + n:
+            k[:, 700 - t0, 0, :] = (k[:, 700 - t0, 0, :].float() * 30.0).to(torch.bfloat16)
+        sp.prefill(0, q, k, v)
+    assert sp.lt.ltri_sync_status() == 0
+    sp.lt.close()
+    print(sp.rep)
