@@ -223,7 +223,7 @@ cudaError_t launch_evict_index(const DevCtx& c, const EvictArgs& a, int layer_co
 // Pass 1 counts negatives (only hand-built maps have any) and zeros (a sparse map is mostly zeros) and builds a
 // log-scale histogram of the positive entries: bin = (position of the leading one, next four bits), which is monotone
 // in the value and spreads a heavy-tailed map over many bins.  If the rank falls among the positives, the remaining
-// low bits of the selected bin are resolved by MSB radix passes of 9 bits.  One private histogram per warp, four loads
+// low bits of the selected bin are resolved by MSB radix passes of 9 bits.  One histogram per few warps, four loads
 // in flight per lane; a thread-block cluster of eight CTAs shares a layer: each counts its share of the rows, then
 // every CTA adds up the eight histograms through distributed shared memory and takes the same decision.
 constexpr int kThetaBits = 9;
@@ -901,21 +901,17 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
 #pragma unroll
     for (int e = 0; e < 8; ++e) ug[e] = 0.f;
     if (nrep == 1) {
+      // (four heads at a time, added as they are: a short loop body, because a kernel that runs once per call fetches
+      // every instruction line from L2 and spends more time on that than on the rows)
       const __nv_bfloat16* row = qg + (size_t)(rep_tok[j * kMaxReps] - a.t0) * c.Hq * kD;
-      for (int h0 = 0; h0 < c.G; h0 += 8) {
-        uint4 raw[8];
+#pragma unroll 1
+      for (int h0 = 0; h0 < c.G; h0 += 4) {
+        uint4 raw[4];
 #pragma unroll
-        for (int hh = 0; hh < 8; ++hh)
+        for (int hh = 0; hh < 4; ++hh)
           raw[hh] = counts(h0 + hh) ? *reinterpret_cast<const uint4*>(row + (size_t)(h0 + hh) * kD) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-        for (int hh = 0; hh < 8; ++hh) {
-          float one[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) one[e] = 0.f;
-          add8(one, raw[hh]);  // (0 + x first, as the general path does)
-#pragma unroll
-          for (int e = 0; e < 8; ++e) ug[e] += one[e];
-        }
+        for (int hh = 0; hh < 4; ++hh) add8(ug, raw[hh]);
       }
     } else {
       for (int hh = 0; hh < c.G; ++hh) {
@@ -1198,8 +1194,8 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
       __syncthreads();
     }
   }
-  // more spans than the threads can hold in registers: the order keys are staged in shared memory (room for `stage`)
-  const bool staged = U == 0 && N > kTopkSelRegs * nt && N <= stage;
+  // the order keys are staged in shared memory where the launch left room for `stage` of them
+  const bool staged = U == 0 && N <= stage;
   if (staged) {
     for (int base = tid; base < N; base += 16 * nt) {
       float v[16];
@@ -1223,6 +1219,9 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
     if (tid == 0) s_cnt = K;
   } else if (mode == kTopkVote) {
     radix_select_top<unsigned long long, 0>(KEY64, N, K, hist, &s_prefix64, &s_need, s_scan, &s_cnt, s_ids);
+  } else if (staged || U > 0) {
+    radix_select_top<unsigned, 0>([&](int i) { return ukey[i]; }, N, K, hist, &s_prefix, &s_need, s_scan, &s_cnt, s_ids,
+                                  s_ckey);
   } else {
     radix_select_top<unsigned, kTopkSelRegs>(KEY, N, K, hist, &s_prefix, &s_need, s_scan, &s_cnt, s_ids, s_ckey);
   }
@@ -1950,9 +1949,9 @@ static cudaError_t launch_topk(const DevCtx& c, int seq, int layer_begin, const 
     // Few (layer, KV head) pairs: several CTAs repeat the selection (it costs them nothing: the GPU is idle) and share the
     // packing, which one CTA of 512 threads alone does at some 60 GB/s (one layer, 512 tokens a KV head: 33 us).
     parts = max(1, min(16, 148 / (c.Hkv * gy)));
-    // more spans than 512 threads hold in registers: read once into shared memory, if they fit, instead of once per pass
-    // (only with a CTA per SM to spare: the keys take an SM's shared memory)
-    if (c.unit == 0 && span_bound > kTopkSelRegs * 512 && span_bound <= 48 * 1024 && c.Hkv * gy <= 148) {
+    // With a CTA per SM to spare the scores are read once into shared memory: any number of them that fits, in short
+    // loops (unrolled over 24 registers per thread, the select is 12 KB of instructions that a lone launch fetches cold)
+    if (c.unit == 0 && span_bound <= 48 * 1024 && c.Hkv * gy <= 148) {
       stage = span_bound;
       smem = stage * (int)sizeof(unsigned);
     }
