@@ -28,6 +28,7 @@ using namespace tc;
 
 constexpr float kLog2eT = 1.4426950408889634f;
 constexpr int kTcThreads = 576;  // 16 softmax warps + TMA producer + MMA issuer
+constexpr int kMaxItemSplit = 8;  // most CTAs that share a work item
 constexpr int kNumBoxes = 5;  // box heights 8,16,32,64,128
 constexpr float kRescaleThreshold = 24.0f;
 // Largest exponent (log2 units) a probability may carry above the softmax reference in the regular launch: 2^90 times
@@ -187,8 +188,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int rank = SPLIT ? (int)cg::this_cluster().block_rank() : 0;
   const int item0 = SPLIT ? (int)blockIdx.x / SP : (int)blockIdx.x;
   const int istep = SPLIT ? nitems : (int)gridDim.x;  // (a cluster has one item)
-  __shared__ float2 s_ml[SPLIT ? 256 : 1];     // this CTA's reference maximum and row sum of every row
-  __shared__ float2 s_tot[SPLIT ? 256 : 1];    // those of the cluster
+  // written by every CTA of the cluster: its reference maximum and row sum of every row, its redo flag
+  __shared__ float2 r_ml[SPLIT ? kMaxItemSplit : 1][SPLIT ? 256 : 1];
+  __shared__ int r_redo[kMaxItemSplit];
+  __shared__ float2 s_tot[SPLIT ? 256 : 1];  // those of the cluster
   const uint32_t sbase = (smem_addr(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = sbase;                 // 64 KB: [half d][256 rows][64]
   const uint32_t sKV = sbase + 65536;        // 2 stages x (K 32 KB | V 32 KB), each [half d][128 slots][64]
@@ -222,9 +225,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     fence_mbar_init();
   }
-  // stale shared memory must never hold non-finite bit patterns: unfilled key slots are multiplied by P = 0
-  for (uint32_t i = tid; i < 131072 / 16; i += kTcThreads)
-    asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(sKV + i * 16), "r"(0) : "memory");
+  // the V stages must never hold non-finite bit patterns: unfilled key slots are multiplied by P = 0 (the logits of unfilled
+  // K slots are masked, whatever they are)
+  for (uint32_t i = tid; i < 65536 / 16; i += kTcThreads)
+    asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(sKV + 32768 + (i >> 11) * 65536 + (i & 2047) * 16), "r"(0)
+                 : "memory");
+  if (tid < 1 + kNumBoxes) prefetch_tmap(tid == 0 ? &maps.q : &kvmaps[tid - 1]);
+  if (SPLIT) cg::this_cluster().barrier_arrive();  // (waited for in front of the first store to another CTA)
   fence_async_smem();
   if (warp == 16) tmem_alloc(smem_addr(&s_tmem_base), 512);
   fence_before_sync();
@@ -233,6 +240,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const uint32_t tmem = s_tmem_base;
   if (!exch) chain_wait();  // everything above set up shared memory, barriers and TMEM only
   const int causal_ri = phase == 0 ? 2 : -1;
+
+  float2 split_ml = make_float2(-INFINITY, 0.f);  // SPLIT: a softmax thread's row at the end of its tiles
 
   // decode a work item
   struct Item {
@@ -263,7 +272,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // Every lane walks the tile list; lane 0 owns the barrier bookkeeping and lanes 0-3 issue the copies of
     // (K low half, K high half, V low half, V high half) so that many small pieces do not serialise on one thread.
     int jt = 0, ok = 1;
-    if (lane == 0) prefetch_tmap(&maps.q);
     for (int item = item0, wi = 0; ok && item < nitems; item += istep, ++wi) {
       const Item w = decode(item);
       if (lane == 0) {
@@ -710,7 +718,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       asm volatile("bar.sync %0, 256;" ::"r"(1 + q) : "memory");  // also: s_sum is reused by the next item
       if (s_quit[q]) break;  // collective decision: all 256 threads of the tile leave after the same item
       if (SPLIT) {  // merged with the other CTAs' parts below
-        if (half == 0) s_ml[rr] = make_float2(m_used, lsum);
+        split_ml = make_float2(m_used, lsum);
         break;
       }
       fence_after_sync();
@@ -812,6 +820,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // wait.
     cg::cluster_group cluster = cg::this_cluster();
     __syncwarp();
+    cluster.barrier_wait();  // (of the arrival at the start: every CTA of the cluster runs)
+    // pushed, not fetched: a fetch is a round trip of some 700 cycles per CTA and row
+    if (warp < 16 && ((warp >> 2) & 1) == 0) {
+      const int rr = (warp >> 3) * 128 + (warp & 3) * 32 + lane;
+      for (int p = 0; p < SP; ++p) cluster.map_shared_rank(&r_ml[rank][0], p)[rr] = split_ml;
+    }
+    __syncwarp();
     fence_before_sync();
     cluster.sync();  // all products of all CTAs have completed, the (m, l) of all rows are there
     fence_after_sync();
@@ -819,18 +834,18 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     float* parts = reinterpret_cast<float*>(smem_raw + (sKV - smem_addr(smem_raw)));
     const Item w = decode(item0);
     const bool any_tile = s_item_tiles[0] > 0;
-    for (int p = 0; p < SP; ++p) redo_any |= *cluster.map_shared_rank(&s_redo, p);
+    if (tid < SP) *cluster.map_shared_rank(&r_redo[rank], tid) = s_redo;
     if (warp < 16) {
       const int q = warp >> 3, half = (warp >> 2) & 1;
       const int rr = q * 128 + (warp & 3) * 32 + lane;
       float M = -INFINITY, L = 0.f;
-      for (int p = 0; p < SP; ++p) M = fmaxf(M, cluster.map_shared_rank(s_ml, p)[rr].x);
+      for (int p = 0; p < SP; ++p) M = fmaxf(M, r_ml[p][rr].x);
       for (int p = 0; p < SP; ++p) {
-        const float2 ml = cluster.map_shared_rank(s_ml, p)[rr];
+        const float2 ml = r_ml[p][rr];
         if (ml.x > -INFINITY) L = fmaf(ml.y, ex2(ml.x - M), L);
       }
       if (half == 0) s_tot[rr] = make_float2(M, L);
-      const float mine = s_ml[rr].x;
+      const float mine = r_ml[rank][rr].x;
       const float scale = mine > -INFINITY ? ex2(mine - M) : 0.f;
       float4* dst = reinterpret_cast<float4*>(cluster.map_shared_rank(parts, rr / rows)) +
                     ((size_t)rank * 32 + half * 16) * rows + rr % rows;
@@ -853,6 +868,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
     }
     cluster.sync();  // (from here on a CTA reads its own shared memory only)
+    for (int p = 0; p < SP; ++p) redo_any |= r_redo[p];
     if (warp < 16 && !s_abort) {
       // thread = (row, block of `cols` columns); consecutive lanes take consecutive rows
       const int rl = tid % rows, cols = rows / 4, c0 = (tid / rows) * cols;
@@ -987,14 +1003,15 @@ bool tc_attention_supported(const DevCtx& c) {
 }
 
 // CTAs that share a work item: a power of two up to 8 such that all clusters run at once (with one CTA per SM 74, 33 and 15
-// clusters of 2, 4 and 8 fit) and every CTA has at least three of the item's `tiles`.  The layers counted are those of the
+// clusters of 2, 4 and 8 fit) and every CTA has at least two of the item's `tiles` (a cluster
+// costs some 8K cycles for the merge, a tile 3.6K).  The layers counted are those of the
 // whole call, so that a call issued in groups of layers gets the same sums as one issued at once.
 static int item_split(const DevCtx& c, const PrefillArgs& a, int tokb, int tiles) {
   const int nitems = ((a.n + tokb - 1) / tokb) * c.Hkv * a.call_layers;
   int sp = 1;
-  if (nitems <= 74 && tiles >= 6) sp = 2;
-  if (nitems <= 33 && tiles >= 12) sp = 4;
-  if (nitems <= 15 && tiles >= 24) sp = 8;
+  if (nitems <= 74 && tiles >= 4) sp = 2;
+  if (nitems <= 33 && tiles >= 8) sp = 4;
+  if (nitems <= 15 && tiles >= 16) sp = 8;
   return sp;
 }
 

@@ -1,7 +1,7 @@
 """Prefill attention with a work item shared by a cluster of 2, 4 or 8 CTAs, against the oracle.
 
 One or two layers of eight query heads on two KV heads are four or eight work items, so the length of the window decides
-how many CTAs share one: six tiles of 128 keys two, twelve four, twenty-four eight.
+how many CTAs share one: four tiles of 128 keys two, eight four, sixteen eight.
 """
 import pytest
 import torch
@@ -14,10 +14,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("window,context,extra", [
-    (700, 1500, dict()),                                                   # two CTAs
+    (500, 1500, dict()),                                                   # two CTAs, then four
     (1500, 2300, dict(n_q_heads=2)),                                       # four CTAs, one query head per KV head
     (3100, 3900, dict(n_layers=1)),                                        # eight CTAs
-    (700, 3200, dict(unit_tokens=64, top_k=12, n_q_heads=16)),             # the retrieved part shared by two as well
+    (700, 3200, dict(unit_tokens=64, top_k=12, n_q_heads=16)),             # the retrieved part shared as well
     (700, 4200, dict(n_layers=1, unit_tokens=128, top_k=24, n_q_heads=4)), # ... by eight
 ])
 def test_shared_work_items(window, context, extra):
