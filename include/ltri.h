@@ -264,7 +264,8 @@ enum {
   LTRI_K_SCORE_TOPK,   /* prefill similarity scores + top-k (Eq. 7-8) */
   LTRI_K_ATTN_RET,     /* prefill attention over the retrieved spans + merge */
   LTRI_K_DEC_RETRIEVE, /* decode scores + top-k */
-  LTRI_K_DEC_ATTN,     /* decode split-KV attention + merge */
+  LTRI_K_DEC_ATTN,     /* decode split-KV attention + merge; a step that runs as one launch (few sequences x layers x KV heads)
+                          counts here as a whole */
   LTRI_K_PAGER_PULL,   /* host-memory pager: pulls of missing units + gather (on the pager's own stream: overlaps
                           the other classes) */
   LTRI_K_COUNT

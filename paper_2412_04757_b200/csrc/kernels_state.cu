@@ -1195,7 +1195,7 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
     }
   }
   // the order keys are staged in shared memory where the launch left room for `stage` of them
-  const bool staged = U == 0 && N <= stage;
+  const bool staged = !DECODE && U == 0 && N <= stage;
   if (staged) {
     for (int base = tid; base < N; base += 16 * nt) {
       float v[16];
@@ -1219,7 +1219,7 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
     if (tid == 0) s_cnt = K;
   } else if (mode == kTopkVote) {
     radix_select_top<unsigned long long, 0>(KEY64, N, K, hist, &s_prefix64, &s_need, s_scan, &s_cnt, s_ids);
-  } else if (staged || U > 0) {
+  } else if (!DECODE && (staged || U > 0)) {
     radix_select_top<unsigned, 0>([&](int i) { return ukey[i]; }, N, K, hist, &s_prefix, &s_need, s_scan, &s_cnt, s_ids,
                                   s_ckey);
   } else {

@@ -860,8 +860,11 @@ int ltri_host_outputs_ready(ltri_ctx* ctx, void* cuda_stream) {
 // holds no shared memory for tiles and leaves more CTAs per SM to hide the latency, stream it faster (33K spans, 32
 // units: 92 against 103 us a step).
 constexpr int kStepSpans = 2560;
-// The same holds for the tokens a CTA attends over, of which it keeps one 16-token tile per warp on the way (12.7K tokens
-// per unit, 64 units: 124 us a step against 130 us as clusters of four).
+// With unit-granular retrieval a step may attend over thousands of scattered tokens per unit, which the split-KV kernel with
+// three CTAs per SM streams faster than a CTA that keeps one 16-token tile per warp on the way (12.7K tokens per unit, 64
+// units: 124 us a step against 130 us as clusters of four).  Spans are few tokens beside the recent ones, and the recent
+// ones stream well either way (64 units, 3K to 15K recent tokens: 46 to 101 us a step as clusters of four, 59 to 116 us as
+// separate launches).
 constexpr int kStepTokens = 1536;
 static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, long long ub) {
   const DevCtx& d = ctx->d;
@@ -877,7 +880,7 @@ static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, 
   for (int i = 4; i >= 1; --i) {
     const int cl = 1 << i;
     if (ctx->step_cluster > 0 ? cl != ctx->step_cluster : known / cl < 64 && cl > 2) continue;
-    if (ctx->step_cluster == 0 && ((d.unit == 0 && ub > (long long)kStepSpans * cl) || tokens > kStepTokens * cl)) continue;
+    if (ctx->step_cluster == 0 && ((d.unit == 0 && ub > (long long)kStepSpans * cl) || (d.unit > 0 && tokens > kStepTokens * cl))) continue;
     if ((long long)units * cl <= ctx->step_cap[i] && dec_step_fits(d, (int)ub, e_max, cl)) return cl;
   }
   return 0;
