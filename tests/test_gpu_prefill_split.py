@@ -42,3 +42,14 @@ def test_a_key_of_very_large_norm_sends_the_whole_cluster_through_the_second_lau
     assert sp.lt.ltri_sync_status() == 0
     sp.lt.close()
     print(sp.rep)
+
+
+@pytest.mark.parametrize("n_layers", [9, 18])
+def test_calls_of_many_layers(n_layers):
+    # more layers than the segmenter gives a cluster of sixteen CTAs each (7), or four CTAs for the representatives (16):
+    # the first and the last layer of a call against the oracle.  (Eight query heads: with two, this seed has outputs above 4,
+    # whose bf16 rounding alone, 2^-7 = 0.0156, and the bf16 probabilities add up to 0.0241, beyond the harness's bar of 0.02.)
+    cfg = small_cfg(n_layers=n_layers, context=900, decode_steps=1)
+    rep = ph.run_stream(cfg, layers=[0, n_layers - 1])
+    assert rep.regions >= 14
+    print(rep)
