@@ -162,6 +162,19 @@ struct PrefillArgs {
 };
 
 // ---- launch wrappers (each returns the cudaError_t of the launch) -------------------
+// Function attributes: the limit of dynamic shared memory of every kernel a context may launch, and the leave for
+// clusters of sixteen.  They belong to the function on the device, not to a context, so they are set when a context is
+// created, at the largest value that any context needs, and never in front of a launch: a limit that follows the size
+// of one call would refuse the larger launch that another context's thread is about to make.
+cudaError_t prepare_kernels(const DevCtx& c, bool tensor_cores);
+cudaError_t prepare_attn(const DevCtx& c);  // the parts of prepare_kernels, one per kernel file
+cudaError_t prepare_attn_tc(const DevCtx& c);
+cudaError_t prepare_map_tc(const DevCtx& c);
+cudaError_t prepare_score();
+cudaError_t prepare_score_tc();
+cudaError_t prepare_state();
+cudaError_t prepare_decode(const DevCtx& c);
+cudaError_t prepare_dec_step(const DevCtx& c);
 cudaError_t launch_init(const DevCtx& c, int seq /* -1: all */, cudaStream_t s);
 cudaError_t launch_append_prefill(const DevCtx& c, const PrefillArgs& a, bool clear_maps, bool late_wait, cudaStream_t s);
 cudaError_t launch_append_decode(const DevCtx& c, const DecBatch& b, int layer_begin, int layer_count, int n_seqs_total,
@@ -235,6 +248,22 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 // wait for the eviction kernel at their end instead of their beginning, so that the two run side by side and
 // everything behind the append kernel still follows both.
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Dynamic shared memory that `fn` may ask for at a launch; bytes < 0: all that its static arrays leave of a block's limit.
+template <typename F>
+inline cudaError_t allow_smem(F* fn, int bytes) {
+  if (bytes < 0) {
+    int dev = 0;
+    cudaFuncAttributes at;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
+    if (e != cudaSuccess) return e;
+    bytes -= (int)at.sharedSizeBytes;
+  }
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+inline cudaError_t first_error(cudaError_t a, cudaError_t b) { return a != cudaSuccess ? a : b; }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_chained_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem,

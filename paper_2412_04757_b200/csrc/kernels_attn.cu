@@ -232,12 +232,12 @@ __global__ void __launch_bounds__(256, 1) k_attn_prefill(DevCtx c, PrefillArgs a
   }
 }
 
+constexpr int kAttnSmem = 32768 * 3, kMapLocalSmem = 3 * 16384, kMapCurSmem = 4 * 16384;
+
 template <int G>
 static cudaError_t launch_attn_g(const DevCtx& c, const PrefillArgs& a, int phase, bool final_out, cudaStream_t s) {
   constexpr int TOK = 128 / G;
-  const int smem = 32768 * 3;
-  cudaFuncSetAttribute(k_attn_prefill<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  k_attn_prefill<G><<<dim3((a.n + TOK - 1) / TOK, c.Hkv, a.layer_count), 256, smem, s>>>(c, a, phase, final_out ? 1 : 0);
+  k_attn_prefill<G><<<dim3((a.n + TOK - 1) / TOK, c.Hkv, a.layer_count), 256, kAttnSmem, s>>>(c, a, phase, final_out ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -450,12 +450,10 @@ template <int G>
 static cudaError_t launch_map_g(const DevCtx& c, const PrefillArgs& a, cudaStream_t s) {
   const int nloc = a.t0 - a.loc_begin;
   if (nloc > 0 && a.loc_begin >= c.Ls) {
-    cudaFuncSetAttribute(k_map_local<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * 16384);
-    k_map_local<G><<<dim3((nloc + 63) / 64, c.Hkv, a.layer_count), 128, 3 * 16384, s>>>(c, a);
+    k_map_local<G><<<dim3((nloc + 63) / 64, c.Hkv, a.layer_count), 128, kMapLocalSmem, s>>>(c, a);
   }
   const int nt = (a.n + 63) / 64;
-  cudaFuncSetAttribute(k_map_cur<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 16384);
-  k_map_cur<G><<<dim3(nt * (nt + 1) / 2, a.layer_count), 128, 4 * 16384, s>>>(c, a);
+  k_map_cur<G><<<dim3(nt * (nt + 1) / 2, a.layer_count), 128, kMapCurSmem, s>>>(c, a);
   return cudaGetLastError();
 }
 
@@ -465,6 +463,22 @@ cudaError_t launch_map_pass(const DevCtx& c, const PrefillArgs& a, cudaStream_t 
     case 2: return launch_map_g<2>(c, a, s);
     case 4: return launch_map_g<4>(c, a, s);
     case 8: return launch_map_g<8>(c, a, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <int G>
+static cudaError_t prepare_attn_g() {
+  return first_error(allow_smem(k_attn_prefill<G>, kAttnSmem),
+                     first_error(allow_smem(k_map_local<G>, kMapLocalSmem), allow_smem(k_map_cur<G>, kMapCurSmem)));
+}
+
+cudaError_t prepare_attn(const DevCtx& c) {
+  switch (c.G) {
+    case 1: return prepare_attn_g<1>();
+    case 2: return prepare_attn_g<2>();
+    case 4: return prepare_attn_g<4>();
+    case 8: return prepare_attn_g<8>();
   }
   return cudaErrorInvalidValue;
 }

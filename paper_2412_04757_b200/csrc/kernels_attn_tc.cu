@@ -1015,6 +1015,28 @@ static int item_split(const DevCtx& c, const PrefillArgs& a, int tokb, int tiles
   return sp;
 }
 
+constexpr int kTcSmem = 65536 + 131072 + 1024;  // queries, two K/V stages, alignment
+
+template <int G>
+static cudaError_t prepare_tc_g() {
+  cudaError_t e = cudaSuccess;
+  for (auto fn : {k_attn_tc<G, false, false, false>, k_attn_tc<G, false, false, true>, k_attn_tc<G, false, true, false>,
+                  k_attn_tc<G, false, true, true>, k_attn_tc<G, true, false, false>, k_attn_tc<G, true, false, true>,
+                  k_attn_tc<G, true, true, false>, k_attn_tc<G, true, true, true>})
+    e = first_error(e, allow_smem(fn, kTcSmem));
+  return e;
+}
+
+cudaError_t prepare_attn_tc(const DevCtx& c) {
+  switch (c.G) {
+    case 1: return prepare_tc_g<1>();
+    case 2: return prepare_tc_g<2>();
+    case 4: return prepare_tc_g<4>();
+    case 8: return prepare_tc_g<8>();
+  }
+  return cudaErrorInvalidValue;
+}
+
 template <int G, bool MERGE>
 static cudaError_t launch_tc_g(const DevCtx& c, const PrefillArgs& a, int phase, bool final_out, const void* kv_maps,
                                cudaStream_t s) {
@@ -1033,7 +1055,6 @@ static cudaError_t launch_tc_g(const DevCtx& c, const PrefillArgs& a, int phase,
       return cudaErrorInvalidValue;
   }
   constexpr int TOKB = 256 / G;
-  const int smem = 65536 + 131072 + 1024;
   const long long v_off = phase == 0 ? (long long)c.NS * c.NL * c.Hkv * c.SR : (long long)c.NL * c.Hkv * c.Rcap;
   static int sms = 0;
   if (sms == 0) {
@@ -1052,8 +1073,7 @@ static cudaError_t launch_tc_g(const DevCtx& c, const PrefillArgs& a, int phase,
   const int grid = sp > 1 ? nitems * sp : min(nitems, ctas);
   if (grid > kTcMaxCtas) return cudaErrorInvalidValue;
   auto launch = [&](auto fn) {
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    return launch_chained_cluster(fn, dim3(grid), dim3(kTcThreads), sp, smem, s, c, a, phase, final_out ? 1 : 0, c.tc_redo,
+    return launch_chained_cluster(fn, dim3(grid), dim3(kTcThreads), sp, kTcSmem, s, c, a, phase, final_out ? 1 : 0, c.tc_redo,
                                   maps, v_off);
   };
   if (sp > 1) {

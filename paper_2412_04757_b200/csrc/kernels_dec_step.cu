@@ -632,15 +632,16 @@ static DecStepFn dec_step_fn(int G) {
   return G == 1 ? k_dec_step<1> : G == 2 ? k_dec_step<2> : G == 4 ? k_dec_step<4> : k_dec_step<8>;
 }
 
-// CTAs of k_dec_step that fit the GPU at once as clusters of `cluster` CTAs; also sets the kernel's attributes.
+cudaError_t prepare_dec_step(const DevCtx& c) {
+  const DecStepFn fn = dec_step_fn(c.G);
+  return first_error(allow_smem(fn, dec_step_smem(kStMaxSlots)),
+                     cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+}
+
+// CTAs of k_dec_step that fit the GPU at once as clusters of `cluster` CTAs (after prepare_dec_step).
 int dec_step_capacity(const DevCtx& c, int cluster) {
   const DecStepFn fn = dec_step_fn(c.G);
   const int smem = dec_step_smem(kStMaxSlots);
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cluster, c.Hkv, 1);
   cfg.blockDim = dim3(kStThreads);

@@ -174,12 +174,22 @@ __global__ void __launch_bounds__(kD) k_decode_merge(DevCtx c, DecBatch b, int l
   out[(((size_t)b.src[bi] * layer_count + l) * c.Hq + h) * kD + e] = __float2bfloat16(ot / lt);
 }
 
+constexpr int kDecSmem = 4 * kDWarpBytes;
+
+cudaError_t prepare_decode(const DevCtx& c) {
+  switch (c.G) {
+    case 1: return allow_smem(k_decode_attn<1>, kDecSmem);
+    case 2: return allow_smem(k_decode_attn<2>, kDecSmem);
+    case 4: return allow_smem(k_decode_attn<4>, kDecSmem);
+    case 8: return allow_smem(k_decode_attn<8>, kDecSmem);
+  }
+  return cudaErrorInvalidValue;
+}
+
 template <int G>
 static cudaError_t launch_dec_g(const DevCtx& c, const DecBatch& b, int layer_begin, int layer_count,
                                 const __nv_bfloat16* q, __nv_bfloat16* out, int nsplit, cudaStream_t s) {
-  const int smem = 4 * kDWarpBytes;
-  cudaFuncSetAttribute(k_decode_attn<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  launch_chained(k_decode_attn<G>, dim3(nsplit, c.Hkv, b.n * layer_count), dim3(kDecThreads), smem, s, c, b, layer_begin,
+  launch_chained(k_decode_attn<G>, dim3(nsplit, c.Hkv, b.n * layer_count), dim3(kDecThreads), kDecSmem, s, c, b, layer_begin,
                  layer_count, q, nsplit);
   return launch_chained(k_decode_merge, dim3(c.Hq, b.n * layer_count), dim3(kD), 0, s, c, b, layer_begin, layer_count, out,
                         nsplit);

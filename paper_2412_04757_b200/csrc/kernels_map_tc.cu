@@ -354,6 +354,8 @@ typedef CUresult (*EncodeFnM)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
                               const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+constexpr int kMapSmem = kMapKT * 32768 + 65536 + 3 * 4096 + 1024;  // key tiles, two query stages, the offset tiles
+
 template <int G>
 static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, cudaStream_t s) {
   static EncodeFnM enc = nullptr;
@@ -402,10 +404,18 @@ static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const 
       }
   }
   const int gloc = (nloc + kt - 1) / kt, gcur = (ncur + kt - 1) / kt;
-  const int smem = kMapKT * 32768 + 65536 + 3 * 4096 + 1024;  // key tiles, two query stages, the offset tiles
-  cudaFuncSetAttribute(k_map_tc<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  return launch_chained(k_map_tc<G>, dim3((gloc + gcur) * qs, c.Hkv, a.layer_count), dim3(kMapThreads), smem, s, c, a, gloc,
-                        nloc, ncur, kt, qs, maps);
+  return launch_chained(k_map_tc<G>, dim3((gloc + gcur) * qs, c.Hkv, a.layer_count), dim3(kMapThreads), kMapSmem, s, c, a,
+                        gloc, nloc, ncur, kt, qs, maps);
+}
+
+cudaError_t prepare_map_tc(const DevCtx& c) {
+  switch (c.G) {
+    case 1: return allow_smem(k_map_tc<1>, kMapSmem);
+    case 2: return allow_smem(k_map_tc<2>, kMapSmem);
+    case 4: return allow_smem(k_map_tc<4>, kMapSmem);
+    case 8: return allow_smem(k_map_tc<8>, kMapSmem);
+  }
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_map_pass_tc(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, cudaStream_t s) {

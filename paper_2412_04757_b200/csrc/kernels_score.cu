@@ -108,10 +108,11 @@ __global__ void __launch_bounds__(128) k_score_mma(DevCtx c, int seq, int layer_
   }
 }
 
+cudaError_t prepare_score() { return allow_smem(k_score_mma, -1); }
+
 cudaError_t launch_score_prefill_mma(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s) {
   const int njb_max = (c.Jmax + 63) / 64;
   const int smem = njb_max * 3 * 16384 + kScoreStages * 16384;
-  cudaFuncSetAttribute(k_score_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const int tiles = (span_bound + 63) / 64;
   // enough tiles per CTA to amortise the split of the representatives, enough CTAs to fill the GPU
   const int per_cta = tiles >= 512 ? 32 : 16;

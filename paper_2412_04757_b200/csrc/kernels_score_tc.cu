@@ -197,14 +197,10 @@ cudaError_t launch_score_prefill_tc(const DevCtx& c, const PrefillArgs& a, int s
   const int per_cta = max(1, min(tiles >= 256 ? 32 : (tiles >= 48 ? 16 : 8), (tiles * c.Hkv * a.layer_count + slots - 1) / slots));
   const int gx = (tiles + per_cta - 1) / per_cta;
   const dim3 grid(gx > 0 ? gx : 1, c.Hkv, a.layer_count);
-  if (two) {
-    cudaFuncSetAttribute(k_score_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    return launch_chained(k_score_tc<2>, grid, dim3(kScThreads), smem, s, c, a.seq, a.layer_begin, per_cta, npad_lay, kr);
-  } else {
-    cudaFuncSetAttribute(k_score_tc<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    return launch_chained(k_score_tc<3>, grid, dim3(kScThreads), smem, s, c, a.seq, a.layer_begin, per_cta, npad_lay, kr);
-  }
-  return cudaGetLastError();
+  return launch_chained(two ? k_score_tc<2> : k_score_tc<3>, grid, dim3(kScThreads), smem, s, c, a.seq, a.layer_begin, per_cta,
+                        npad_lay, kr);
 }
+
+cudaError_t prepare_score_tc() { return first_error(allow_smem(k_score_tc<2>, -1), allow_smem(k_score_tc<3>, -1)); }
 
 }  // namespace ltri

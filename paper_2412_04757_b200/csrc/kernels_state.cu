@@ -938,6 +938,7 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
 }
 
 constexpr int kSegWideLayers = 7;    // clusters of 16 that run at once
+constexpr int kThetaWideSmem = 32 * kThetaBins * (int)sizeof(unsigned);  // a histogram per warp
 constexpr int kSegShareLayers = 16;  // up to here four CTAs share a layer's representatives
 
 cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start,
@@ -951,11 +952,8 @@ cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_
     // Few layers: 16 CTAs of 1024 threads share one, which gives every pair of rows a warp of its own (a cluster of 16
     // needs a GPC to itself, so seven run at once).  More: 8 CTAs of 512 threads.
     if (layer_count <= kSegWideLayers) {
-      const int hsmem = 32 * kThetaBins * (int)sizeof(unsigned);
       auto fn = m <= 512 ? k_theta_select<17> : k_theta_select<33>;
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, hsmem);
-      cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      launch_chained_cluster(fn, dim3(layer_count * 16), dim3(1024), 16, hsmem, s, c, layer_begin, m, rank, tables ? 1 : 0);
+      launch_chained_cluster(fn, dim3(layer_count * 16), dim3(1024), 16, kThetaWideSmem, s, c, layer_begin, m, rank, tables ? 1 : 0);
     } else {
       const int hsmem = (kThetaThreads / 32) * kThetaBins * (int)sizeof(unsigned);
       launch_chained_cluster(k_theta_select<0>, dim3(layer_count * 8), dim3(kThetaThreads), 8, hsmem, s, c, layer_begin, m,
@@ -1044,7 +1042,6 @@ cudaError_t launch_score_prefill(const DevCtx& c, const PrefillArgs& a, int span
   DecBatch dummy;
   dummy.n = 0;
   const size_t smem = (size_t)c.Jmax * kD * sizeof(float);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k_score<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k_score<false><<<dim3((span_bound + 63) / 64, c.Hkv, a.layer_count), 256, smem, s>>>(c, a.seq, a.layer_begin, dummy,
                                                                                        a.layer_count, nullptr);
   return cudaGetLastError();
@@ -1938,6 +1935,17 @@ static int topk_unit_smem(const DevCtx& c) {
   return (int)sizeof(unsigned) * (c.vote ? 2 * n + 4 : n);
 }
 
+constexpr int kTopkStage = 48 * 1024;  // most order keys a prefill select keeps in shared memory
+
+cudaError_t prepare_state() {
+  cudaError_t e = cudaSuccess;
+  for (auto fn : {k_theta_select<17>, k_theta_select<33>})
+    e = first_error(e, first_error(allow_smem(fn, kThetaWideSmem),
+                                   cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)));
+  for (auto fn : {k_topk<false>, k_topk<true>}) e = first_error(e, allow_smem(fn, -1));
+  return first_error(e, allow_smem(k_score<false>, -1));
+}
+
 // Top-k of the call.  Under collaborative voting (Sec. 3.5) two launches: the ballots of the layers with a retrieval
 // head, then the vote (a layer reads the ballots of the layers up to its own, also those of earlier calls for the same
 // chunk or step).
@@ -1951,14 +1959,10 @@ static cudaError_t launch_topk(const DevCtx& c, int seq, int layer_begin, const 
     parts = max(1, min(16, 148 / (c.Hkv * gy)));
     // With a CTA per SM to spare the scores are read once into shared memory: any number of them that fits, in short
     // loops (unrolled over 24 registers per thread, the select is 12 KB of instructions that a lone launch fetches cold)
-    if (c.unit == 0 && span_bound <= 48 * 1024 && c.Hkv * gy <= 148) {
+    if (c.unit == 0 && span_bound <= kTopkStage && c.Hkv * gy <= 148) {
       stage = span_bound;
       smem = stage * (int)sizeof(unsigned);
     }
-  }
-  if (smem > 32 * 1024) {  // (static shared memory comes on top: ask for the larger limit in good time)
-    cudaError_t e = cudaFuncSetAttribute(k_topk<DECODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
   }
   if (c.vote)
     launch_chained(k_topk<DECODE>, dim3(c.Hkv, gy), dim3(512), smem, s, c, seq, layer_begin, b, layer_count, evicted_end,

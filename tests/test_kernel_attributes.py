@@ -1,0 +1,35 @@
+"""Function attributes (a kernel's limit of dynamic shared memory) belong to the device, not to a context.  A launch that set
+one to the size of its own call could lower it under the larger launch that another context's thread is about to make, which
+is then refused half-way through a call.  The window between the two is too narrow to be hit on demand, so the rule itself
+is checked: attributes are set by the prepare functions, which ltri_create runs, and nowhere else."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "..", "paper_2412_04757_b200", "csrc")
+FILES = sorted(os.path.basename(f) for f in glob.glob(os.path.join(CSRC, "*.cu*")))
+# a definition at the start of a line: its name, then everything up to the closing brace in the first column
+FUNCTION = re.compile(r"^[A-Za-z][^\n;=]*?\b(\w+)\([^;{}]*\)\s*\{.*?^\}", re.M | re.S)
+
+
+@pytest.mark.parametrize("name", FILES)
+def test_attributes_are_set_when_a_context_is_created_only(name):
+    text = open(os.path.join(CSRC, name)).read()
+    calls = text.count("cudaFuncSetAttribute(") + text.count("allow_smem(")
+    inside = 0
+    for f in FUNCTION.finditer(text):
+        n = f.group(0).count("cudaFuncSetAttribute(") + f.group(0).count("allow_smem(")
+        assert n == 0 or f.group(1).startswith("prepare_") or f.group(1) == "allow_smem", f"{name}: {f.group(1)} sets a limit"
+        inside += n
+    assert inside == calls, f"{name}: an attribute is set outside the functions seen here"
+
+
+def test_every_prepare_function_runs_at_creation():
+    text = {f: open(os.path.join(CSRC, f)).read() for f in FILES}
+    parts = set(re.findall(r"^cudaError_t (prepare_\w+)\([^;]*;", text["common.cuh"], re.M)) - {"prepare_kernels"}
+    body = [f.group(0) for f in FUNCTION.finditer(text["ltri_api.cu"]) if f.group(1) == "prepare_kernels"]
+    assert len(body) == 1 and parts and all(p + "(" in body[0] for p in parts)
+    create = [f.group(0) for f in FUNCTION.finditer(text["ltri_api.cu"]) if f.group(1) == "ltri_create"]
+    assert len(create) == 1 and "prepare_kernels(ctx->d" in create[0]
