@@ -1943,6 +1943,9 @@ cudaError_t prepare_state() {
     e = first_error(e, first_error(allow_smem(fn, kThetaWideSmem),
                                    cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)));
   for (auto fn : {k_topk<false>, k_topk<true>}) e = first_error(e, allow_smem(fn, -1));
+  // (48 KB of keys beside the static arrays: more than a kernel may use without asking)
+  e = first_error(e, first_error(allow_smem(k_dec_retrieve, kFusedMaxSpans * (int)sizeof(unsigned)),
+                                 allow_smem(k_dec_retrieve_cl, kRetSliceMax * (int)sizeof(float))));
   return first_error(e, allow_smem(k_score<false>, -1));
 }
 
