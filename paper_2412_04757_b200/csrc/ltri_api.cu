@@ -903,6 +903,21 @@ static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, 
   return 0;
 }
 
+// Whether the one-launch step may write `out`.  Its clusters read their queries and the new K/V rows and write their outputs
+// on their own, so a buffer that shares memory with `out` has to be read by the cluster that overwrites it and by no other:
+// true of queries replaced by their own outputs, except under a retrieval head, whose queries every KV head reads.  The
+// separate launches have read everything before the first output is written.
+static bool step_may_write(const ltri_ctx* ctx, const void* out, const void* q, const void* k, const void* v, size_t rows) {
+  const DevCtx& d = ctx->d;
+  const size_t qn = rows * d.Hq * kD * sizeof(__nv_bfloat16), kn = rows * d.Hkv * kD * sizeof(__nv_bfloat16);
+  const uintptr_t o = reinterpret_cast<uintptr_t>(out);
+  auto apart = [&](const void* p, size_t n) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(p);
+    return x + n <= o || o + qn <= x;
+  };
+  return (apart(q, qn) || (q == out && ctx->ret_head.empty())) && apart(k, kn) && apart(v, kn);
+}
+
 int ltri_decode_step(ltri_ctx* ctx, const int32_t* seq_ids, int n_seqs, int layer_begin, int layer_count,
                      const void* q, const void* k, const void* v, void* out, void* cuda_stream) {
   if (!ctx || !seq_ids) return LTRI_EINVAL;
@@ -949,6 +964,7 @@ int ltri_decode_step(ltri_ctx* ctx, const int32_t* seq_ids, int n_seqs, int laye
       }
     }
   }
+  const bool one_launch = step_may_write(ctx, out, q, k, v, (size_t)n_seqs * layer_count);
   for (int i0 = 0; i0 < n_seqs; i0 += kDecBatch) {
     DecBatch b;
     b.n = std::min(kDecBatch, n_seqs - i0);
@@ -961,7 +977,7 @@ int ltri_decode_step(ltri_ctx* ctx, const int32_t* seq_ids, int n_seqs, int laye
       b.shift[i] = d.paged ? s.base - d.Lsp : 0;
     }
     const int units = b.n * layer_count * d.Hkv;
-    if (const int cl = step_cluster_size(ctx, b, units, ub)) {
+    if (const int cl = one_launch ? step_cluster_size(ctx, b, units, ub) : 0) {
       int e_max = 0;
       for (int i = 0; i < b.n; ++i) e_max = std::max(e_max, b.loc_begin[i]);
       Scope sc(ctx, st, LTRI_K_DEC_ATTN, 1);
