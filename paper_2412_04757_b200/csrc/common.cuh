@@ -112,6 +112,10 @@ struct DevCtx {
   int* status;           // [4]: first error code, detail...
   int* tc_redo;          // [kTcMaxCtas]  per CTA of the tensor-core attention kernel: its work has to be redone
   long long wait_limit;  // upper bound of any single device-side wait, in SM clock cycles
+  // what the device offers, read by the dispatch on the host (ltri_create asks; see kernels_state.cu and kernels_attn_tc.cu)
+  int sms;               // streaming multiprocessors
+  int theta_wide;        // layers whose threshold select may take a cluster of sixteen CTAs each (0: no such cluster)
+  int item_cluster;      // most CTAs that may share an attention work item
 };
 
 __host__ __device__ inline size_t unit_of(const DevCtx& c, int seq, int layer) { return (size_t)seq * c.NL + layer; }
@@ -225,6 +229,8 @@ cudaError_t launch_decode_attn(const DevCtx& c, const DecBatch& b, int layer_beg
 
 // a whole decode step in one launch, clusters of `cluster` CTAs (a power of two up to 16) per (sequence, layer, KV head);
 // contexts without collaborative voting.  indexed_end: end of the indexed prefix (the largest of the batch).
+int theta_wide_clusters();                            // clusters of sixteen CTAs of the threshold select that run at once
+bool attn_tc_cluster_runs(const DevCtx& c, int cluster);  // whether that many CTAs can share an attention work item
 int dec_step_capacity(const DevCtx& c, int cluster);  // CTAs that run at once (0: this cluster size is not available)
 bool dec_step_fits(const DevCtx& c, int span_bound, int indexed_end, int cluster);
 cudaError_t launch_dec_step(const DevCtx& c, const DecBatch& b, int layer_begin, int layer_count, const __nv_bfloat16* q,
@@ -262,6 +268,27 @@ inline cudaError_t allow_smem(F* fn, int bytes) {
     bytes -= (int)at.sharedSizeBytes;
   }
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+// Clusters of `cluster` CTAs of `fn` that run at once; 0 when the device, or the part of it this process was given, cannot
+// run one.
+template <typename F>
+inline int active_clusters(F* fn, int cluster, int threads, int smem) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cluster);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
 }
 inline cudaError_t first_error(cudaError_t a, cudaError_t b) { return a != cudaSuccess ? a : b; }
 

@@ -29,6 +29,7 @@ using namespace tc;
 constexpr float kLog2eT = 1.4426950408889634f;
 constexpr int kTcThreads = 576;  // 16 softmax warps + TMA producer + MMA issuer
 constexpr int kMaxItemSplit = 8;  // most CTAs that share a work item
+constexpr int kTcSmem = 65536 + 131072 + 1024;  // queries, two K/V stages, alignment
 constexpr int kNumBoxes = 5;  // box heights 8,16,32,64,128
 constexpr float kRescaleThreshold = 24.0f;
 // Largest exponent (log2 units) a probability may carry above the softmax reference in the regular launch: 2^90 times
@@ -1005,17 +1006,29 @@ bool tc_attention_supported(const DevCtx& c) {
 // CTAs that share a work item: a power of two up to 8 such that all clusters run at once (with one CTA per SM 74, 33 and 15
 // clusters of 2, 4 and 8 fit) and every CTA has at least two of the item's `tiles` (the merge costs some 6K cycles, a tile
 // 3.6K; 36 tiles, 64 items: 86 us a launch with one CTA per item, 57 with two).  The layers counted are those of the whole
-// call, so that a call issued in groups of layers gets the same sums as one issued at once.
+// call, so that a call issued in groups of layers gets the same sums as one issued at once.  The counts are those of a whole
+// GPU and stay what they are on another: the split decides how the sums are rounded.
 static int item_split(const DevCtx& c, const PrefillArgs& a, int tokb, int tiles) {
   const int nitems = ((a.n + tokb - 1) / tokb) * c.Hkv * a.call_layers;
   int sp = 1;
   if (nitems <= 74 && tiles >= 4) sp = 2;
   if (nitems <= 33 && tiles >= 8) sp = 4;
   if (nitems <= 15 && tiles >= 16) sp = 8;
-  return sp;
+  return min(sp, c.item_cluster);
 }
 
-constexpr int kTcSmem = 65536 + 131072 + 1024;  // queries, two K/V stages, alignment
+bool attn_tc_cluster_runs(const DevCtx& c, int cluster) {
+  auto runs = [&](auto local, auto merging) {
+    return active_clusters(local, cluster, kTcThreads, kTcSmem) > 0 && active_clusters(merging, cluster, kTcThreads, kTcSmem) > 0;
+  };
+  switch (c.G) {
+    case 1: return runs(k_attn_tc<1, false, false, true>, k_attn_tc<1, false, true, true>);
+    case 2: return runs(k_attn_tc<2, false, false, true>, k_attn_tc<2, false, true, true>);
+    case 4: return runs(k_attn_tc<4, false, false, true>, k_attn_tc<4, false, true, true>);
+    case 8: return runs(k_attn_tc<8, false, false, true>, k_attn_tc<8, false, true, true>);
+  }
+  return false;
+}
 
 template <int G>
 static cudaError_t prepare_tc_g() {
@@ -1056,20 +1069,14 @@ static cudaError_t launch_tc_g(const DevCtx& c, const PrefillArgs& a, int phase,
   }
   constexpr int TOKB = 256 / G;
   const long long v_off = phase == 0 ? (long long)c.NS * c.NL * c.Hkv * c.SR : (long long)c.NL * c.Hkv * c.Rcap;
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 148;
-  }
-  int ctas = sms;
+  int ctas = c.sms;
   // testing aid: fewer CTAs make every CTA walk several work items even on small problems
-  if (const char* cap = getenv("LTRI_TC_MAX_CTAS")) ctas = max(1, min(sms, atoi(cap)));
+  if (const char* cap = getenv("LTRI_TC_MAX_CTAS")) ctas = max(1, min(c.sms, atoi(cap)));
   // persistent CTAs: one per SM (the kernel needs the whole TMEM and most of the shared memory of an SM)
   const int nitems = ((a.n + TOKB - 1) / TOKB) * c.Hkv * a.layer_count;
   // the regular launch, then the one that redoes the work of the CTAs that asked for it (they return at once otherwise)
   const int tiles = phase == 0 ? (a.sink_end + 127) / 128 + (a.t0 - a.loc_begin + a.n + 127) / 128 : a.ret_tiles;
-  const int sp = phase == 1 || ctas < sms ? 1 : item_split(c, a, TOKB, tiles);
+  const int sp = phase == 1 || ctas < c.sms ? 1 : item_split(c, a, TOKB, tiles);
   const int grid = sp > 1 ? nitems * sp : min(nitems, ctas);
   if (grid > kTcMaxCtas) return cudaErrorInvalidValue;
   auto launch = [&](auto fn) {

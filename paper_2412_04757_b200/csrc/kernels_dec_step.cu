@@ -640,24 +640,7 @@ cudaError_t prepare_dec_step(const DevCtx& c) {
 
 // CTAs of k_dec_step that fit the GPU at once as clusters of `cluster` CTAs (after prepare_dec_step).
 int dec_step_capacity(const DevCtx& c, int cluster) {
-  const DecStepFn fn = dec_step_fn(c.G);
-  const int smem = dec_step_smem(kStMaxSlots);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cluster, c.Hkv, 1);
-  cfg.blockDim = dim3(kStThreads);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cluster;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return n * cluster;
+  return cluster * active_clusters(dec_step_fn(c.G), cluster, kStThreads, dec_step_smem(kStMaxSlots));
 }
 
 // order keys a CTA of the cluster needs: its slice of the spans, or two tables of the units of the indexed range

@@ -390,11 +390,11 @@ static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const 
   int kt = kMapKT, qs = 1;
   const int heads = c.Hkv * a.layer_count;
   auto ctas_of = [&](int k, int q) { return ((nloc + k - 1) / k + (ncur + k - 1) / k) * q * heads; };
-  if (ctas_of(kMapKT, 1) <= 3 * 148) {
+  if (ctas_of(kMapKT, 1) <= 3 * c.sms) {
     long long best = -1;
     for (int k = kMapKT; k >= 1; --k)
       for (int q = 1; q <= 8 && q <= nblk; q *= 2) {
-        const long long waves = (ctas_of(k, q) + 147) / 148;
+        const long long waves = (ctas_of(k, q) + c.sms - 1) / c.sms;
         const long long cost = waves * (6 + k * ((nblk + q - 1) / q));
         if (best < 0 || cost < best) {
           best = cost;

@@ -193,7 +193,7 @@ cudaError_t launch_score_prefill_tc(const DevCtx& c, const PrefillArgs& a, int s
   const int tiles = (span_bound + 127) / 128;
   // A CTA amortises the split of the representatives over several index tiles, but no more of them than leave a CTA for
   // every slot of the GPU (one layer, 12 tiles: 16 CTAs of 8 tiles took 9 us, 96 CTAs of one tile take 5).
-  const int slots = 148 * (two ? 2 : 1);
+  const int slots = c.sms * (two ? 2 : 1);
   const int per_cta = max(1, min(tiles >= 256 ? 32 : (tiles >= 48 ? 16 : 8), (tiles * c.Hkv * a.layer_count + slots - 1) / slots));
   const int gx = (tiles + per_cta - 1) / per_cta;
   const dim3 grid(gx > 0 ? gx : 1, c.Hkv, a.layer_count);

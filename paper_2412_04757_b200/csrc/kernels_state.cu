@@ -3,6 +3,8 @@
 // top-k selection (Eq. 8).  All segmentation arithmetic is integer and order-independent.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "select_util.cuh"
 
@@ -937,9 +939,14 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   }
 }
 
-constexpr int kSegWideLayers = 7;    // clusters of 16 that run at once
+constexpr int kSegWideLayers = 7;    // most layers that get a cluster of 16 (as many run at once on a whole GPU)
 constexpr int kThetaWideSmem = 32 * kThetaBins * (int)sizeof(unsigned);  // a histogram per warp
 constexpr int kSegShareLayers = 16;  // up to here four CTAs share a layer's representatives
+
+int theta_wide_clusters() {
+  return std::min({kSegWideLayers, active_clusters(k_theta_select<17>, 16, 1024, kThetaWideSmem),
+                   active_clusters(k_theta_select<33>, 16, 1024, kThetaWideSmem)});
+}
 
 cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start,
                              int slot, int theta_mode, float theta, long long theta_q_abs, int max_spans, int n,
@@ -950,8 +957,8 @@ cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_
     if (rank < 0) rank = 0;
     if (rank > N - 1) rank = N - 1;
     // Few layers: 16 CTAs of 1024 threads share one, which gives every pair of rows a warp of its own (a cluster of 16
-    // needs a GPC to itself, so seven run at once).  More: 8 CTAs of 512 threads.
-    if (layer_count <= kSegWideLayers) {
+    // needs a GPC to itself, so seven run at once).  More, or no GPC to be had: 8 CTAs of 512 threads.
+    if (layer_count <= c.theta_wide) {
       auto fn = m <= 512 ? k_theta_select<17> : k_theta_select<33>;
       launch_chained_cluster(fn, dim3(layer_count * 16), dim3(1024), 16, kThetaWideSmem, s, c, layer_begin, m, rank, tables ? 1 : 0);
     } else {
@@ -1959,10 +1966,10 @@ static cudaError_t launch_topk(const DevCtx& c, int seq, int layer_begin, const 
   if (!DECODE && !c.host_kv && !c.vote) {
     // Few (layer, KV head) pairs: several CTAs repeat the selection (it costs them nothing: the GPU is idle) and share the
     // packing, which one CTA of 512 threads alone does at some 60 GB/s (one layer, 512 tokens a KV head: 33 us).
-    parts = max(1, min(16, 148 / (c.Hkv * gy)));
+    parts = max(1, min(16, c.sms / (c.Hkv * gy)));
     // With a CTA per SM to spare the scores are read once into shared memory: any number of them that fits, in short
     // loops (unrolled over 24 registers per thread, the select is 12 KB of instructions that a lone launch fetches cold)
-    if (c.unit == 0 && span_bound <= kTopkStage && c.Hkv * gy <= 148) {
+    if (c.unit == 0 && span_bound <= kTopkStage && c.Hkv * gy <= c.sms) {
       stage = span_bound;
       smem = stage * (int)sizeof(unsigned);
     }

@@ -238,7 +238,6 @@ struct ltri_ctx {
   std::vector<int> ret_head;   // [n_layers] copy of the caller's retrieval heads (empty: none)
   std::vector<float> head_w;
   int last_cuda = 0;
-  int sm_count = 148;
   bool use_tc = false;     // tcgen05/TMEM/TMA attention kernels (default when available)
   int dec_fused = -1;      // decode retrieval in one launch: -1 auto, 0 never, 1 whenever the index fits, 2 cluster kernel
   int step_cap[5] = {0, 0, 0, 0, 0};  // one-launch decode step: CTAs that run at once as clusters of 1 << i
@@ -428,10 +427,11 @@ int ltri_create(const ltri_params* p, void* cuda_stream, ltri_ctx** out) {
     if (std::atoi(f) != 0) ctx->ret_phase = 1;
   ctx->st.resize((size_t)p->max_seqs * p->n_layers);
   for (auto& s : ctx->st) s.E = p->n_sink;
-  int dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess) {
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) ctx->sm_count = sms;
+  {
+    int dev = 0, sms = 0;
+    const bool known = cudaGetDevice(&dev) == cudaSuccess &&
+                       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0;
+    ctx->d.sms = known ? sms : 148;
   }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const char* impl = std::getenv("LTRI_ATTN_IMPL");  // "mma" selects the warp-MMA kernels (debugging aid)
@@ -445,8 +445,15 @@ int ltri_create(const ltri_params* p, void* cuda_stream, ltri_ctx** out) {
   // whatever the index size (any of them keeps the one-launch step out)
   if (const char* f = std::getenv("LTRI_DEC_FUSED")) ctx->dec_fused = std::max(0, std::min(2, std::atoi(f)));
   if (const char* f = std::getenv("LTRI_DEC_CLUSTER")) ctx->step_cluster = std::atoi(f);
+  // Clusters are used up to the size that the device can run.  (Testing aid: LTRI_MAX_CLUSTER, the largest size to count on.)
+  const char* mc = std::getenv("LTRI_MAX_CLUSTER");
+  const int most = mc ? std::atoi(mc) : 16;
   if (ctx->dec_fused < 0 && !ctx->d.vote)
-    for (int i = 1; i < 5; ++i) ctx->step_cap[i] = dec_step_capacity(ctx->d, 1 << i);
+    for (int i = 1; i < 5 && 1 << i <= most; ++i) ctx->step_cap[i] = dec_step_capacity(ctx->d, 1 << i);
+  ctx->d.theta_wide = most >= 16 ? theta_wide_clusters() : 0;
+  ctx->d.item_cluster = 1;
+  if (ctx->use_tc)
+    for (int cl = 2; cl <= std::min(8, most) && attn_tc_cluster_runs(ctx->d, cl); cl *= 2) ctx->d.item_cluster = cl;
   // unfilled tile slots and over-fetched rows must hold finite values: start from an all-zero cache
   const size_t kv_bytes = (size_t)p->max_seqs * p->n_layers * ctx->d.Hkv * (size_t)ctx->d.SR * kD * 2 * sizeof(__nv_bfloat16);
   // (paged decode numbers K rows from the start of the K slabs through the unit caches in 31 bits)
@@ -991,7 +998,7 @@ int ltri_decode_step(ltri_ctx* ctx, const int32_t* seq_ids, int n_seqs, int laye
     {
       const LayerState& s0 = ctx->at(seq_ids[i0], layer_begin);
       const long long known = d.Ls + (s0.t + 1 - s0.E);
-      const int wave = 3 * ctx->sm_count;
+      const int wave = 3 * ctx->d.sms;
       const int max_split = (int)std::max<long long>(1, std::min<long long>(kMaxDecSplit, known / 512));
       double best = -1.0;
       for (int ns = 1; ns <= max_split; ++ns) {
@@ -1010,7 +1017,7 @@ int ltri_decode_step(ltri_ctx* ctx, const int32_t* seq_ids, int n_seqs, int laye
     const bool one_cta = ub <= 12288;
     // (unit-granular retrieval ranks units, which only the two-launch path does)
     const bool fused = d.unit == 0 && ub <= dec_retrieve_fused_max_spans() &&
-                       (ctx->dec_fused >= 1 || (ctx->dec_fused < 0 && (!one_cta || units >= ctx->sm_count)));
+                       (ctx->dec_fused >= 1 || (ctx->dec_fused < 0 && (!one_cta || units >= ctx->d.sms)));
     if (!fused) {
       Scope sc(ctx, st, LTRI_K_APPEND, 1);
       LTRI_CUDA(ctx, launch_append_decode(d, b, layer_begin, layer_count, n_seqs, kb, vb, st));
@@ -1020,7 +1027,7 @@ int ltri_decode_step(ltri_ctx* ctx, const int32_t* seq_ids, int n_seqs, int laye
       Scope sc(ctx, st, LTRI_K_DEC_RETRIEVE, 1);
       // CTA size of the one-CTA kernel: 1024 threads fit once per SM, 512 twice; with more CTAs than SMs the smaller
       // size keeps all of them resident instead of running a second, partly empty wave
-      const int ret_threads = units > ctx->sm_count ? 512 : 1024;
+      const int ret_threads = units > ctx->d.sms ? 512 : 1024;
       LTRI_CUDA(ctx, launch_dec_retrieve_fused(d, b, layer_begin, layer_count, qb, kb, vb, (int)ub, ctx->dec_fused == 2,
                                                ret_threads, st));
     } else {

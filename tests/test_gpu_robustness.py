@@ -311,3 +311,37 @@ def test_retrieved_attention_merge_equals_the_continuation(monkeypatch):
     assert worst <= 2e-2
     a.close()
     b.close()
+
+
+def test_a_device_that_cannot_run_large_clusters(monkeypatch):
+    # On a part of a GPU, clusters of sixteen CTAs, or any, may not be available.  Counting on at most eight, the threshold
+    # comes from the kernel of smaller clusters: the same integers, so every output of a prefill call is the same.  Without
+    # clusters no attention item is shared and a decode step is several launches.
+    cfg = small_cfg(n_layers=2, context=1500, window=500, decode_steps=2)   # items shared by two, then four CTAs
+    st = inputs.SyntheticStream(cfg)
+    lts = {}
+    for limit in ("16", "8", "1"):
+        monkeypatch.setenv("LTRI_MAX_CLUSTER", limit)
+        lts[limit] = binding.Ltri(ph.params_of(cfg))
+    whole = binding.Ltri(ph.params_of(cfg))
+    shared = False
+    for t0, n in st.prefill_chunks():
+        q, k, v = (x.cuda() for x in st.tokens(t0, n))
+        out = {limit: lt.ltri_prefill_chunk(0, 0, 2, q, k, v) for limit, lt in lts.items()}
+        monkeypatch.setenv("LTRI_TC_MAX_CTAS", "147")    # (a testing aid that keeps items from being shared)
+        ref = whole.ltri_prefill_chunk(0, 0, 2, q, k, v)
+        monkeypatch.delenv("LTRI_TC_MAX_CTAS")
+        assert torch.equal(out["16"], out["8"]) and torch.equal(out["1"], ref)
+        shared |= not torch.equal(out["16"], out["1"])
+    assert shared
+    for layer in range(2):
+        assert lts["16"].ltri_get_spans(0, layer).tolist() == lts["8"].ltri_get_spans(0, layer).tolist()
+    steps = {}
+    for limit, lt in lts.items():
+        before = lt.ltri_launch_count()
+        lt.ltri_decode_step([0], 0, 2, *(x.cuda() for x in _decode_inputs(st, cfg.context)))
+        steps[limit] = lt.ltri_launch_count() - before
+        assert lt.ltri_sync_status() == 0
+        lt.close()
+    assert steps["16"] == steps["8"] == 1 and steps["1"] > 1
+    whole.close()
