@@ -293,7 +293,7 @@ inline int active_clusters(F* fn, int cluster, int threads, int smem) {
 inline cudaError_t first_error(cudaError_t a, cudaError_t b) { return a != cudaSuccess ? a : b; }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chained_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem,
+[[nodiscard]] inline cudaError_t launch_chained_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem,
                                           cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -311,7 +311,7 @@ inline cudaError_t launch_chained_cluster(void (*kernel)(KArgs...), dim3 grid, d
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+[[nodiscard]] inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                   Args&&... args) {
   return launch_chained_cluster(kernel, grid, block, 1, smem, s, static_cast<Args&&>(args)...);
 }

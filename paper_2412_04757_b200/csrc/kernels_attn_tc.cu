@@ -1083,12 +1083,9 @@ static cudaError_t launch_tc_g(const DevCtx& c, const PrefillArgs& a, int phase,
     return launch_chained_cluster(fn, dim3(grid), dim3(kTcThreads), sp, kTcSmem, s, c, a, phase, final_out ? 1 : 0, c.tc_redo,
                                   maps, v_off);
   };
-  if (sp > 1) {
-    launch(k_attn_tc<G, false, MERGE, true>);
-    return launch(k_attn_tc<G, true, MERGE, true>);
-  }
-  launch(k_attn_tc<G, false, MERGE, false>);
-  return launch(k_attn_tc<G, true, MERGE, false>);
+  const cudaError_t e = sp > 1 ? launch(k_attn_tc<G, false, MERGE, true>) : launch(k_attn_tc<G, false, MERGE, false>);
+  if (e != cudaSuccess) return e;
+  return sp > 1 ? launch(k_attn_tc<G, true, MERGE, true>) : launch(k_attn_tc<G, true, MERGE, false>);
 }
 
 cudaError_t launch_attn_prefill_tc(const DevCtx& c, const PrefillArgs& a, int phase, bool final_out,

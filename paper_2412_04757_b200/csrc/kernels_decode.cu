@@ -189,8 +189,9 @@ cudaError_t prepare_decode(const DevCtx& c) {
 template <int G>
 static cudaError_t launch_dec_g(const DevCtx& c, const DecBatch& b, int layer_begin, int layer_count,
                                 const __nv_bfloat16* q, __nv_bfloat16* out, int nsplit, cudaStream_t s) {
-  launch_chained(k_decode_attn<G>, dim3(nsplit, c.Hkv, b.n * layer_count), dim3(kDecThreads), kDecSmem, s, c, b, layer_begin,
-                 layer_count, q, nsplit);
+  const cudaError_t e = launch_chained(k_decode_attn<G>, dim3(nsplit, c.Hkv, b.n * layer_count), dim3(kDecThreads), kDecSmem,
+                                       s, c, b, layer_begin, layer_count, q, nsplit);
+  if (e != cudaSuccess) return e;
   return launch_chained(k_decode_merge, dim3(c.Hq, b.n * layer_count), dim3(kD), 0, s, c, b, layer_begin, layer_count, out,
                         nsplit);
 }

@@ -951,6 +951,7 @@ int theta_wide_clusters() {
 cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start,
                              int slot, int theta_mode, float theta, long long theta_q_abs, int max_spans, int n,
                              int t0, const __nv_bfloat16* q, cudaStream_t s, bool tables, int seg_unit) {
+  cudaError_t e;
   if (theta_mode == 1) {
     const long long N = (long long)m * (m + 1) / 2;
     long long rank = (long long)floor((double)theta * (double)(N - 1));
@@ -960,33 +961,28 @@ cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_
     // needs a GPC to itself, so seven run at once).  More, or no GPC to be had: 8 CTAs of 512 threads.
     if (layer_count <= c.theta_wide) {
       auto fn = m <= 512 ? k_theta_select<17> : k_theta_select<33>;
-      launch_chained_cluster(fn, dim3(layer_count * 16), dim3(1024), 16, kThetaWideSmem, s, c, layer_begin, m, rank, tables ? 1 : 0);
+      e = launch_chained_cluster(fn, dim3(layer_count * 16), dim3(1024), 16, kThetaWideSmem, s, c, layer_begin, m, rank,
+                                 tables ? 1 : 0);
     } else {
       const int hsmem = (kThetaThreads / 32) * kThetaBins * (int)sizeof(unsigned);
-      launch_chained_cluster(k_theta_select<0>, dim3(layer_count * 8), dim3(kThetaThreads), 8, hsmem, s, c, layer_begin, m,
-                             rank, tables ? 1 : 0);
+      e = launch_chained_cluster(k_theta_select<0>, dim3(layer_count * 8), dim3(kThetaThreads), 8, hsmem, s, c, layer_begin,
+                                 m, rank, tables ? 1 : 0);
     }
   } else {
-    launch_chained(k_theta_set, dim3(layer_count), dim3(1), 0, s, c, layer_begin, theta_q_abs,
-                   (long long)nearbyint((double)theta * (double)kQScale), tables ? 1 : 0);
+    e = launch_chained(k_theta_set, dim3(layer_count), dim3(1), 0, s, c, layer_begin, theta_q_abs,
+                       (long long)nearbyint((double)theta * (double)kQScale), tables ? 1 : 0);
   }
-  const dim3 rows((m + 7) / 8, layer_count);
-  if (m <= 256)
-    launch_chained(k_seg_rowscan<2>, rows, dim3(256), 0, s, c, layer_begin, m);
-  else if (m <= 512)
-    launch_chained(k_seg_rowscan<4>, rows, dim3(256), 0, s, c, layer_begin, m);
-  else
-    launch_chained(k_seg_rowscan<8>, rows, dim3(256), 0, s, c, layer_begin, m);
-  if (m <= 512)
-    launch_chained(k_seg_colscan<32>, dim3((m + 31) / 32, layer_count), dim3(1024),
-                   (size_t)(32 * 33 + m + 32) * sizeof(long long), s, c, layer_begin, m, seg_unit, reg_start);
-  else
-    launch_chained(k_seg_colscan<16>, dim3((m + 15) / 16, layer_count), dim3(1024),
-                   (size_t)(64 * 17 + m + 16) * sizeof(long long), s, c, layer_begin, m, seg_unit, reg_start);
+  if (e != cudaSuccess) return e;
+  e = launch_chained(m <= 256 ? k_seg_rowscan<2> : m <= 512 ? k_seg_rowscan<4> : k_seg_rowscan<8>,
+                     dim3((m + 7) / 8, layer_count), dim3(256), 0, s, c, layer_begin, m);
+  if (e != cudaSuccess) return e;
+  const int cx = m <= 512 ? 32 : 16;  // columns per CTA; 1024 / cx row groups
+  e = launch_chained(m <= 512 ? k_seg_colscan<32> : k_seg_colscan<16>, dim3((m + cx - 1) / cx, layer_count), dim3(1024),
+                     (size_t)(1024 / cx * (cx + 1) + m + cx) * sizeof(long long), s, c, layer_begin, m, seg_unit, reg_start);
+  if (e != cudaSuccess) return e;
   NmsArgs a{seq, layer_begin, m, reg_start, slot, max_spans, n, t0, q, tables ? 1 : 0, seg_unit};
   const int cl = q && layer_count <= kSegShareLayers ? 4 : 1;
-  launch_chained_cluster(k_seg_nms, dim3(layer_count * cl), dim3(1024), cl, 0, s, c, a);
-  return cudaGetLastError();
+  return launch_chained_cluster(k_seg_nms, dim3(layer_count * cl), dim3(1024), cl, 0, s, c, a);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1974,12 +1970,13 @@ static cudaError_t launch_topk(const DevCtx& c, int seq, int layer_begin, const 
       smem = stage * (int)sizeof(unsigned);
     }
   }
-  if (c.vote)
-    launch_chained(k_topk<DECODE>, dim3(c.Hkv, gy), dim3(512), smem, s, c, seq, layer_begin, b, layer_count, evicted_end,
-                   (int)kTopkBallot, 1, 0);
-  launch_chained(k_topk<DECODE>, dim3(c.Hkv * parts, gy), dim3(512), smem, s, c, seq, layer_begin, b, layer_count,
-                 evicted_end, (int)(c.vote ? kTopkVote : kTopkSelect), parts, stage);
-  return cudaGetLastError();
+  if (c.vote) {
+    const cudaError_t e = launch_chained(k_topk<DECODE>, dim3(c.Hkv, gy), dim3(512), smem, s, c, seq, layer_begin, b,
+                                         layer_count, evicted_end, (int)kTopkBallot, 1, 0);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_chained(k_topk<DECODE>, dim3(c.Hkv * parts, gy), dim3(512), smem, s, c, seq, layer_begin, b, layer_count,
+                        evicted_end, (int)(c.vote ? kTopkVote : kTopkSelect), parts, stage);
 }
 
 cudaError_t launch_topk_prefill(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s) {

@@ -1,7 +1,9 @@
 """Function attributes (a kernel's limit of dynamic shared memory) belong to the device, not to a context.  A launch that set
 one to the size of its own call could lower it under the larger launch that another context's thread is about to make, which
 is then refused half-way through a call.  The window between the two is too narrow to be hit on demand, so the rule itself
-is checked: attributes are set by the prepare functions, which ltri_create runs, and nowhere else."""
+is checked: attributes are set by the prepare functions, which ltri_create runs, and nowhere else.
+
+In the same way a refused launch has to end its call where it happens: nothing on a GPU refuses one on demand."""
 import glob
 import os
 import re
@@ -33,3 +35,10 @@ def test_every_prepare_function_runs_at_creation():
     assert len(body) == 1 and parts and all(p + "(" in body[0] for p in parts)
     create = [f.group(0) for f in FUNCTION.finditer(text["ltri_api.cu"]) if f.group(1) == "ltri_create"]
     assert len(create) == 1 and "prepare_kernels(ctx->d" in create[0]
+
+
+@pytest.mark.parametrize("name", FILES)
+def test_the_result_of_every_launch_is_looked_at(name):
+    # a statement that begins with the launch drops its result, and the kernels behind it run on what it did not write
+    text = open(os.path.join(CSRC, name)).read()
+    assert not re.search(r"(^|[;{}]|\)|\belse)\s*\n\s*launch(_chained(_cluster)?)?\(", text), name
