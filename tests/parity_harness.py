@@ -45,6 +45,7 @@ class Report:
     vote_changes: int = 0   # selections that the ballots of other layers changed (collaborative voting)
     cache_hits: int = 0     # host-memory pager: units found in / fetched into the unit caches (last checked layer)
     cache_misses: int = 0
+    step_launches: set = dataclasses.field(default_factory=set)   # kernels launched per decode step
 
 
 def params_of(cfg: inputs.StreamConfig, max_seqs=None) -> binding.LtriParams:
@@ -349,7 +350,9 @@ class StreamPair:
         """q [n_seqs][L][Hq][d], k, v [n_seqs][L][Hkv][d] bf16 on the CPU."""
         cfg, lt, rep = self.cfg, self.lt, self.rep
         L = cfg.n_layers
+        launched = lt.ltri_launch_count()
         out = lt.ltri_decode_step(seq_ids, 0, L, q.to(self.dev), k.to(self.dev), v.to(self.dev))
+        rep.step_launches.add(lt.ltri_launch_count() - launched)
         torch.cuda.synchronize(self.dev)
         assert lt.ltri_sync_status() == 0
         rep.calls += 1

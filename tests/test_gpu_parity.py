@@ -19,6 +19,19 @@ def small_cfg(**kw):
     return inputs.StreamConfig(**base)
 
 
+# decode steps of small workloads: one launch, or the separate launches that larger steps take
+ROUTES = pytest.mark.parametrize("fused", [None, "0"], ids=["one_launch", "separate"])
+
+
+def set_route(monkeypatch, fused):
+    if fused is not None:
+        monkeypatch.setenv("LTRI_DEC_FUSED", fused)
+
+
+def check_route(rep, fused):
+    assert (rep.step_launches == {1}) if fused is None else (min(rep.step_launches) > 1), rep.step_launches
+
+
 def test_cfg0_full_stream_and_decode():
     cfg = inputs.config(0)
     rep = ph.run_stream(cfg, layers=[0])
@@ -81,23 +94,29 @@ def test_maximum_sizes():
     print(rep)
 
 
+@ROUTES
 @pytest.mark.parametrize("U,persist", [(64, False), (128, False), (40, True)])
-def test_unit_granular_retrieval(U, persist):
+def test_unit_granular_retrieval(U, persist, fused, monkeypatch):
     # Eq. 8 as printed: fixed units of U tokens ranked by the maximum over their spans and fetched whole; unit
     # selections, the token count of every decode step and the outputs are checked against the oracle
+    set_route(monkeypatch, fused)
     cfg = small_cfg(n_layers=2, context=1536, decode_steps=4, unit_tokens=U, persist_decode=persist, top_k=3)
     rep = ph.run_stream(cfg, layers=[0, 1])
     assert rep.sel_checks > 20
+    check_route(rep, fused)
     print(rep)
 
 
+@ROUTES
 @pytest.mark.parametrize("phi_milli,U", [(300, 0), (500, 0), (300, 64)])
-def test_overlapping_spans_from_nms_with_iou_threshold(phi_milli, U):
+def test_overlapping_spans_from_nms_with_iou_threshold(phi_milli, U, fused, monkeypatch):
     # NMS with an IoU threshold above zero: spans overlap, selected overlapping spans are attended once per token
+    set_route(monkeypatch, fused)
     cfg = small_cfg(n_layers=2, context=1536, decode_steps=4, nms_iou_milli=phi_milli, unit_tokens=U, top_k=6,
                     max_spans_per_region=8)
     rep = ph.run_stream(cfg, layers=[0, 1])
     assert rep.sel_checks > 20
+    check_route(rep, fused)
     print(rep)
 
 
@@ -154,31 +173,36 @@ def test_segmentation_per_memory_unit(U, C, chunk, phi):
     print(rep)
 
 
+@ROUTES
 @pytest.mark.parametrize("cache_units,decay,extra", [
     (4, 0.1, dict(unit_tokens=48, window=256)), (9, 0.5, dict(segment_per_unit=True, max_spans_per_region=3, persist_decode=True)),
     (6, 1.0, dict(retrieval_head=(2, -1), retrieval_head_score=(0.5, 0.0), collab_vote=True)),
 ])
-def test_host_memory_pager(cache_units, decay, extra):
+def test_host_memory_pager(cache_units, decay, extra, fused, monkeypatch):
     # Sec. 3.4: evicted rows are mirrored in host memory, the retrieved units of a prefill call come from a unit
     # cache in device memory or, when missing, over the bus from the mirror; decode steps read their units from the
     # cache slots as well (with the persistent mechanism: both sets).  The harness checks the usual parity and, after
     # every call and step, the cache's tags, usage scores and hit/miss counters against the policy model.  The context
     # length leaves the last unit of the indexed range partial.
+    set_route(monkeypatch, fused)
     kw = dict(n_layers=2, context=2048 - 40, decode_steps=6, unit_tokens=64, top_k=4, host_kv=True,
               cache_units=cache_units, score_decay=decay)
     kw.update(extra)    # (units of 48 tokens with a window of 256: the indexed range ends inside a unit during decode)
     cfg = small_cfg(**kw)
     rep = ph.run_stream(cfg, layers=[0, 1])
     assert rep.cache_misses > 10 and rep.cache_hits > 10
+    check_route(rep, "0" if "collab_vote" in extra else fused)   # (votes are counted by separate launches only)
     print(rep)
 
 
+@ROUTES
 @pytest.mark.parametrize("groups", ["1", "2"])
-def test_host_memory_pager_is_bit_identical_to_the_resident_path(groups, monkeypatch):
+def test_host_memory_pager_is_bit_identical_to_the_resident_path(groups, fused, monkeypatch):
     # the same stream through a paged and a resident context: every output bit and every selection equal, also
     # with irregular call sizes (units that are still growing bypass the cache) and after a sequence reset; the
     # paged call issued as one group of layers or as two whose pulls run under the other group's kernels
     monkeypatch.setenv("LTRI_PAGER_GROUPS", groups)
+    set_route(monkeypatch, fused)
     cfg = small_cfg(n_layers=2, context=1800, decode_steps=4, unit_tokens=48, top_k=5)
     paged = dataclasses.replace(cfg, host_kv=True, cache_units=7, score_decay=0.1)
     st = inputs.SyntheticStream(cfg)
@@ -208,10 +232,12 @@ def test_host_memory_pager_is_bit_identical_to_the_resident_path(groups, monkeyp
     b.close()
 
 
-def test_sliding_slabs_through_long_decode_and_their_capacity():
+@ROUTES
+def test_sliding_slabs_through_long_decode_and_their_capacity(fused, monkeypatch):
     # a paged context holds sink + window in device memory (2 x (window + 2 chunks) + slack rows): a long decode
     # slides the slabs once more, stays bit-identical to the resident path, and ends with a capacity error -- not a
     # fault -- when the tokens since the last eviction no longer fit
+    set_route(monkeypatch, fused)
     cfg = small_cfg(n_layers=1, context=640, chunk=64, window=128, n_sink=16, decode_steps=900, unit_tokens=32, top_k=3,
                     max_spans_per_region=2)
     paged = dataclasses.replace(cfg, host_kv=True, cache_units=4, score_decay=0.1)
@@ -301,10 +327,12 @@ def test_irregular_call_sizes_and_single_token_calls():
     print(sp.rep)
 
 
+@ROUTES
 @pytest.mark.parametrize("paged", [False, True])
-def test_batched_decode_independent_sequences(paged):
+def test_batched_decode_independent_sequences(paged, fused, monkeypatch):
     # paged: every sequence has its own unit caches and its own sliding slabs (sequence 0 is long enough to slide once,
     # the others are not), and a batched decode step carries one row shift per sequence
+    set_route(monkeypatch, fused)
     kw = dict(unit_tokens=32, host_kv=True, cache_units=5, window=128, chunk=64, context=1024) if paged else {}
     cfg = small_cfg(**{**dict(n_layers=2, n_seqs=3, context=768, decode_steps=4), **kw})
     sp = ph.StreamPair(cfg, layers=[0, 1], seqs=[0, 1, 2])
@@ -327,6 +355,7 @@ def test_batched_decode_independent_sequences(paged):
         order = [2, 0, 1] if step % 2 else [0, 1, 2]
         sp.decode(order, torch.stack([qs[i] for i in order]), torch.stack([ks[i] for i in order]),
                   torch.stack([vs[i] for i in order]))
+    check_route(sp.rep, fused)
     sp.lt.close()
     print(sp.rep)
 

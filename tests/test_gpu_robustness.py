@@ -146,14 +146,19 @@ def test_retrieval_and_attention_from_a_loaded_span_index(unit_tokens):
     print(sp.rep)
 
 
-@pytest.mark.parametrize("fused", ["0", "1", "2"])
+def _set_decode_path(monkeypatch, path):
+    """"0" to "2": separate launches with one of the retrievers; "c2" to "c16": one launch in clusters of that size."""
+    monkeypatch.setenv(*(("LTRI_DEC_CLUSTER", path[1:]) if path[0] == "c" else ("LTRI_DEC_FUSED", path)))
+
+
+@pytest.mark.parametrize("fused", ["0", "1", "2", "c2", "c4", "c8", "c16"])
 def test_equal_scores_at_the_cut_go_to_the_lower_span(fused, monkeypatch):
     # Eq. 8 with ties: the loaded index holds only three distinct vectors per KV head (span s gets vector s mod 3),
     # so the scores of a call take three values among the loaded spans and the top-k cut falls inside a group of
     # exactly equal scores; the picks among them must be the lowest span ids, in the prefill retriever and in each
-    # of the three decode retrieval paths.  The harness tolerates a different pick among near-equal scores and
+    # of the decode retrieval paths.  The harness tolerates a different pick among near-equal scores and
     # counts it: here the count must stay zero.
-    monkeypatch.setenv("LTRI_DEC_FUSED", fused)
+    _set_decode_path(monkeypatch, fused)
     cfg = small_cfg(n_layers=2, context=1536, decode_steps=3, top_k=5)
     sp = ph.StreamPair(cfg, [0, 1])
     st = inputs.SyntheticStream(cfg)
@@ -184,17 +189,18 @@ def test_equal_scores_at_the_cut_go_to_the_lower_span(fused, monkeypatch):
         sp.decode([0], *_decode_inputs(st, cfg.context + s))
     assert ties_at_cut > 0
     assert sp.rep.sel_checks >= 16 and sp.rep.sel_flips == 0, sp.rep
+    assert (sp.rep.step_launches == {1}) == (fused[0] == "c"), sp.rep
     sp.lt.close()
     print(sp.rep)
 
 
-@pytest.mark.parametrize("fused", ["1", "2"])
+@pytest.mark.parametrize("fused", ["1", "2", "c2", "c16"])
 def test_hundreds_of_equal_scores_fall_back_to_the_radix_passes(fused, monkeypatch):
     # Eq. 8 with a whole index of equal scores: every loaded span gets the same vector, so several hundred scores are
     # exactly equal and the short cut of the select (which ranks at most 256 keys near the maximum against each
     # other) has to hand over to the radix passes and their id-ordered tie pass; picks = the lowest span ids.
-    # (both one-launch decode retrievers: one CTA per KV head, and the cluster of eight)
-    monkeypatch.setenv("LTRI_DEC_FUSED", fused)
+    # (both one-launch decode retrievers, one CTA per KV head and the cluster of eight, and the one-launch step)
+    _set_decode_path(monkeypatch, fused)
     cfg = small_cfg(n_layers=1, context=12288, decode_steps=2, top_k=6, max_spans_per_region=8, seg_min=8, seg_max=24)
     sp = ph.StreamPair(cfg, [0], deep=False)
     st = inputs.SyntheticStream(cfg)
@@ -216,6 +222,7 @@ def test_hundreds_of_equal_scores_fall_back_to_the_radix_passes(fused, monkeypat
     for s in range(cfg.decode_steps):
         sp.decode([0], *_decode_inputs(st, cfg.context + s))
     assert sp.rep.sel_flips == 0, sp.rep
+    assert (sp.rep.step_launches == {1}) == (fused[0] == "c"), sp.rep
     sel = sp.lt.ltri_get_selected(0, 0)
     assert sel.shape[1] == cfg.top_k
     sp.lt.close()
