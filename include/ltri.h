@@ -202,7 +202,14 @@ int ltri_reset_sequence(ltri_ctx* ctx, int seq, void* cuda_stream);
  * (Eq. 7-8); attention runs over [sink | selected spans | local | current (causal)].
  * Each (sequence, layer) is its own stream: its tokens must arrive in order, and a layer
  * that already decoded cannot prefill again (LTRI_ESTATE).  The layers of one call must
- * all be at the same position. */
+ * all be at the same position.
+ * Rounding: the same calls give the same bits, but a layer's bits may depend on how many
+ * layers share its call.  A call of few work items (256 (token, head) rows of one KV head
+ * and layer; at most 74) lets several CTAs share an item's keys and merges their partial
+ * softmaxes, a call of more does not, so outputs and row statistics are rounded in another
+ * order.  Where two candidates agree to that rounding, spans and selections can differ too.
+ * A decode step's sums are likewise divided by the (sequence, layer, KV head) units of the
+ * step. */
 int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count, int n_tokens, const void* q,
                        const void* k, const void* v, void* out, void* cuda_stream);
 

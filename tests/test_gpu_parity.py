@@ -270,7 +270,8 @@ def test_sliding_slabs_through_long_decode_and_their_capacity(fused, monkeypatch
 
 def test_voting_layer_by_layer_calls_match_one_call():
     # a real model submits one layer at a time: the ballots of the earlier layers of the same chunk are read from the
-    # context's state and the selections must equal those of the all-layers call
+    # context's state and the selections must equal those of the all-layers call (the few work items of one and of three
+    # layers are shared by as many CTAs, so the outputs are the same bits)
     cfg = small_cfg(n_layers=3, context=1024, decode_steps=0, unit_tokens=64, top_k=3, retrieval_head=(2, 5, -1),
                     retrieval_head_score=(0.4, 0.6, 0.0), collab_vote=True)
     st = inputs.SyntheticStream(cfg)
@@ -389,6 +390,7 @@ def test_warp_mma_fallback_path(monkeypatch):
 
 
 def test_layer_ranges_are_independent_streams():
+    # (one and two of these layers have four and eight work items with few key tiles: shared alike, so the bits are the same)
     cfg = small_cfg(n_layers=2, context=512, decode_steps=0)
     lt = binding.Ltri(ph.params_of(cfg))
     st = inputs.SyntheticStream(cfg)
@@ -406,6 +408,29 @@ def test_layer_ranges_are_independent_streams():
     for a, b in zip(outs_all, outs_split):
         assert torch.equal(a, b)
     lt.close()
+
+
+def test_layer_groupings_differ_in_rounding_only():
+    # 512-token calls of 32 heads over up to 2048 keys: the 64 work items of one layer are shared by two CTAs each, the 128
+    # of two layers are not.  Calls of the same layers give the same bits, calls of other groupings the same result.
+    cfg = small_cfg(n_layers=2, n_q_heads=32, n_kv_heads=8, context=2048, chunk=512, window=2048, decode_steps=0)
+    st = inputs.SyntheticStream(cfg, device="cuda:0")
+    together, again, apart = (binding.Ltri(ph.params_of(cfg)) for _ in range(3))
+    differ = 0
+    for t0, n in st.prefill_chunks():
+        q, k, v = st.tokens(t0, n)
+        a = together.ltri_prefill_chunk(0, 0, 2, q, k, v)
+        assert torch.equal(a, again.ltri_prefill_chunk(0, 0, 2, q, k, v))
+        b = torch.cat([apart.ltri_prefill_chunk(0, l, 1, q[l:l + 1].contiguous(), k[l:l + 1].contiguous(), v[l:l + 1].contiguous())
+                       for l in range(2)])
+        differ += not torch.equal(a, b)
+        # each is within REL_FRO and MAX_ABS of the exact result
+        d = a.double() - b.double()
+        assert float(d.norm() / a.double().norm()) <= ph.REL_FRO and float(d.abs().max()) <= 2 * ph.MAX_ABS
+    assert differ > 0
+    for lt in (together, again, apart):
+        assert lt.ltri_sync_status() == 0
+        lt.close()
 
 
 def test_state_and_capacity_errors():

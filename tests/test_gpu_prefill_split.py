@@ -3,11 +3,14 @@
 One or two layers of eight query heads on two KV heads are four or eight work items, so the length of the window decides
 how many CTAs share one: four tiles of 128 keys two, eight four, sixteen eight.
 """
+import dataclasses
+
 import pytest
 import torch
 
-from paper_2412_04757_b200 import inputs
+from paper_2412_04757_b200 import binding, inputs
 from tests import parity_harness as ph
+from tests.test_gpu_fullsize import check_call
 from tests.test_gpu_parity import small_cfg
 
 pytestmark = pytest.mark.gpu
@@ -52,4 +55,24 @@ def test_calls_of_many_layers(n_layers):
     cfg = small_cfg(n_layers=n_layers, context=900, decode_steps=1)
     rep = ph.run_stream(cfg, layers=[0, n_layers - 1])
     assert rep.regions >= 14
+    print(rep)
+
+
+@pytest.mark.parametrize("chunk", [512, 1024])
+def test_one_layer_calls_at_full_size(chunk):
+    # one layer of 32 query heads on 8 KV heads with a window of 4096: the 64 work items of a 512-token call are shared by
+    # two CTAs each, the 128 of a 1024-token call are not
+    cfg = dataclasses.replace(inputs.config(2), n_layers=1, context=8192 + chunk, chunk=chunk, decode_steps=0, needle=False)
+    lt = binding.Ltri(ph.params_of(cfg))
+    st = inputs.SyntheticStream(cfg, device="cuda:0")
+    K, V = [], []
+    rep = ph.Report()
+    for t0, n in st.prefill_chunks():
+        q, k, v = st.tokens(t0, n)
+        out = lt.ltri_prefill_chunk(0, 0, 1, q, k, v)
+        K.append(k[0].cpu())
+        V.append(v[0].cpu())
+    check_call(lt, cfg, 0, 0, t0, torch.cat(K), torch.cat(V), q[0].cpu(), out, rep, [0, 1, n // 2, n - 1], f"call at {t0}")
+    assert lt.ltri_sync_status() == 0
+    lt.close()
     print(rep)
