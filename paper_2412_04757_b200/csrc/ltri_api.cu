@@ -884,12 +884,24 @@ int ltri_host_outputs_ready(ltri_ctx* ctx, void* cuda_stream) {
 // holds no shared memory for tiles and leaves more CTAs per SM to hide the latency, stream it faster (33K spans, 32
 // units: 92 against 103 us a step).
 constexpr int kStepSpans = 2560;
+// Against the three launches that an index beyond one CTA's shared memory takes (kOneCtaSpans), the line is where all units
+// together read kStepRows rows (18K spans and 4.3K known tokens: 32 units, 851K rows, 62.7 us a step in one launch and 60.9
+// in three; 24 units, 639K rows, 52.9 and 56.9).
+constexpr int kOneCtaSpans = 12288;
+constexpr long long kStepRows = 768 * 1024;
 // With unit-granular retrieval a step may attend over thousands of scattered tokens per unit, which the split-KV kernel with
 // three CTAs per SM streams faster than a CTA that keeps one 16-token tile per warp on the way (12.7K tokens per unit, 64
 // units: 124 us a step against 130 us as clusters of four).  Spans are few tokens beside the recent ones, and the recent
 // ones stream well either way (64 units, 3K to 15K recent tokens: 46 to 101 us a step as clusters of four, 59 to 116 us as
 // separate launches).
 constexpr int kStepTokens = 1536;
+// A small index of which every unit is fetched costs the separate launches no selection and leaves them one range of tokens
+// (48 units, clusters of four: 5.7K tokens a unit, 51 us a step in one launch and 45 separately; 4.2K tokens, 39 and 41.  96
+// units, clusters of two: 2.6K tokens 49 and 46, 2.1K tokens 40 and 40.  16 units, clusters of eight: 8.8K tokens 41.5 and
+// 40.0, 6.7K tokens 33 and 33.  8 units, and 32 as clusters of eight, are faster in one launch up to 8.8K tokens.)
+static int step_tokens_all(int cluster, int units) {
+  return cluster <= 4 ? 1088 : cluster == 8 && units < 24 ? 864 : kStepTokens;
+}
 static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, long long ub) {
   const DevCtx& d = ctx->d;
   int e_max = 0;
@@ -901,11 +913,15 @@ static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, 
   // tokens a unit attends over: known ones, and about top_k (with the persistent set twice that) units or mean spans
   const long long item = d.unit > 0 ? d.unit : ub > 0 ? (e_max + ub - 1) / ub * 2 : 0;
   const long long tokens = known + std::min<long long>(e_max, (long long)d.topk * item * (d.persist ? 2 : 1));
+  const bool all = d.unit > 0 && e_max > d.Ls && (e_max - 1) / d.unit - d.Ls / d.unit < d.topk;
+  const bool automatic = ctx->step_cluster == 0;
+  if (automatic && d.unit == 0 && ub > kOneCtaSpans && units * (ub + 2 * known) > kStepRows) return 0;
   for (int i = 4; i >= 1; --i) {
     const int cl = 1 << i;
-    if (ctx->step_cluster > 0 ? cl != ctx->step_cluster : known / cl < 64 && cl > 2) continue;
-    if (ctx->step_cluster == 0 && ((d.unit == 0 && ub > (long long)kStepSpans * cl) || (d.unit > 0 && tokens > kStepTokens * cl))) continue;
-    if ((long long)units * cl <= ctx->step_cap[i] && dec_step_fits(d, (int)ub, e_max, cl)) return cl;
+    if (automatic ? known / cl < 64 && cl > 2 : cl != ctx->step_cluster) continue;
+    if (automatic && (d.unit > 0 ? tokens > kStepTokens * cl : ub > (long long)kStepSpans * cl)) continue;
+    if ((long long)units * cl > ctx->step_cap[i] || !dec_step_fits(d, (int)ub, e_max, cl)) continue;
+    return automatic && all && tokens > step_tokens_all(cl, units) * cl ? 0 : cl;
   }
   return 0;
 }
@@ -1014,7 +1030,7 @@ int ltri_decode_step(ltri_ctx* ctx, const int32_t* seq_ids, int n_seqs, int laye
     // retrieval in one launch with the scores in shared memory: one CTA per (sequence, layer, KV head) when there are
     // enough heads to fill the GPU and the index fits one CTA (12K spans), a cluster of eight CTAs per head for a larger
     // index (up to 98K spans); otherwise the scores go through global memory in two launches
-    const bool one_cta = ub <= 12288;
+    const bool one_cta = ub <= kOneCtaSpans;
     // (unit-granular retrieval ranks units, which only the two-launch path does)
     const bool fused = d.unit == 0 && ub <= dec_retrieve_fused_max_spans() &&
                        (ctx->dec_fused >= 1 || (ctx->dec_fused < 0 && (!one_cta || units >= ctx->d.sms)));

@@ -120,3 +120,78 @@ def test_outputs_written_over_the_inputs(shared, heads, one_launch, monkeypatch)
     assert lt.ltri_sync_status() == 0
     lt.close()
     twin.close()
+
+
+@pytest.mark.parametrize("seqs,context,one_launch", [
+    (6, 4096, True), (6, 5120, False),      # 48 units as clusters of four: 1088 tokens per CTA are the line
+    (12, 1920, True), (12, 2560, False),    # 96 units as clusters of two
+    (2, 6656, True), (2, 7680, False),      # 16 units as clusters of eight: 864 tokens per CTA
+    (4, 7680, True),                        # 32 units as clusters of eight
+])
+def test_route_of_steps_that_fetch_every_unit(seqs, context, one_launch, monkeypatch):
+    # a small index of units, all of them fetched: either route attends over every token
+    cfg = small_cfg(n_layers=1, n_q_heads=16, n_kv_heads=8, context=context, chunk=512, window=512, n_seqs=seqs,
+                    unit_tokens=128, top_k=64, decode_steps=1)
+    st = inputs.SyntheticStream(cfg, device="cuda:0")
+    lts = [binding.Ltri(ph.params_of(cfg))]
+    monkeypatch.setenv("LTRI_DEC_FUSED", "0")
+    lts.append(binding.Ltri(ph.params_of(cfg)))
+    K, V = [], []
+    for t0, n in st.prefill_chunks():
+        q, k, v = st.tokens(t0, n)
+        K.append(k[0])
+        V.append(v[0])
+        for lt in lts:
+            for s in range(seqs):
+                lt.ltri_prefill_chunk(s, 0, 1, q, k, v)
+    q, k, v = (x.permute(1, 0, 2, 3).expand(seqs, -1, -1, -1).contiguous() for x in st.tokens(context, 1, kind=1))
+    K, V = torch.cat(K + [k[0]]).double(), torch.cat(V + [v[0]]).double()
+    p = torch.softmax(torch.einsum("gjd,tgd->gjt", q[0, 0].double().view(8, 2, 128), K) / 128 ** 0.5, dim=-1)
+    want = torch.einsum("gjt,tgd->gjd", p, V).reshape(16, 128).cpu().numpy()
+    rep = ph.Report()
+    for lt, one in zip(lts, (one_launch, False)):
+        before = lt.ltri_launch_count()
+        out = lt.ltri_decode_step(list(range(seqs)), 0, 1, q, k, v)
+        assert (lt.ltri_launch_count() - before == 1) == one
+        for s in range(seqs):
+            ph.check_output(out[s, 0], want, rep, f"sequence {s}")
+        assert lt.ltri_sync_status() == 0
+        lt.close()
+
+
+@pytest.mark.parametrize("seqs,one_launch", [(3, True), (4, False)])
+def test_route_of_steps_over_a_large_index(seqs, one_launch, monkeypatch):
+    # 18K spans and 4.3K known tokens: 24 units read 639K rows, 32 read 851K; the line lies at 768K
+    N, window = 18000, 4096
+    context = (N + window + 300) // 128 * 128
+    cfg = small_cfg(n_layers=1, n_q_heads=16, n_kv_heads=8, context=context, window=window, n_sink=16, n_seqs=seqs,
+                    top_k=32, max_spans_per_region=64, decode_steps=1)
+    lts = [binding.Ltri(ph.params_of(cfg))]
+    monkeypatch.setenv("LTRI_DEC_FUSED", "1")
+    lts.append(binding.Ltri(ph.params_of(cfg)))
+    g = torch.Generator(device="cuda").manual_seed(4)
+    q, k, v = (torch.randn(1, 128, h, 128, generator=g, device="cuda").to(torch.bfloat16) for h in (16, 8, 8))
+    for _ in range(context // 128):
+        for lt in lts:
+            for s in range(seqs):
+                lt.ltri_prefill_chunk(s, 0, 1, q, k, v)
+    E = lts[0].ltri_get_stats(0, 0).evicted_end
+    lens = np.full(N, (E - 16) // N)
+    lens[:(E - 16) % N] += 1
+    spans = np.stack([16 + np.concatenate([[0], np.cumsum(lens)[:-1]]), lens], axis=1).astype(np.int32)
+    idx = torch.randn(8, N, 128, generator=torch.Generator().manual_seed(5)).to(torch.bfloat16)
+    for lt in lts:
+        for s in range(seqs):
+            lt.ltri_debug_load_index(s, 0, E, spans, inputs.bf16_bits(idx))
+    q, k, v = (torch.randn(seqs, 1, h, 128, generator=g, device="cuda").to(torch.bfloat16) for h in (16, 8, 8))
+    outs = []
+    for lt, one in zip(lts, (one_launch, False)):
+        before = lt.ltri_launch_count()
+        outs.append(lt.ltri_decode_step(list(range(seqs)), 0, 1, q, k, v))
+        assert (lt.ltri_launch_count() - before == 1) == one
+        assert lt.ltri_sync_status() == 0
+    for s in range(seqs):
+        assert (lts[0].ltri_get_selected(s, 0) == lts[1].ltri_get_selected(s, 0)).all()
+    assert float((outs[0].float() - outs[1].float()).abs().max()) <= ph.MAX_ABS
+    for lt in lts:
+        lt.close()
