@@ -235,7 +235,7 @@ int ltri_host_outputs_ready(ltri_ctx* ctx, void* cuda_stream);
  *   seq_ids  HOST array [n_seqs] of distinct sequence slots
  *   q   [n_seqs][layer_count][n_q_heads ][head_dim]
  *   k,v [n_seqs][layer_count][n_kv_heads][head_dim]
- *   out [n_seqs][layer_count][n_q_heads ][head_dim]
+ *   out [n_seqs][layer_count][n_q_heads ][head_dim]   (may be q itself)
  * Appends the token, scores the summed query of each KV-head group against the index,
  * selects top-k spans and attends over [sink | selected spans | every token since the
  * last eviction].  Decode never evicts, votes or segments. */

@@ -362,16 +362,17 @@ __device__ inline int select_reps(const long long* __restrict__ votes, int start
           bv = held[k];
           bi = start + k * 32 + lane;
         }
-    } else
-    for (int i = lane; i < len; i += 32) {
-      int tok = start + i;
-      bool used = false;
-      for (int q = 0; q < r; ++q) used |= (toks[q] == tok);
-      if (used) continue;
-      long long v = votes[tok];
-      if (v > bv || (v == bv && tok < bi)) {
-        bv = v;
-        bi = tok;
+    } else {
+      for (int i = lane; i < len; i += 32) {
+        int tok = start + i;
+        bool used = false;
+        for (int q = 0; q < r; ++q) used |= (toks[q] == tok);
+        if (used) continue;
+        long long v = votes[tok];
+        if (v > bv || (v == bv && tok < bi)) {
+          bv = v;
+          bi = tok;
+        }
       }
     }
 #pragma unroll

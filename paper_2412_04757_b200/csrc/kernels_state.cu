@@ -220,7 +220,6 @@ cudaError_t launch_evict_index(const DevCtx& c, const EvictArgs& a, int layer_co
 }
 
 // ------------------------------------------------------------------------------------------
-// ------------------------------------------------------------------------------------------
 // a3 segmenter, step 1: exact rank selection of theta (quantile mode) over the causal entries of Mq.
 // Pass 1 counts negatives (only hand-built maps have any) and zeros (a sparse map is mostly zeros) and builds a
 // log-scale histogram of the positive entries: bin = (position of the leading one, next four bits), which is monotone

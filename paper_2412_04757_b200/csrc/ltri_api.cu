@@ -689,7 +689,7 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
   }
   const long long shift = d.paged ? s0.base - d.Lsp : 0;
   a.shift = shift;
-  // The eviction kernel (one CTA per layer) goes first and releases the append kernel behind it at once: the two
+  // The eviction kernel (eight small CTAs per layer) goes first and releases the append kernel behind it at once: the two
   // touch different data and run side by side; the append kernel waits for the eviction kernel at its end.  They are
   // timed together (class LTRI_K_EVICT); a call that evicts nothing times its append kernel alone (LTRI_K_APPEND).
   {

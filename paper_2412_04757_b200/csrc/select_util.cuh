@@ -429,9 +429,10 @@ __device__ __forceinline__ int merge_ranges_warp(int M, ItemF&& item, int* s_rs,
   return nr;
 }
 
-// a0 inside the one-launch decode retrieval: the CTA of (sequence, layer, KV head) also stores that head's new K and V
-// row (threads 0-31: sixteen 16-byte pieces each), so a decode step needs no separate append launch.  The attention
-// kernel, launched next, is the first reader of the row.  (Resident contexts only: the one-launch path is never paged.)
+// a0 inside the one-launch decode kernels: one CTA of (sequence, layer, KV head) also stores that head's new K and V row
+// (threads 0-31: sixteen 16-byte pieces each; in a sliding slab the window row, and the sink's own row for a sink token), so a
+// decode step needs no separate append launch.  Other CTAs of the same launch must not read the row from the slab: the
+// retrievers leave it to the attention kernel launched next, the one-launch step takes it from the caller's tensors.
 __device__ __forceinline__ void append_decode_row(const DevCtx& c, const DecBatch& b, int bi, int l, int layer_count,
                                                   size_t unit, int g, const __nv_bfloat16* __restrict__ k,
                                                   const __nv_bfloat16* __restrict__ v) {
