@@ -445,7 +445,9 @@ int ltri_create(const ltri_params* p, void* cuda_stream, ltri_ctx** out) {
   // whatever the index size (any of them keeps the one-launch step out)
   if (const char* f = std::getenv("LTRI_DEC_FUSED")) ctx->dec_fused = std::max(0, std::min(2, std::atoi(f)));
   if (const char* f = std::getenv("LTRI_DEC_CLUSTER")) ctx->step_cluster = std::atoi(f);
-  // Clusters are used up to the size that the device can run.  (Testing aid: LTRI_MAX_CLUSTER, the largest size to count on.)
+  // Clusters that need a whole GPC, or the shared memory of several SMs, are used up to the size that the device can run; those
+  // of up to eight small CTAs (segmenter, index build, large-index retriever) always.  (Testing aid: LTRI_MAX_CLUSTER, the
+  // largest size of the former to count on.)
   const char* mc = std::getenv("LTRI_MAX_CLUSTER");
   const int most = mc ? std::atoi(mc) : 16;
   if (ctx->dec_fused < 0 && !ctx->d.vote)
