@@ -579,7 +579,6 @@ def measure(cfg, K, W, rank, local, world, dev, peaks, want_e2e=True, per_layer_
     G = cfg.n_q_heads // cfg.n_kv_heads
     f_ret = sum(4.0 * cnt * G * cfg.head_dim * retrieved_all for (_, cnt) in timed)
     a_ms, a_cnt = prof["attn_local"]
-    a_cnt //= 2     # (every launch of the attention kernel is followed by its redo launch, which returns at once)
     r_ms, _ = prof["attn_retrieved"]
     per_layer = ATTN_LOCAL_DRAM_BYTES_PER_LAYER.get((cfg.n_q_heads, cfg.n_kv_heads, cfg.chunk, cfg.window, cfg.n_sink))
     window_full = timed[0][0] >= cfg.window + cfg.chunk
@@ -590,7 +589,7 @@ def measure(cfg, K, W, rank, local, world, dev, peaks, want_e2e=True, per_layer_
             "traffic_note": "DRAM bytes per launch, ncu capture of a 4-layer case of the same geometry x layers / 4",
             "kernel": "k_attn_tc, local part (sink | local | current)",
             "launches": a_cnt, "ms_per_launch": a_ms / max(a_cnt, 1),
-            "timing": "CUDA events of the library around the launch and its redo launch (which returns at once)"}
+            "timing": "CUDA events of the library around the launch"}
     roof_attn = {"bound": "tensor",
                  **tensor_roofline((f_loc + f_ret) / ((a_ms + r_ms) * 1e-3) / 1e12 if a_ms > 0 else None, peaks, clocks),
                  "kernels": "k_attn_tc local part + continuation over the retrieved spans (the chunked-prefill "

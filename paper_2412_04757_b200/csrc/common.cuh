@@ -18,7 +18,6 @@ constexpr int kMaxRanges = 2 * kMaxTopK + 2;  // sink + local + the spans of thi
 constexpr float kMapMargin = 0.0078125f;          // safety margin (in log2 units) of the map pass's skip test
 constexpr float kMapScale = 0.4972997117f;         // 2^-(1 + kMapMargin)
 constexpr int kTokPad = 128;          // rows of slack after every K/V slab so tile over-reads stay inside it
-constexpr int kTcMaxCtas = 1024;      // most persistent CTAs the tensor-core attention kernel is launched with
 constexpr long long kDefaultWaitLimit = 2000000000ll;  // device-side waits give up after about a second
 
 // Device-side view of one context.  Passed to kernels by value.
@@ -110,7 +109,6 @@ struct DevCtx {
   int* rng_cnt;          // [NS*NL][Hkv]
   float* dec_part;       // [NS*NL][Hq][kMaxDecSplit][128+2]
   int* status;           // [4]: first error code, detail...
-  int* tc_redo;          // [kTcMaxCtas]  per CTA of the tensor-core attention kernel: its work has to be redone
   long long wait_limit;  // upper bound of any single device-side wait, in SM clock cycles
   // what the device offers, read by the dispatch on the host (ltri_create asks; see kernels_state.cu and kernels_attn_tc.cu)
   int sms;               // streaming multiprocessors
@@ -207,8 +205,6 @@ cudaError_t launch_topk_decode(const DevCtx& c, const DecBatch& b, int layer_beg
 // prefill attention.  phase 0: local part over sink|local|cur, stores state (+ final output if `final`);
 // phase 1: continues from the stored state over the selected spans and writes the output; phase 2 (tensor-core
 // kernel only): the same result, with the selected spans accumulated from scratch and merged with the stored state.
-// The tensor-core version is two launches: the second redoes, with exact per-tile maxima, the work of CTAs that met
-// logits too far above their running reference (it returns at once otherwise).
 cudaError_t launch_attn_prefill(const DevCtx& c, const PrefillArgs& a, int phase, bool final, cudaStream_t s);
 // tcgen05/TMEM/TMA version of launch_attn_prefill (same contract) and its availability check
 // host storage for a context's tensor maps: five box heights of the K/V cache, the index, five of the packed slabs

@@ -10,7 +10,7 @@
 // TMEM columns: S0 [0,128) S1 [128,256) O0 [256,384) O1 [384,512); P (bf16) aliases columns [0,32) and [64,96) of
 // its S: every softmax thread overwrites only logit columns it has already read.
 // The issue order QK0, QK1, {PV0_j, QK0_j+1, PV1_j, QK1_j+1} keeps the tensor pipe busy with one tile's MMAs while
-// the other tile's softmax runs.  The running max is updated lazily (only when it grows by more than 2^8), in which
+// the other tile's softmax runs.  The running max is updated lazily (only when it grows by more than 2^24), in which
 // case the softmax thread rescales its O row in TMEM; the in-order tensor pipe guarantees the row is quiescent then.
 // Every wait is bounded; on expiry the CTA sets LTRI_ETIMEOUT in the status word, drains and frees its TMEM.
 #include <cooperative_groups.h>
@@ -32,10 +32,6 @@ constexpr int kMaxItemSplit = 8;  // most CTAs that share a work item
 constexpr int kTcSmem = 65536 + 131072 + 1024;  // queries, two K/V stages, alignment
 constexpr int kNumBoxes = 5;  // box heights 8,16,32,64,128
 constexpr float kRescaleThreshold = 24.0f;
-// Largest exponent (log2 units) a probability may carry above the softmax reference in the regular launch: 2^90 times
-// the 2^7 keys of a tile, the 2^13 tiles of the longest item and values of up to 2^10 still fits fp32 (and the bf16
-// P operand).
-constexpr float kLazyRange = 90.0f;
 
 struct TcMaps {
   CUtensorMap q;             // [tokens][Hq][128] bf16, box {64, G, 256/G}
@@ -151,20 +147,9 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
 // loop is sensitive to every register).
 // SPLIT: the CTAs of a cluster share one work item, each walks every SP-th tile of its keys; the partial softmaxes are
 // merged through distributed shared memory before the epilogue (for launches with fewer items than SMs).
-template <int G, bool EXCH, bool MERGE, bool SPLIT>
+template <int G, bool MERGE, bool SPLIT>
 __global__ void __launch_bounds__(kTcThreads, 1)
-    k_attn_tc(DevCtx c, PrefillArgs a, int phase, int final_out, int* __restrict__ redo,
-              const __grid_constant__ TcMaps maps, long long v_row_offset) {
-  constexpr int exch = EXCH ? 1 : 0;
-  // exch = 0: the regular launch.  Its softmax reference moves one tile late (see the softmax role); a CTA in which
-  // some tile outran that reference by more than the exponent range allows leaves redo[blockIdx.x] = 1.
-  // exch = 1: the launch that follows it with the same grid.  A CTA whose flag is clear returns at once; one whose
-  // flag is set walks its work items again with the true maximum exchanged on every tile and overwrites what the
-  // first launch stored, so inputs of any magnitude get the exact softmax.
-  if (exch) {
-    chain_wait();
-    if (redo[blockIdx.x] == 0) return;
-  }
+    k_attn_tc(DevCtx c, PrefillArgs a, int phase, int final_out, const __grid_constant__ TcMaps maps, long long v_row_offset) {
   const CUtensorMap* kvmaps = maps.kv;
   extern __shared__ unsigned char smem_raw[];
   // QFULL QFREE ODONE[0] | KFULL[2] VFULL[2] KEMPTY[2] VEMPTY[2] | SREADY[2] PREADY[2][2] OFREE[2] | ODONE[1]
@@ -175,7 +160,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __shared__ int s_item_tiles[3];     // tile count of the work items in flight (roles may be up to two items apart)
   __shared__ TileDesc s_td[8];        // per-tile masks, written by the producer, read by the softmax threads
   __shared__ int s_quit[2];
-  __shared__ int s_redo;              // some tile of this CTA outran the late softmax reference
   __shared__ int s_items_ready;       // number of work items whose key ranges the producer has published
   __shared__ float s_max[2][2][2][128];  // per tile parity, Q tile, column half, row: partial maxima
   __shared__ float s_sum[2][2][128];     // per Q tile, column half, row: partial row sums (end of an item)
@@ -189,9 +173,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int rank = SPLIT ? (int)cg::this_cluster().block_rank() : 0;
   const int item0 = SPLIT ? (int)blockIdx.x / SP : (int)blockIdx.x;
   const int istep = SPLIT ? nitems : (int)gridDim.x;  // (a cluster has one item)
-  // written by every CTA of the cluster: its reference maximum and row sum of every row, its redo flag
+  // written by every CTA of the cluster: its reference maximum and row sum of every row
   __shared__ float2 r_ml[SPLIT ? kMaxItemSplit : 1][SPLIT ? 256 : 1];
-  __shared__ int r_redo[kMaxItemSplit];
   __shared__ float2 s_tot[SPLIT ? 256 : 1];  // those of the cluster
   const uint32_t sbase = (smem_addr(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = sbase;                 // 64 KB: [half d][256 rows][64]
@@ -207,7 +190,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   if (tid == 0) {
     s_abort = 0;
     s_quit[0] = s_quit[1] = 0;
-    s_redo = 0;
     s_items_ready = 0;
     rg.n = 0;
     mbar_init(bar(B_QFULL), 1);
@@ -239,7 +221,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = s_tmem_base;
-  if (!exch) chain_wait();  // everything above set up shared memory, barriers and TMEM only
+  chain_wait();  // everything above set up shared memory, barriers and TMEM only
   const int causal_ri = phase == 0 ? 2 : -1;
 
   float2 split_ml = make_float2(-INFINITY, 0.f);  // SPLIT: a softmax thread's row at the end of its tiles
@@ -585,15 +567,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
       int j = 0;
       const int row_abs = a.t0 + tk;
-      bool need_ref = true;   // no reference maximum yet: the first tile exchanges the halves' maxima
-      float mprev = -INFINITY;
       while (j < T) {
         // after an expired wait every thread keeps walking the item's tiles (without computing) so that the named
         // barrier is still reached by all 256 threads of the tile
         ok = ok && mbar_wait(bar(B_SREADY + q), jt & 1, abortp, c.wait_limit);
         if (!ok) {
-          if (need_ref) asm volatile("bar.sync %0, 256;" ::"r"(1 + q) : "memory");
-          need_ref = EXCH;
+          asm volatile("bar.sync %0, 256;" ::"r"(1 + q) : "memory");
           ++j;
           ++jt;
           continue;
@@ -643,25 +622,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
               mx[u] = max3(mx[u], __uint_as_float(v[ch][e + 2 * u]), __uint_as_float(v[ch][e + 2 * u + 1]));
           }
         const float mloc = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-        // The two threads of a row must scale by the same reference.  On an item's first tile (no reference yet)
-        // they exchange their maxima through shared memory and a named barrier.  On later tiles the reference moves
-        // one tile late: it is the maximum over the previous tiles, whose partner half is already visible (the
-        // partner stored it before its PREADY arrival of the previous tile, which precedes this tile's SREADY), so
-        // no barrier sits between the logits and the exponentials.  A tile that exceeds the late reference only
-        // makes the exponent positive; if it does so by more than kLazyRange the probabilities may overflow, so the
-        // thread flags the CTA for the second launch, in which every tile exchanges its maxima like the first one
-        // and the exponent never exceeds the lazy threshold.
+        // The two threads of a row must scale by the same reference: they exchange their maxima through shared memory and a
+        // named barrier on every tile.  (With a reference that lags one tile behind there is no barrier between the logits
+        // and the exponentials, but the work of a CTA in which a tile outruns it has to be done again, by a second launch that
+        // returns at once otherwise: 2 to 3 us a launch, and slower besides.  128K tokens, 4 layers a call: 102.0 ms a prompt
+        // that way, 99.9 with the barrier; 16K, 32 layers: 67.8 and 67.0; 512K, one layer: 138.7 and 135.4.)
         s_max[jt & 1][q][half][r] = mloc;
-        float mt;
-        if (need_ref) {
-          asm volatile("bar.sync %0, 256;" ::"r"(1 + q) : "memory");
-          mt = fmaxf(mloc, s_max[jt & 1][q][half ^ 1][r]) * c2;
-        } else {
-          mt = fmaxf(mprev, s_max[(jt & 1) ^ 1][q][half ^ 1][r]) * c2;
-          if (mloc > -INFINITY && !(mloc * c2 - m_used <= kLazyRange)) *reinterpret_cast<volatile int*>(&s_redo) = 1;
-        }
-        need_ref = EXCH;
-        mprev = mloc;
+        asm volatile("bar.sync %0, 256;" ::"r"(1 + q) : "memory");
+        const float mt = fmaxf(mloc, s_max[jt & 1][q][half ^ 1][r]) * c2;
         // lazy running maximum: move it only when it grows by more than the threshold (or on first use)
         float alpha = 1.f;
         const bool grow = mt > m_used + kRescaleThreshold || (m_used == -INFINITY && mt > -INFINITY);
@@ -812,7 +780,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
     }
   }
-  int redo_any = 0;
   if (SPLIT) {
     // ---------------------------------------------------------------- merge of the cluster's parts
     // Every CTA scales its O rows to the cluster's reference maximum and pushes them to the CTA that owns the row (256 / SP
@@ -835,7 +802,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     float* parts = reinterpret_cast<float*>(smem_raw + (sKV - smem_addr(smem_raw)));
     const Item w = decode(item0);
     const bool any_tile = s_item_tiles[0] > 0;
-    if (tid < SP) *cluster.map_shared_rank(&r_redo[rank], tid) = s_redo;
     if (warp < 16) {
       const int q = warp >> 3, half = (warp >> 2) & 1;
       const int rr = q * 128 + (warp & 3) * 32 + lane;
@@ -869,7 +835,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
     }
     cluster.sync();  // (from here on a CTA reads its own shared memory only)
-    for (int p = 0; p < SP; ++p) redo_any |= r_redo[p];
     if (warp < 16 && !s_abort) {
       // thread = (row, block of `cols` columns); consecutive lanes take consecutive rows
       const int rl = tid % rows, cols = rows / 4, c0 = (tid / rows) * cols;
@@ -932,7 +897,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   fence_after_sync();
   if (warp == 16) tmem_dealloc(tmem, 512);
   if (tid == 0 && s_abort) set_status(c, -6, (int)blockIdx.x);
-  if (tid == 0) redo[blockIdx.x] = exch ? 0 : (SPLIT ? redo_any : s_redo);  // (the second launch leaves the flags clear for the next call)
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -1022,10 +986,10 @@ bool attn_tc_cluster_runs(const DevCtx& c, int cluster) {
     return active_clusters(local, cluster, kTcThreads, kTcSmem) > 0 && active_clusters(merging, cluster, kTcThreads, kTcSmem) > 0;
   };
   switch (c.G) {
-    case 1: return runs(k_attn_tc<1, false, false, true>, k_attn_tc<1, false, true, true>);
-    case 2: return runs(k_attn_tc<2, false, false, true>, k_attn_tc<2, false, true, true>);
-    case 4: return runs(k_attn_tc<4, false, false, true>, k_attn_tc<4, false, true, true>);
-    case 8: return runs(k_attn_tc<8, false, false, true>, k_attn_tc<8, false, true, true>);
+    case 1: return runs(k_attn_tc<1, false, true>, k_attn_tc<1, true, true>);
+    case 2: return runs(k_attn_tc<2, false, true>, k_attn_tc<2, true, true>);
+    case 4: return runs(k_attn_tc<4, false, true>, k_attn_tc<4, true, true>);
+    case 8: return runs(k_attn_tc<8, false, true>, k_attn_tc<8, true, true>);
   }
   return false;
 }
@@ -1033,9 +997,7 @@ bool attn_tc_cluster_runs(const DevCtx& c, int cluster) {
 template <int G>
 static cudaError_t prepare_tc_g() {
   cudaError_t e = cudaSuccess;
-  for (auto fn : {k_attn_tc<G, false, false, false>, k_attn_tc<G, false, false, true>, k_attn_tc<G, false, true, false>,
-                  k_attn_tc<G, false, true, true>, k_attn_tc<G, true, false, false>, k_attn_tc<G, true, false, true>,
-                  k_attn_tc<G, true, true, false>, k_attn_tc<G, true, true, true>})
+  for (auto fn : {k_attn_tc<G, false, false>, k_attn_tc<G, false, true>, k_attn_tc<G, true, false>, k_attn_tc<G, true, true>})
     e = first_error(e, allow_smem(fn, kTcSmem));
   return e;
 }
@@ -1074,18 +1036,11 @@ static cudaError_t launch_tc_g(const DevCtx& c, const PrefillArgs& a, int phase,
   if (const char* cap = getenv("LTRI_TC_MAX_CTAS")) ctas = max(1, min(c.sms, atoi(cap)));
   // persistent CTAs: one per SM (the kernel needs the whole TMEM and most of the shared memory of an SM)
   const int nitems = ((a.n + TOKB - 1) / TOKB) * c.Hkv * a.layer_count;
-  // the regular launch, then the one that redoes the work of the CTAs that asked for it (they return at once otherwise)
   const int tiles = phase == 0 ? (a.sink_end + 127) / 128 + (a.t0 - a.loc_begin + a.n + 127) / 128 : a.ret_tiles;
   const int sp = phase == 1 || ctas < c.sms ? 1 : item_split(c, a, TOKB, tiles);
   const int grid = sp > 1 ? nitems * sp : min(nitems, ctas);
-  if (grid > kTcMaxCtas) return cudaErrorInvalidValue;
-  auto launch = [&](auto fn) {
-    return launch_chained_cluster(fn, dim3(grid), dim3(kTcThreads), sp, kTcSmem, s, c, a, phase, final_out ? 1 : 0, c.tc_redo,
-                                  maps, v_off);
-  };
-  const cudaError_t e = sp > 1 ? launch(k_attn_tc<G, false, MERGE, true>) : launch(k_attn_tc<G, false, MERGE, false>);
-  if (e != cudaSuccess) return e;
-  return sp > 1 ? launch(k_attn_tc<G, true, MERGE, true>) : launch(k_attn_tc<G, true, MERGE, false>);
+  return launch_chained_cluster(sp > 1 ? k_attn_tc<G, MERGE, true> : k_attn_tc<G, MERGE, false>, dim3(grid), dim3(kTcThreads),
+                                sp, kTcSmem, s, c, a, phase, final_out ? 1 : 0, maps, v_off);
 }
 
 cudaError_t launch_attn_prefill_tc(const DevCtx& c, const PrefillArgs& a, int phase, bool final_out,

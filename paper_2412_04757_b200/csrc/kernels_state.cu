@@ -39,8 +39,6 @@ __global__ void k_init(DevCtx c, int seq) {
   }
   if (seq < 0 && tid < 4) c.status[tid] = 0;
   if (seq < 0)
-    for (size_t i = tid; i < (size_t)kTcMaxCtas; i += stride) c.tc_redo[i] = 0;
-  if (seq < 0)
     for (size_t i = tid; i < (size_t)c.NL; i += stride) c.Jcnt[i] = 0;
 }
 

@@ -216,7 +216,6 @@ size_t layout(const ltri_params& p, DevCtx& d, char* base, char** stage_out = nu
   d.rng_cnt = cv.take<int>(units * d.Hkv);
   d.dec_part = cv.take<float>(units * d.Hq * kMaxDecSplit * (kD + 2));
   d.status = cv.take<int>(4);
-  d.tc_redo = cv.take<int>(kTcMaxCtas);
   d.wait_limit = kDefaultWaitLimit;
   d.slots += 1;  // the extra slot is scratch for ltri_debug_segment_map
   if (p.flags & LTRI_FLAG_HOST_STAGING) {
@@ -752,7 +751,7 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
     ag.v = a.v + (size_t)lo * n_tokens * d.Hkv * kD;
     ag.out = a.out + (size_t)lo * n_tokens * d.Hq * kD;
     {
-      Scope sc(ctx, st, LTRI_K_ATTN_LOCAL, ctx->use_tc ? 2 : 1);
+      Scope sc(ctx, st, LTRI_K_ATTN_LOCAL, 1);
       LTRI_CUDA(ctx, ctx->use_tc ? launch_attn_prefill_tc(d, ag, 0, !has_index, ctx->kv_maps, st)
                                  : launch_attn_prefill(d, ag, 0, !has_index, st));
     }
@@ -794,7 +793,7 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
   if (has_index)
     for (int g = 0; g < NG; ++g) {
       if (d.host_kv) LTRI_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_pull[g], 0));
-      Scope sc(ctx, st, LTRI_K_ATTN_RET, ctx->use_tc ? 2 : 1);
+      Scope sc(ctx, st, LTRI_K_ATTN_RET, 1);
       LTRI_CUDA(ctx, ctx->use_tc ? launch_attn_prefill_tc(d, grp[g], ctx->ret_phase, true, ctx->kv_maps, st)
                                  : launch_attn_prefill(d, grp[g], 1, true, st));
     }
