@@ -17,6 +17,8 @@ constexpr int kMaxDecSplit = 32;
 constexpr int kMaxRanges = 2 * kMaxTopK + 2;  // sink + local + the spans of this step's and of the persistent selection
 constexpr float kMapMargin = 0.0078125f;          // safety margin (in log2 units) of the map pass's skip test
 constexpr float kMapScale = 0.4972997117f;         // 2^-(1 + kMapMargin)
+constexpr int kSegSms = 16;            // SMs that a layer of the one-launch segmenter occupies
+constexpr int kSegPasses = 3, kSegHistBits = 12;  // its histograms: 7 bits behind the leading one, 12 more, 12 more
 constexpr int kTokPad = 128;          // rows of slack after every K/V slab so tile over-reads stay inside it
 constexpr long long kDefaultWaitLimit = 2000000000ll;  // device-side waits give up after about a second
 
@@ -90,6 +92,9 @@ struct DevCtx {
   int* Mq;               // [NL][chunk][chunk]
   long long* Rsuf;       // [NL][chunk][chunk]
   long long* best;       // [NL][2*chunk]
+  // one-launch segmenter, clear between launches: histograms [NL][kSegPasses][1 << kSegHistBits], candidates [NL][2*chunk]
+  unsigned* seg_hist;
+  long long* seg_best;
   long long* thetaq;     // [NL]
   float2* rowstat;       // [NL][chunk][Hq]   (reference maximum m in scaled log2 units, row sum l)
   float* rowq;           // [NL][chunk][Hq]   -m - log2(l) + 21 + kMapMargin: offset that turns a scaled logit into
@@ -112,7 +117,7 @@ struct DevCtx {
   long long wait_limit;  // upper bound of any single device-side wait, in SM clock cycles
   // what the device offers, read by the dispatch on the host (ltri_create asks; see kernels_state.cu and kernels_attn_tc.cu)
   int sms;               // streaming multiprocessors
-  int theta_wide;        // layers whose threshold select may take a cluster of sixteen CTAs each (0: no such cluster)
+  int seg_wide;          // layers that the one-launch segmenter takes, a cluster of sixteen CTAs each (0: no such cluster)
   int item_cluster;      // most CTAs that may share an attention work item
 };
 
@@ -187,6 +192,10 @@ cudaError_t launch_evict_index(const DevCtx& c, const EvictArgs& a, int layer_co
 cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start, int slot,
                            int theta_mode, float theta, long long theta_q_abs, int max_spans, int n, int t0,
                            const __nv_bfloat16* q, cudaStream_t s, bool tables = false, int seg_unit = 0);
+// The same in one launch, for prefill calls of few layers.
+bool segment_in_one(const DevCtx& c, int layer_count);
+cudaError_t launch_segment_in_one(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start, int slot,
+                                  long long theta_q_abs, int n, int t0, const __nv_bfloat16* q, cudaStream_t s);
 cudaError_t launch_score_prefill(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s);
 // tensor-core version of launch_score_prefill (split-bf16 representatives)
 cudaError_t launch_score_prefill_mma(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s);
@@ -225,7 +234,7 @@ cudaError_t launch_decode_attn(const DevCtx& c, const DecBatch& b, int layer_beg
 
 // a whole decode step in one launch, clusters of `cluster` CTAs (a power of two up to 16) per (sequence, layer, KV head);
 // contexts without collaborative voting.  indexed_end: end of the indexed prefix (the largest of the batch).
-int theta_wide_clusters();                            // clusters of sixteen CTAs of the threshold select that run at once
+int segment_wide_clusters(const DevCtx& c);           // clusters of sixteen CTAs of the one-launch segmenter that run at once
 bool attn_tc_cluster_runs(const DevCtx& c, int cluster);  // whether that many CTAs can share an attention work item
 int dec_step_capacity(const DevCtx& c, int cluster);  // CTAs that run at once (0: this cluster size is not available)
 bool dec_step_fits(const DevCtx& c, int span_bound, int indexed_end, int cluster);

@@ -4,8 +4,10 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
+#include "mma_util.cuh"
 #include "select_util.cuh"
 
 namespace ltri {
@@ -38,8 +40,11 @@ __global__ void k_init(DevCtx c, int seq) {
     }
   }
   if (seq < 0 && tid < 4) c.status[tid] = 0;
-  if (seq < 0)
+  if (seq < 0) {
     for (size_t i = tid; i < (size_t)c.NL; i += stride) c.Jcnt[i] = 0;
+    for (size_t i = tid; i < ((size_t)c.NL * kSegPasses << kSegHistBits); i += stride) c.seg_hist[i] = 0u;
+    for (size_t i = tid; i < (size_t)c.NL * 2 * c.chunk; i += stride) c.seg_best[i] = 0;
+  }
 }
 
 cudaError_t launch_init(const DevCtx& c, int seq, cudaStream_t s) {
@@ -264,13 +269,22 @@ __device__ __forceinline__ unsigned log_bin(unsigned v) {
   return ((unsigned)e << 4) | frac;
 }
 
+// rank of theta among the causal entries of a layer's map under its own quantile level: the same double arithmetic as on
+// the host
+__device__ __forceinline__ long long layer_rank(const DevCtx& c, int layer, int m) {
+  const long long N = (long long)m * (m + 1) / 2;
+  const long long rank = (long long)floor((double)c.theta_l[layer] * (double)(N - 1));
+  return rank < 0 ? 0 : (rank > N - 1 ? N - 1 : rank);
+}
+// absolute threshold of a layer under its own theta
+__device__ __forceinline__ long long layer_theta_q(const DevCtx& c, int layer, bool one_head) {
+  return (long long)rint((double)c.theta_l[layer] * (one_head ? 1.0 : (double)c.Hq) * (double)kQScale);
+}
+
 constexpr int kThetaThreads = 512;
 
-// H > 0: the cluster has a warp for every pair of rows (i, m - 1 - i) of the map, m + 1 entries in all, and a lane keeps
-// its (at most H) entries in registers, so the map is read once and every pass counts from registers.  H = 0: any
-// size, every pass reads the map.
-template <int H>
-__global__ void __launch_bounds__(H > 0 ? 1024 : kThetaThreads)
+
+__global__ void __launch_bounds__(kThetaThreads)
     k_theta_select(DevCtx c, int layer_begin, int m, long long rank, int tables) {
   chain_wait();
   namespace cg = cooperative_groups;
@@ -279,11 +293,7 @@ __global__ void __launch_bounds__(H > 0 ? 1024 : kThetaThreads)
   const int CL = (int)cluster.num_blocks(), NW = blockDim.x >> 5;
   const int layer = layer_begin + blockIdx.x / CL;
   const int part = (int)cluster.block_rank();
-  if (tables && c.theta_l) {  // the layer's own quantile level: the same double arithmetic as on the host
-    const long long N = (long long)m * (m + 1) / 2;
-    rank = (long long)floor((double)c.theta_l[layer] * (double)(N - 1));
-    rank = rank < 0 ? 0 : (rank > N - 1 ? N - 1 : rank);
-  }
+  if (tables && c.theta_l) rank = layer_rank(c, layer, m);
   const int* Mq = c.Mq + (size_t)layer * c.chunk * c.chunk;
   // this CTA's histogram, then its counts of negatives and zeros: two copies that the passes use in turn, so that one
   // cluster barrier per pass is enough
@@ -295,27 +305,7 @@ __global__ void __launch_bounds__(H > 0 ? 1024 : kThetaThreads)
   __shared__ int s_cls;  // 0: answer found, 1: among positives (bin chosen), -1: among negatives
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned* myhist = hist + warp * kThetaBins;
-  int held[H > 0 ? H : 1];
-  const int pair = part * NW + warp;  // rows pair and m - 1 - pair
-  const int na = 2 * pair < m ? pair + 1 : 0, nb = 2 * pair < m && pair != m - 1 - pair ? m - pair : 0;
-  if (H > 0) {
-    const int* ra = Mq + (size_t)pair * c.chunk;
-    const int* rb = Mq + (size_t)(m - 1 - pair) * c.chunk - na;
-#pragma unroll
-    for (int t = 0; t < H; ++t) {
-      const int k = t * 32 + lane;
-      held[t] = k < na + nb ? (k < na ? ra[k] : rb[k]) : 0;
-    }
-  }
-  auto visit = [&](auto&& f) {
-    if (H > 0) {
-#pragma unroll
-      for (int t = 0; t < H; ++t)
-        if (t * 32 + lane < na + nb) f(held[t]);
-    } else {
-      for_each_causal(Mq, c.chunk, m, part, CL, f);
-    }
-  };
+  auto visit = [&](auto&& f) { for_each_causal(Mq, c.chunk, m, part, CL, f); };
   int pass = 0;
   // sums the per-warp histograms into loc, then the cluster's loc arrays into tot
   auto combine = [&](bool with_counts) {
@@ -434,6 +424,13 @@ __global__ void __launch_bounds__(H > 0 ? 1024 : kThetaThreads)
   cluster.sync();  // nobody leaves while its histogram may still be read
 }
 
+// rank of theta among the m (m + 1) / 2 causal entries
+static long long quantile_rank(float theta, int m) {
+  const long long N = (long long)m * (m + 1) / 2;
+  const long long rank = (long long)floor((double)theta * (double)(N - 1));
+  return rank < 0 ? 0 : (rank > N - 1 ? N - 1 : rank);
+}
+
 // absolute threshold: thq in units of the map summed over all heads, thq1 in units of a single (retrieval) head's map;
 // with per-layer tables the layer's own theta, scaled here
 __global__ void k_theta_set(DevCtx c, int layer_begin, long long thq, long long thq1, int tables) {
@@ -441,7 +438,7 @@ __global__ void k_theta_set(DevCtx c, int layer_begin, long long thq, long long 
   const int layer = layer_begin + blockIdx.x;
   const bool one = ret_head_of(c, layer) >= 0;
   long long t = one ? thq1 : thq;
-  if (tables && c.theta_l) t = (long long)rint((double)c.theta_l[layer] * (one ? 1.0 : (double)c.Hq) * (double)kQScale);
+  if (tables && c.theta_l) t = layer_theta_q(c, layer, one);
   c.thetaq[layer] = t;
 }
 
@@ -610,20 +607,17 @@ struct NmsArgs {
   int seg_unit;              // > 0: every unit of this many tokens (absolute grid) keeps max_spans spans of its own
 };
 
-// A cluster of CTAs may share a layer (its launch says how many): the first CTA runs the NMS and the gap fill, then the
-// spans are dealt to all of them for the representatives.  One layer alone took 40 us (regions of 512) to 73 us (1024) in a
-// single CTA, most of it 32 rounds of two barriers over 1024 threads and five dependent 64-bit shuffles each.
-__global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
-  chain_wait();
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
-  const int CL = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
+// Steps 4 and the representatives, by all CTAs of a cluster (CL of them, this one is `part`): the first CTA runs the NMS
+// and the gap fill, then the spans are dealt to all of them for the representatives.  gbest: the candidates; votes: the
+// votes of token t at votes[t], for the region's tokens.
+__device__ __forceinline__ void spans_and_reps(const DevCtx& c, const NmsArgs& a, cooperative_groups::cluster_group& cluster,
+                                               int CL, int part, int lidx, const long long* gbest, const long long* votes) {
   __shared__ long long skey[768];  // scratch of the query representatives: token lists and counts per span
-  __shared__ int kx[kMaxTopK], ky[kMaxTopK];
+  __shared__ int kx[kMaxTopK], ky[kMaxTopK], ox[kMaxTopK], oy[kMaxTopK];  // kept spans, as found and by start
   __shared__ int out_start[2 * kMaxTopK + 1], out_len[2 * kMaxTopK + 1];
   __shared__ int s_nout;
   __shared__ int s_ucnt[kMaxTopK + 2];  // segmentation per unit: spans kept in every unit the region touches
-  const int lidx = blockIdx.x / CL, layer = a.layer_begin + lidx;
+  const int layer = a.layer_begin + lidx;
   const size_t unit = unit_of(c, a.seq, layer);
   const int m = a.m;
   const int SU = a.seg_unit;
@@ -632,111 +626,148 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   const int phi_milli = a.tables && c.phi_l ? c.phi_l[layer] : c.phi_milli;
   const float rep_lambda = a.tables && c.lambda_l ? c.lambda_l[layer] : c.rep_lambda;
   const int ncand = 2 * m - 1;
-  const long long* gbest = c.best + (size_t)layer * 2 * c.chunk;
   // Greedy NMS without a sort: the candidate the sorted sweep would reach next is the best one that is still alive
   // (key larger, or equal key and smaller anti-diagonal), so every round takes the block-wide maximum over the alive
   // candidates, keeps it, and lets every thread strike out its own candidates that the new span suppresses (or whose
   // unit is full).  At most max_spans rounds of two barriers each instead of sorting up to 2047 keys.
   // Candidate of anti-diagonal cd: key = (S << 10) | (1023 - len) > 0; x = (cd - len) / 2, y = x + len.
-  // The rounds run in the first 8 or 16 warps, four candidates per thread, with one barrier each: the warps' best are
-  // found with three warp-wide integer reductions and meet in one of two arrays that the rounds use in turn.
-  __shared__ uint4 s_wbest[2][16];
+  // The rounds run in the first 8 warps, one barrier each: the warps' best meet in one of two arrays that the rounds use in
+  // turn.  A key is held as its upper 32 significant bits (of the largest key) and the rest, so that one warp-wide maximum
+  // nearly always names the winner.  (Bound: latency of the chain suppress - warp maximum - barrier - maximum.  With three
+  // warp-wide reductions per maximum and a branch per candidate a round took 1300 cycles, now 750.)
+  constexpr int NT = 256, NW = NT / 32;
+  __shared__ uint4 s_wbest[2][NW];
   __shared__ int s_kept;
+  __shared__ unsigned s_bits;  // bits of the largest key
   const int tid = threadIdx.x, wlane = tid & 31, wid = tid >> 5;
-  const int NT = ncand > 1024 ? 512 : 256;
-  if (SU > 0) {
+  if (SU > 0)
     for (int t = tid; t < kMaxTopK + 2; t += blockDim.x) s_ucnt[t] = 0;
-    __syncthreads();
-  }
+  if (tid == 0) s_bits = 0u;
+  __syncthreads();
   if (part == 0 && tid < NT) {
-    auto round_barrier = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(NT) : "memory"); };
-    const int nw = NT >> 5;
-    unsigned khi[4], klo[4];
-    int cx[4], cy[4];
+    auto round_barrier = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };
+    // CU candidates per thread: tid, tid + NT, ...
+    auto rounds = [&](auto cu_tag, auto plain_tag) {
+      constexpr int CU = decltype(cu_tag)::value;
+      constexpr bool PLAIN = decltype(plain_tag)::value;  // any overlap suppresses, no limit per unit
+      unsigned khi[CU], klo[CU], bits = 0u;
+      int cx[CU], cy[CU];
+      {
+        long long key[CU];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int cd = tid + u * NT;
-      const long long key = cd < ncand ? gbest[cd] : 0;
-      const int len = 1023 - (int)(key & 1023);
-      cx[u] = (cd - len) >> 1;
-      cy[u] = cx[u] + len;
-      khi[u] = key > 0 ? (unsigned)(key >> 32) : 0u;  // (key 0: not alive)
-      klo[u] = key > 0 ? (unsigned)key : 0u;
-    }
-    // warp-wide best of (hi, lo) descending, then cd ascending
-    auto reduce = [&](unsigned& hi, unsigned& lo, int& cd) {
-      const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
-      const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-      cd = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? cd : 0x7fffffff);
-      hi = mh;
-      lo = ml;
-    };
-    int kept = 0;
-    while (kept < cap_total) {
-      unsigned bh = 0, bl = 0;
-      int bc = 0x7fffffff;
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (khi[u] > bh || (khi[u] == bh && klo[u] > bl)) {  // (ascending candidates: an equal one does not replace)
-          bh = khi[u];
-          bl = klo[u];
-          bc = tid + u * NT;
+        for (int u = 0; u < CU; ++u) {
+          const int cd = tid + u * NT;
+          key[u] = cd < ncand ? max(__ldcg(gbest + cd), 0ll) : 0;  // (0: not alive)
+          const int len = 1023 - (int)(key[u] & 1023);
+          cx[u] = (cd - len) >> 1;
+          cy[u] = cx[u] + len;
+          bits = max(bits, 64u - (unsigned)__clzll(key[u]));
         }
-      reduce(bh, bl, bc);
-      uint4* buf = s_wbest[kept & 1];
-      if (wlane == 0) buf[wid] = make_uint4(bh, bl, (unsigned)bc, 0u);
-      round_barrier();
-      const uint4 w = wlane < nw ? buf[wlane] : make_uint4(0u, 0u, 0x7fffffffu, 0u);
-      bh = w.x;
-      bl = w.y;
-      bc = (int)w.z;
-      reduce(bh, bl, bc);
-      if ((bh | bl) == 0u) break;  // nothing alive is left (the same decision in every thread)
-      const int wl = 1023 - (int)(bl & 1023);
-      const int wx = (bc - wl) >> 1, wy = wx + wl;
-      if (tid == 0) {
-        kx[kept] = wx;
-        ky[kept] = wy;
-        if (SU > 0) ++s_ucnt[unit_idx(wx)];
-      }
-      ++kept;
-      if (SU > 0) round_barrier();  // the unit counts are up to date
+        bits = __reduce_max_sync(0xffffffffu, bits);
+        if (wlane == 0) atomicMax(&s_bits, bits);
+        round_barrier();
+        const unsigned sh = max(s_bits, 32u) - 32u;
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if ((khi[u] | klo[u]) != 0u &&
-            (tid + u * NT == bc || nms_suppressed(cx[u], cy[u], wx, wy, phi_milli) ||
-             (SU > 0 && s_ucnt[unit_idx(cx[u])] >= a.max_spans)))
-          khi[u] = klo[u] = 0u;
-      if (SU > 0) round_barrier();  // (everybody has read them)
-    }
-    if (tid == 0) s_kept = kept;
+        for (int u = 0; u < CU; ++u) {
+          khi[u] = (unsigned)(key[u] >> sh);
+          klo[u] = (unsigned)key[u] & ((1u << sh) - 1u);
+        }
+      }
+      const unsigned sh = max(s_bits, 32u) - 32u;
+      // the lane that holds the warp-wide best of (hi, lo) descending, then cd ascending
+      auto winner = [&](unsigned hi, unsigned lo, int cd) {
+        const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+        unsigned at = __ballot_sync(0xffffffffu, hi == mh);
+        if (at & (at - 1u)) {
+          const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+          const int mc = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? cd : 0x7fffffff);
+          at = __ballot_sync(0xffffffffu, hi == mh && lo == ml && cd == mc);
+        }
+        return __ffs(at) - 1;
+      };
+      int kept = 0;
+      while (kept < cap_total) {
+        unsigned bh = khi[0], bl = klo[0];
+        int bc = tid;
+#pragma unroll
+        for (int u = 1; u < CU; ++u) {
+          const bool more = khi[u] > bh || (khi[u] == bh && klo[u] > bl);  // (ascending: an equal one does not replace)
+          bh = more ? khi[u] : bh;
+          bl = more ? klo[u] : bl;
+          bc = more ? tid + u * NT : bc;
+        }
+        uint4* buf = s_wbest[kept & 1];
+        if (wlane == winner(bh, bl, bc)) buf[wid] = make_uint4(bh, bl, (unsigned)bc, 0u);
+        round_barrier();
+        uint4 w = wlane < NW ? buf[wlane] : make_uint4(0u, 0u, 0x7fffffffu, 0u);
+        w = buf[winner(w.x, w.y, (int)w.z) & (NW - 1)];  // (nothing alive: any of the empty entries)
+        if ((w.x | w.y) == 0u) break;  // nothing alive is left (the same decision in every thread)
+        const int wl = 1023 - (int)(((w.x << sh) | w.y) & 1023u);
+        const int wx = ((int)w.z - wl) >> 1, wy = wx + wl;
+        if (tid == 0) {
+          kx[kept] = wx;
+          ky[kept] = wy;
+          if (!PLAIN && SU > 0) ++s_ucnt[unit_idx(wx)];
+        }
+        ++kept;
+        if (PLAIN) {
+#pragma unroll
+          for (int u = 0; u < CU; ++u) {
+            const bool apart = cy[u] < wx || cx[u] > wy;
+            khi[u] = apart ? khi[u] : 0u;
+            klo[u] = apart ? klo[u] : 0u;
+          }
+        } else {
+          if (SU > 0) round_barrier();  // the unit counts are up to date
+#pragma unroll
+          for (int u = 0; u < CU; ++u)
+            if ((khi[u] | klo[u]) != 0u &&
+                (tid + u * NT == (int)w.z || nms_suppressed(cx[u], cy[u], wx, wy, phi_milli) ||
+                 (SU > 0 && s_ucnt[unit_idx(cx[u])] >= a.max_spans)))
+              khi[u] = klo[u] = 0u;
+          if (SU > 0) round_barrier();  // (everybody has read them)
+        }
+      }
+      if (tid == 0) s_kept = kept;
+    };
+    using four = std::integral_constant<int, 4>;
+    using eight = std::integral_constant<int, 8>;
+    const bool plain = SU == 0 && phi_milli == 0, few = ncand <= 4 * NT;
+    if (plain && few)
+      rounds(four(), std::true_type());
+    else if (plain)
+      rounds(eight(), std::true_type());
+    else if (few)
+      rounds(four(), std::false_type());
+    else
+      rounds(eight(), std::false_type());
   }
+  __syncthreads();
+  // order the kept spans by start, a warp per span; with phi > 0 two of them may share their start: then the shorter first
+  if (part == 0)
+    for (int w = wid; w < s_kept; w += blockDim.x >> 5) {
+      const int x = kx[w], y = ky[w];
+      int rank = 0;
+#pragma unroll
+      for (int b = 0; b < kMaxTopK; b += 32) {
+        const int q = b + wlane;
+        rank += __popc(__ballot_sync(0xffffffffu, q < s_kept && (kx[q] < x || (kx[q] == x && ky[q] < y))));
+      }
+      if (wlane == 0) {
+        ox[rank] = x;
+        oy[rank] = y;
+      }
+    }
   __syncthreads();
   if (part == 0 && threadIdx.x < 32) {
     const int lane = threadIdx.x, kept = s_kept;
-    // order the kept spans by start (rank sort), then gap fill
-    int rank0 = 0, rank1 = 0;
-    const int x0 = lane < kept ? kx[lane] : 0x7fffffff;
-    const int x1 = lane + 32 < kept ? kx[lane + 32] : 0x7fffffff;
-    const int y0 = lane < kept ? ky[lane] : 0, y1 = lane + 32 < kept ? ky[lane + 32] : 0;
-    for (int q = 0; q < kept; ++q) {  // with phi > 0 two kept spans may share their start: then the shorter first
-      rank0 += kx[q] < x0 || (kx[q] == x0 && ky[q] < y0);
-      rank1 += kx[q] < x1 || (kx[q] == x1 && ky[q] < y1);
-    }
-    __syncwarp();
-    if (lane < kept) kx[rank0] = x0;
-    if (lane + 32 < kept) kx[rank1] = x1;
-    __syncwarp();
-    if (lane < kept) ky[rank0] = y0;
-    if (lane + 32 < kept) ky[rank1] = y1;
-    __syncwarp();
     if (SU == 0) {
       // two entries per lane: the end of everything covered in front of a span (a prefix maximum: with phi > 0 kept spans
       // may overlap) tells whether an uncovered run precedes it, the number of such runs where it goes
       int covered = 0, no = 0;
       for (int base = 0; base < kept; base += 32) {
         const int q = base + lane;
-        const int sx = q < kept ? kx[q] : 0x7fffffff, sy = q < kept ? ky[q] + 1 : 0;
+        const int sx = q < kept ? ox[q] : 0x7fffffff, sy = q < kept ? oy[q] + 1 : 0;
         int inc = sy;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -778,30 +809,33 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
         }
       };
       for (int q = 0; q < kept; ++q) {
-        if (kx[q] > pos) emit_gap(pos, kx[q]);
+        if (ox[q] > pos) emit_gap(pos, ox[q]);
         if (no < 2 * kMaxTopK + 1) {
-          out_start[no] = kx[q];
-          out_len[no++] = ky[q] - kx[q] + 1;
+          out_start[no] = ox[q];
+          out_len[no++] = oy[q] - ox[q] + 1;
         }
-        pos = max(pos, ky[q] + 1);  // kept spans may overlap when phi > 0
+        pos = max(pos, oy[q] + 1);  // kept spans may overlap when phi > 0
       }
       if (pos < m) emit_gap(pos, m);
       s_nout = no;
     }
   }
-  if (CL > 1) {
-    cluster.sync();
-    if (part > 0) {
-      const int n = *cluster.map_shared_rank(&s_nout, 0);
-      if (threadIdx.x == 0) s_nout = n;
-      for (int t = threadIdx.x; t < min(n, 2 * kMaxTopK + 1); t += blockDim.x) {
-        out_start[t] = cluster.map_shared_rank(out_start, 0)[t];
-        out_len[t] = cluster.map_shared_rank(out_len, 0)[t];
+  __syncthreads();
+  if (CL > 1) {  // pushed to the others, not fetched by them: one barrier and no round trip
+    if (part == 0) {
+      const int n = min(s_nout, 2 * kMaxTopK + 1);
+      for (int t = tid; t < (n + 1) * CL; t += blockDim.x) {
+        const int r = t % CL, i = t / CL;
+        if (i == n) {
+          if (r > 0) *cluster.map_shared_rank(&s_nout, r) = s_nout;
+        } else if (r > 0) {
+          cluster.map_shared_rank(out_start, r)[i] = out_start[i];
+          cluster.map_shared_rank(out_len, r)[i] = out_len[i];
+        }
       }
     }
-    cluster.sync();  // (the first CTA's shared memory is not read after this point)
+    cluster.sync();  // (from here on a CTA reads its own shared memory only)
   }
-  __syncthreads();
   const int nout = s_nout;
   const size_t ps = (unit * c.slots + a.slot) * c.Jmax;
   if (nout > c.Jmax) {
@@ -820,7 +854,6 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   // query representatives.  First one warp per span picks the representative tokens, then one warp per
   // (span, KV head) sums their query rows with all loads of the head group in flight at once.
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  const long long* votes = c.votes + unit * c.Tpad;
   const __nv_bfloat16* q = a.q + (size_t)lidx * a.n * c.Hq * kD;
   int* rep_tok = reinterpret_cast<int*>(skey);          // [Jmax][kMaxReps]
   int* rep_cnt = rep_tok + (2 * kMaxTopK + 1) * kMaxReps;
@@ -936,13 +969,354 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
   }
 }
 
+// A cluster of CTAs may share a layer (its launch says how many).
+__global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
+  chain_wait();
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int CL = (int)cluster.num_blocks(), lidx = blockIdx.x / CL, layer = a.layer_begin + lidx;
+  if (CL > 1) cluster.sync();  // (every CTA runs before the first store to another)
+  spans_and_reps(c, a, cluster, CL, (int)cluster.block_rank(), lidx, c.best + (size_t)layer * 2 * c.chunk,
+                 c.votes + unit_of(c, a.seq, layer) * c.Tpad);
+}
+
+// The segmenter of a few layers in one launch: threshold, both cumulative sums, candidates, NMS and representatives.  A
+// cluster of 16 CTAs shares a layer's m x m map: CTA p holds the row blocks p and 31 - p of 32 (33 column blocks whatever
+// p is) and keeps the raw row suffix sums RS[i][x] = sum_{j=x..i} Mq[i][j] in shared memory.  With T(x,y) the sum of RS
+// over the rows x..y of column x, the score of Fig. 2 is S(x,y) = T(x,y) - theta * len (len + 1) / 2, so the map is read
+// once, and the column sums of the 32 row blocks and the histograms of the entries cross the cluster behind one barrier.
+// Both go through L2: gathered from the other CTAs' shared memory, 64 KB a CTA, they took 8K cycles each time.
+// Bound: latency, a dozen dependent steps.  As four launches, with the map and a 64-bit table of sums going through L2 between
+// them, a layer took 36 us (256 tokens), 45 (512) and 66 (1024); now 20, 30 and 55.
+// The map's entries are not negative and a row's sum over all heads is at most Hq * (2^20 + 512), so RS fits 32 bits; PT, the
+// type of a block's column sums (at most 32 rows), is 32 bits up to 64 heads.
+constexpr int kSegThreads = 1024, kSegCluster = kSegSms, kSegBlocks = 2 * kSegCluster;
+constexpr int kSegFrac = 7;                         // the first histogram has 2^7 bins per power of two,
+constexpr int kSegBits = kSegHistBits;              // the others resolve 12 bits a pass
+constexpr int kSegBins = 1 << kSegBits;             // (four per thread)
+constexpr int kSegRowVec = 1024 / 128;              // 128-entry groups of the longest row
+static_assert(kSegBins == 4 * kSegThreads, "four bins per thread");
+
+struct SegArgs {
+  NmsArgs nms;
+  int theta_mode;         // 1: quantile (of rank `rank`), otherwise the threshold is given
+  int bh;                 // rows of a block: m / 32, rounded up
+  long long rank, thq, thq1;
+};
+
+// monotone log-scale bin of a positive value: exponent and first bits of its fp32 form (rounded towards zero)
+__device__ __forceinline__ unsigned seg_bin(unsigned v) {
+  return (__float_as_uint(__uint2float_rz(v)) >> (23 - kSegFrac)) - (127u << kSegFrac);
+}
+
+__host__ __device__ inline int seg_stride(int blocks, int bh) { return (blocks * bh + 3) & ~3; }
+// dynamic shared memory: histogram | T above each half of the two blocks, per column | candidates [2m + 1] | votes [m] (8 bytes
+// each) | row sums
+__host__ __device__ inline size_t seg_rows_at(int m, int bh) {
+  return kSegBins * 4 + (((size_t)2 * (kSegBlocks + 1) * bh + 3 * m + 2) & ~(size_t)1) * 8;
+}
+static size_t seg_smem(int m, int bh) {  // (two row strides, each rounded up by at most three words)
+  return seg_rows_at(m, bh) + (size_t)bh * ((kSegBlocks + 1) * bh + 6) * sizeof(unsigned);
+}
+
+template <typename PT>
+__global__ void __launch_bounds__(kSegThreads, 1) k_segment(DevCtx c, SegArgs a) {
+  chain_wait();
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int part = (int)cluster.block_rank(), lidx = blockIdx.x / kSegCluster, layer = a.nms.layer_begin + lidx;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NW = kSegThreads / 32;
+  const int m = a.nms.m, BH = a.bh;
+  const size_t unit = unit_of(c, a.nms.seq, layer);
+  // blocks A = part and B = 31 - part: columns (up to the block's last row), row strides of the sums
+  const int bA = part, bB = kSegBlocks - 1 - part;
+  const int nA = (bA + 1) * BH, nB = (bB + 1) * BH, ldA = seg_stride(bA + 1, BH), ldB = seg_stride(bB + 1, BH);
+  extern __shared__ __align__(16) unsigned char dyn[];
+  unsigned* hist = reinterpret_cast<unsigned*>(dyn);                    // [kSegBins]
+  long long* above = reinterpret_cast<long long*>(hist + kSegBins);     // [2][nA + nB]: first half, second half of the rows
+  long long* sbest = above + 2 * (kSegBlocks + 1) * BH;                 // [2m - 1]
+  long long* svotes = sbest + (2 * m + 1);                              // [m]
+  unsigned* RS = reinterpret_cast<unsigned*>(dyn + seg_rows_at(m, BH));  // A's rows, then B's
+  __shared__ unsigned s_wsum[NW], s_bin;
+  __shared__ long long s_rank;
+  // what the cluster adds up: histograms [pass][bin] and candidates; clear at the start, left clear at the end
+  unsigned* ghist = c.seg_hist + (size_t)layer * kSegPasses * kSegBins;
+  long long* gbest = c.seg_best + (size_t)layer * 2 * c.chunk;
+  PT* gsum = reinterpret_cast<PT*>(c.Rsuf + (size_t)layer * c.chunk * c.chunk);  // [block][m] column sums of the blocks
+  const int* Mq = c.Mq + (size_t)layer * c.chunk * c.chunk;
+  const long long* votes = c.votes + unit * c.Tpad + a.nms.reg_start;
+  const bool quant = a.theta_mode == 1;
+
+  reinterpret_cast<uint4*>(hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
+  if (a.nms.q)  // (on their way until the representatives are chosen)
+    for (int t = tid; t < m; t += kSegThreads) cp_async8(smem_u32(svotes + t), votes + t);
+  cp_async_commit();
+  for (int t = tid; t < 2 * m - 1; t += kSegThreads) sbest[t] = 0;
+  __syncthreads();
+
+  // ---- the rows: histogram of the entries, suffix sums.  A warp per row; a lane holds four consecutive entries of every
+  // group of 128, all of them requested before the first is used.
+  const int bh2 = 2 * BH;
+  auto row_of = [&](int lr) { return lr < BH ? bA * BH + lr : bB * BH + lr - BH; };
+  auto sums_of = [&](int lr) { return lr < BH ? RS + lr * ldA : RS + BH * ldA + (lr - BH) * ldB; };
+#pragma unroll 1
+  for (int lr = warp; lr < bh2; lr += NW) {
+    const int i = row_of(lr), ld = lr < BH ? ldA : ldB;
+    const int last = i < m ? i : -1;  // (rows behind the map: zeros)
+    const int* row = Mq + (size_t)i * c.chunk;
+    unsigned* rs = sums_of(lr);
+    int4 v[kSegRowVec];
+#pragma unroll
+    for (int k = 0; k < kSegRowVec; ++k) {
+      const int x = k * 128 + lane * 4;
+      v[k] = x <= last ? *reinterpret_cast<const int4*>(row + x) : make_int4(0, 0, 0, 0);
+    }
+    unsigned carry = 0;
+#pragma unroll
+    for (int k = kSegRowVec - 1; k >= 0; --k) {
+      if (k * 128 >= ld) continue;  // (uniform over the warp)
+      const int x = k * 128 + lane * 4;
+      const unsigned e0 = (unsigned)v[k].x, e1 = x + 1 <= last ? (unsigned)v[k].y : 0u,
+                     e2 = x + 2 <= last ? (unsigned)v[k].z : 0u, e3 = x + 3 <= last ? (unsigned)v[k].w : 0u;
+      const unsigned s3 = e3, s2 = s3 + e2, s1 = s2 + e1, s0 = s1 + e0;
+      unsigned inc = s0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_down_sync(0xffffffffu, inc, o);
+        if (lane + o < 32) inc += t;
+      }
+      const unsigned right = carry + inc - s0;
+      if (x < ld) *reinterpret_cast<uint4*>(rs + x) = make_uint4(right + s0, right + s1, right + s2, right + s3);
+      carry += __shfl_sync(0xffffffffu, inc, 0);
+      if (quant) {
+        if (e0 != 0u) atomicAdd(&hist[seg_bin(e0)], 1u);
+        if (e1 != 0u) atomicAdd(&hist[seg_bin(e1)], 1u);
+        if (e2 != 0u) atomicAdd(&hist[seg_bin(e2)], 1u);
+        if (e3 != 0u) atomicAdd(&hist[seg_bin(e3)], 1u);
+      }
+    }
+  }
+  __syncthreads();
+  // adds this CTA's histogram to the cluster's
+  auto flush = [&](int pass) {
+    const uint4 h = reinterpret_cast<const uint4*>(hist)[tid];
+    unsigned* g = ghist + pass * kSegBins + tid * 4;
+    if (h.x) atomicAdd(g, h.x);
+    if (h.y) atomicAdd(g + 1, h.y);
+    if (h.z) atomicAdd(g + 2, h.z);
+    if (h.w) atomicAdd(g + 3, h.w);
+  };
+  if (quant) flush(0);
+  // ---- column sums of the two blocks; the sum over the first half of a block's rows stays here
+  const int hb = (BH + 1) >> 1;
+  for (int t = tid; t < nA + nB; t += kSegThreads) {
+    const bool inA = t < nA;
+    const int ld = inA ? ldA : ldB, x = inA ? t : t - nA, b = inA ? bA : bB;
+    const unsigned* col = inA ? RS + x : RS + BH * ldA + x;
+    PT sum = 0;
+#pragma unroll 8
+    for (int y = 0; y < hb; ++y) sum += col[y * ld];
+    above[nA + nB + t] = (long long)sum;
+#pragma unroll 8
+    for (int y = hb; y < BH; ++y) sum += col[y * ld];
+    if (x < m && b * BH < m) gsum[(size_t)b * m + x] = sum;
+  }
+  cluster.sync();
+
+  // ---- what the cluster knows: the histogram, and the column sums of the row blocks above this CTA's
+  // the bin of the cluster's histogram in which rank `rank` falls (-1: among the zeros), and its rank inside it, to every thread
+  auto pick = [&](int pass, long long rank) {
+    const uint4 h = __ldcg(reinterpret_cast<const uint4*>(ghist + pass * kSegBins) + tid);
+    const unsigned own = h.x + h.y + h.z + h.w;
+    unsigned inc = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned u = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += u;
+    }
+    if (lane == 31) s_wsum[warp] = inc;
+    __syncthreads();
+    const unsigned w = s_wsum[lane];
+    if (pass == 0) rank -= (long long)m * (m + 1) / 2 - __reduce_add_sync(0xffffffffu, w);  // the zeros are not counted
+    inc += __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u);
+    const long long at = rank - (long long)(inc - own);  // rank counted from this thread's first bin
+    if (at >= 0 && at < (long long)own) {
+      const unsigned r = (unsigned)at, c1 = h.x, c2 = c1 + h.y, c3 = c2 + h.z;
+      s_bin = tid * 4 + (r >= c1) + (r >= c2) + (r >= c3);
+      s_rank = r - (r >= c3 ? c3 : r >= c2 ? c2 : r >= c1 ? c1 : 0u);
+    }
+    if (rank < 0 && tid == 0) s_bin = 0xffffffffu;
+    __syncthreads();
+  };
+  long long thq = a.thq;
+  unsigned prefix = 0;
+  int hi = 0;  // bits of theta still unknown
+  if (quant) {
+    pick(0, a.nms.tables && c.theta_l ? layer_rank(c, layer, m) : a.rank);
+    const unsigned bin = s_bin;  // (the same in every CTA)
+    if (bin == 0xffffffffu) {
+      thq = 0;
+    } else {
+      const int e = (int)(bin >> kSegFrac);
+      const unsigned frac = bin & ((1u << kSegFrac) - 1u);
+      if (e <= kSegFrac) {  // the bin holds a single value
+        thq = (long long)((1u << e) | (frac >> (kSegFrac - e)));
+      } else {
+        hi = e - kSegFrac;
+        prefix = (1u << e) | (frac << hi);  // the leading one and the bits behind it
+      }
+    }
+  } else {
+    const bool one = ret_head_of(c, layer) >= 0;
+    if (one) thq = a.thq1;
+    if (a.nms.tables && c.theta_l) thq = layer_theta_q(c, layer, one);
+  }
+  // T(x, y) of the row above a block: the sums of the blocks from column x's own down to it
+  for (int t = tid; t < nA + nB; t += kSegThreads) {
+    const bool inA = t < nA;
+    const int x = inA ? t : t - nA, b = inA ? bA : bB;
+    long long sum = 0;
+    const int q0 = x / BH, n = x < m ? min(b, (m + BH - 1) / BH) - q0 : 0;  // (sixteen in flight)
+    const PT* from = gsum + (size_t)q0 * m + x;
+#pragma unroll 1
+    for (int q = 0; q < n; q += 16, from += (size_t)16 * m)
+#pragma unroll
+      for (int i = 0; i < 16; ++i) sum += q + i < n ? __ldcg(from + (size_t)i * m) : (PT)0;
+    above[t] = sum;
+    above[nA + nB + t] += sum;
+  }
+  // ---- theta: the low bits over the entries that share the bits found so far
+  for (int pass = 1; hi > 0; ++pass) {  // (the same decisions in every CTA of the cluster)
+    const int lo = max(0, hi - kSegBits);
+    const unsigned dmask = (1u << (hi - lo)) - 1u;
+    const long long left = s_rank;
+    reinterpret_cast<uint4*>(hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+#pragma unroll 1
+    for (int lr = warp; lr < bh2; lr += NW) {
+      const int ld = lr < BH ? ldA : ldB;
+      const unsigned* rs = sums_of(lr);
+#pragma unroll 4
+      for (int x = lane * 4; x - lane * 4 < ld; x += 128) {
+        uint4 r = make_uint4(0u, 0u, 0u, 0u);
+        if (x < ld) r = *reinterpret_cast<const uint4*>(rs + x);
+        unsigned next = __shfl_down_sync(0xffffffffu, r.x, 1);
+        if (lane == 31) next = x + 4 < ld ? rs[x + 4] : 0u;
+        auto count = [&](unsigned val) {
+          if ((val >> hi) == (prefix >> hi)) atomicAdd(&hist[(val >> lo) & dmask], 1u);
+        };
+        count(r.x - r.y);
+        count(r.y - r.z);
+        count(r.z - r.w);
+        count(r.w - next);
+      }
+    }
+    __syncthreads();
+    flush(pass);
+    cluster.sync();
+    pick(pass, left);
+    prefix |= s_bin << lo;
+    hi = lo;
+    thq = (long long)prefix;
+  }
+  __syncthreads();
+  if (part == 0 && tid == 0) c.thetaq[layer] = thq;
+  if (c.rep_mode == 1) {  // the table that the area ratios are read from (see k_seg_rowscan), over the blocks' column sums
+    cluster.sync();
+    for (int lr = warp; lr < bh2; lr += NW) {
+      const int i = row_of(lr);
+      if (i >= m) continue;
+      long long* out = c.Rsuf + ((size_t)layer * c.chunk + i) * c.chunk;
+      for (int x = lane; x <= i; x += 32) out[x] = (long long)sums_of(lr)[x] - thq * (i - x + 1);
+    }
+  }
+  // ---- S(x, y) and the best point of every anti-diagonal (see k_seg_colscan).  A warp takes 32 columns of half a block, a
+  // column per lane, row by row; the best of an anti-diagonal moves one lane down with every row, so that only what leaves
+  // the warp takes an atomic (64-bit maxima in shared memory are loops).  Bound: issue slots, some 25 instructions an entry.
+  const int SU = a.nms.seg_unit;
+  const int gA = (nA + 31) >> 5, gB = (nB + 31) >> 5;
+#pragma unroll 1
+  for (int w = warp; w < 2 * (gA + gB); w += NW) {
+    const int half = w & 1, grp = w >> 1;
+    const bool inA = grp < gA;
+    const int x0 = (inA ? grp : grp - gA) * 32, x = x0 + lane, n = inA ? nA : nB, ld = inA ? ldA : ldB;
+    const int yb = (inA ? bA : bB) * BH, y1 = min(min(m, yb + BH), half ? yb + BH : yb + hb);
+    const bool col_ok = x < n;
+    const int ymax = !col_ok ? -1 : SU > 0 ? ((a.nms.reg_start + x) / SU + 1) * SU - a.nms.reg_start - 1 : m;
+    const unsigned* col = (inA ? RS : RS + BH * ldA) + min(x, n - 1);
+    long long* out = reinterpret_cast<long long*>(hist) + warp * 16;  // what leaves the warp, a row's at a time
+    long long best = 0;
+    const int y0 = max(half ? yb + hb : yb, x0);  // (above the diagonal of the first column there is nothing)
+    if (y0 >= y1) continue;
+    // S = D + the half block's own rows, D = T above the half block - theta * len (len + 1) / 2 from row to row (the recurrence
+    // holds for len <= 0 too); the own rows above the diagonal are zeros
+    const int len0 = y0 - x + 1;
+    long long step = thq * len0;
+    long long D = (col_ok ? above[(half ? nA + nB : 0) + (inA ? x : nA + x)] : 0) - ((thq * len0 * (len0 - 1)) >> 1);
+    PT own = 0;
+    unsigned low = (unsigned)(1024 - len0);
+#pragma unroll 2
+    for (int y = y0; y < y1; ++y) {
+      own += col[(y - yb) * ld];
+      D -= step;
+      step += thq;
+      const long long S = D + (long long)own;
+      if (y >= x && y <= ymax && S > 0) best = max(best, (S << 10) | (long long)low);
+      --low;
+      if (lane == 0) out[y - y0] = best;
+      best = __shfl_down_sync(0xffffffffu, best, 1);
+      if (lane == 31) best = 0;
+    }
+    __syncwarp();
+    const long long left = lane < y1 - y0 ? out[lane] : 0;  // what left the warp after row y0 + lane
+    __syncwarp();
+    // (lane l now holds the anti-diagonal of column x + 1 in the last row)
+    auto give = [&](long long key, int cd) {
+      if (key > 0 && key > *reinterpret_cast<volatile long long*>(&sbest[cd])) atomicMax(&sbest[cd], key);
+    };
+    give(left, min(x0 + y0 + lane, 2 * m - 2));
+    give(best, min(x + y1, 2 * m - 2));
+  }
+  __syncthreads();
+  for (int t = tid; t < 2 * m - 1; t += kSegThreads) {
+    const long long key = sbest[t];
+    if (key > 0) atomicMax(&gbest[t], key);
+  }
+  cp_async_wait<0>();  // (this thread's votes; the barriers below order all of them)
+  cluster.sync();
+  if (part > 0)
+    for (int t = (part - 1) * kSegThreads + tid; t < kSegPasses * kSegBins / 4; t += (kSegCluster - 1) * kSegThreads)
+      reinterpret_cast<uint4*>(ghist)[t] = make_uint4(0u, 0u, 0u, 0u);
+  spans_and_reps(c, a.nms, cluster, kSegCluster, part, lidx, gbest, svotes - a.nms.reg_start);
+  if (part == 0)  // (read by this CTA only, before the barriers in there)
+    for (int t = tid; t < 2 * m - 1; t += kSegThreads) gbest[t] = 0;
+}
+
 constexpr int kSegWideLayers = 7;    // most layers that get a cluster of 16 (as many run at once on a whole GPU)
-constexpr int kThetaWideSmem = 32 * kThetaBins * (int)sizeof(unsigned);  // a histogram per warp
 constexpr int kSegShareLayers = 16;  // up to here four CTAs share a layer's representatives
 
-int theta_wide_clusters() {
-  return std::min({kSegWideLayers, active_clusters(k_theta_select<17>, 16, 1024, kThetaWideSmem),
-                   active_clusters(k_theta_select<33>, 16, 1024, kThetaWideSmem)});
+static bool seg_wide_sums(const DevCtx& c) { return c.Hq > 64; }
+
+int segment_wide_clusters(const DevCtx& c) {
+  const int smem = (int)seg_smem(c.chunk, (c.chunk + kSegBlocks - 1) / kSegBlocks);
+  return std::min(kSegWideLayers, seg_wide_sums(c) ? active_clusters(k_segment<unsigned long long>, kSegCluster, kSegThreads, smem)
+                                                   : active_clusters(k_segment<unsigned>, kSegCluster, kSegThreads, smem));
+}
+
+// A cluster of 16 needs a GPC to itself, so seven run at once; more layers keep the GPU busy as separate launches.
+bool segment_in_one(const DevCtx& c, int layer_count) { return layer_count <= c.seg_wide; }
+
+cudaError_t launch_segment_in_one(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start, int slot,
+                                  long long theta_q_abs, int n, int t0, const __nv_bfloat16* q, cudaStream_t s) {
+  SegArgs a;
+  a.nms = NmsArgs{seq, layer_begin, m, reg_start, slot, c.C, n, t0, q, 1, c.seg_unit};
+  a.theta_mode = c.theta_mode;
+  a.bh = (m + kSegBlocks - 1) / kSegBlocks;
+  a.rank = quantile_rank(c.theta, m);
+  a.thq = theta_q_abs;
+  a.thq1 = (long long)nearbyint((double)c.theta * (double)kQScale);
+  return launch_chained_cluster(seg_wide_sums(c) ? k_segment<unsigned long long> : k_segment<unsigned>,
+                                dim3(layer_count * kSegCluster), dim3(kSegThreads), kSegCluster, seg_smem(m, a.bh), s, c, a);
 }
 
 cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start,
@@ -950,21 +1324,9 @@ cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_
                              int t0, const __nv_bfloat16* q, cudaStream_t s, bool tables, int seg_unit) {
   cudaError_t e;
   if (theta_mode == 1) {
-    const long long N = (long long)m * (m + 1) / 2;
-    long long rank = (long long)floor((double)theta * (double)(N - 1));
-    if (rank < 0) rank = 0;
-    if (rank > N - 1) rank = N - 1;
-    // Few layers: 16 CTAs of 1024 threads share one, which gives every pair of rows a warp of its own (a cluster of 16
-    // needs a GPC to itself, so seven run at once).  More, or no GPC to be had: 8 CTAs of 512 threads.
-    if (layer_count <= c.theta_wide) {
-      auto fn = m <= 512 ? k_theta_select<17> : k_theta_select<33>;
-      e = launch_chained_cluster(fn, dim3(layer_count * 16), dim3(1024), 16, kThetaWideSmem, s, c, layer_begin, m, rank,
-                                 tables ? 1 : 0);
-    } else {
-      const int hsmem = (kThetaThreads / 32) * kThetaBins * (int)sizeof(unsigned);
-      e = launch_chained_cluster(k_theta_select<0>, dim3(layer_count * 8), dim3(kThetaThreads), 8, hsmem, s, c, layer_begin,
-                                 m, rank, tables ? 1 : 0);
-    }
+    const int hsmem = (kThetaThreads / 32) * kThetaBins * (int)sizeof(unsigned);
+    e = launch_chained_cluster(k_theta_select, dim3(layer_count * 8), dim3(kThetaThreads), 8, hsmem, s, c, layer_begin, m,
+                               quantile_rank(theta, m), tables ? 1 : 0);
   } else {
     e = launch_chained(k_theta_set, dim3(layer_count), dim3(1), 0, s, c, layer_begin, theta_q_abs,
                        (long long)nearbyint((double)theta * (double)kQScale), tables ? 1 : 0);
@@ -1939,8 +2301,8 @@ constexpr int kTopkStage = 48 * 1024;  // most order keys a prefill select keeps
 
 cudaError_t prepare_state() {
   cudaError_t e = cudaSuccess;
-  for (auto fn : {k_theta_select<17>, k_theta_select<33>})
-    e = first_error(e, first_error(allow_smem(fn, kThetaWideSmem),
+  for (auto fn : {k_segment<unsigned>, k_segment<unsigned long long>})
+    e = first_error(e, first_error(allow_smem(fn, -1),
                                    cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)));
   for (auto fn : {k_topk<false>, k_topk<true>}) e = first_error(e, allow_smem(fn, -1));
   // (48 KB of keys beside the static arrays: more than a kernel may use without asking)

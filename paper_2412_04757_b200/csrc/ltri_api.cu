@@ -198,6 +198,8 @@ size_t layout(const ltri_params& p, DevCtx& d, char* base, char** stage_out = nu
   d.Mq = cv.take<int>((size_t)d.NL * d.chunk * d.chunk);
   d.Rsuf = cv.take<long long>((size_t)d.NL * d.chunk * d.chunk);
   d.best = cv.take<long long>((size_t)d.NL * 2 * d.chunk);
+  d.seg_hist = cv.take<unsigned>((size_t)d.NL * kSegPasses << kSegHistBits);
+  d.seg_best = cv.take<long long>((size_t)d.NL * 2 * d.chunk);
   d.thetaq = cv.take<long long>(d.NL);
   d.rowstat = cv.take<float2>((size_t)d.NL * d.chunk * d.Hq);
   d.rowq = cv.take<float>((size_t)d.NL * d.chunk * d.Hq);
@@ -451,7 +453,7 @@ int ltri_create(const ltri_params* p, void* cuda_stream, ltri_ctx** out) {
   const int most = mc ? std::atoi(mc) : 16;
   if (ctx->dec_fused < 0 && !ctx->d.vote)
     for (int i = 1; i < 5 && 1 << i <= most; ++i) ctx->step_cap[i] = dec_step_capacity(ctx->d, 1 << i);
-  ctx->d.theta_wide = most >= 16 ? theta_wide_clusters() : 0;
+  ctx->d.seg_wide = most >= 16 ? segment_wide_clusters(ctx->d) : 0;
   ctx->d.item_cluster = 1;
   if (ctx->use_tc)
     for (int cl = 2; cl <= std::min(8, most) && attn_tc_cluster_runs(ctx->d, cl); cl *= 2) ctx->d.item_cluster = cl;
@@ -760,7 +762,11 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
       Scope sc(ctx, st, LTRI_K_MAP, ctx->use_tc ? 1 : ((a.t0 - a.loc_begin > 0 && a.loc_begin >= d.Ls) ? 2 : 1));
       LTRI_CUDA(ctx, ctx->use_tc ? launch_map_pass_tc(d, ag, ctx->kv_maps, st) : launch_map_pass(d, ag, st));
     }
-    if (m > 0) {
+    if (m > 0 && segment_in_one(d, ag.layer_count)) {
+      Scope sc(ctx, st, LTRI_K_SEGMENT, 1);
+      LTRI_CUDA(ctx, launch_segment_in_one(d, seq, ag.layer_begin, ag.layer_count, m, reg_start, slot, thq_abs, n_tokens, t0,
+                                           ag.q, st));
+    } else if (m > 0) {
       Scope sc(ctx, st, LTRI_K_SEGMENT, 4);
       LTRI_CUDA(ctx, launch_segment(d, seq, ag.layer_begin, ag.layer_count, m, reg_start, slot, d.theta_mode, d.theta,
                                     thq_abs, d.C, n_tokens, t0, ag.q, st, /*tables=*/true, d.seg_unit));
