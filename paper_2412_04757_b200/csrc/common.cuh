@@ -192,10 +192,11 @@ cudaError_t launch_evict_index(const DevCtx& c, const EvictArgs& a, int layer_co
 cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start, int slot,
                            int theta_mode, float theta, long long theta_q_abs, int max_spans, int n, int t0,
                            const __nv_bfloat16* q, cudaStream_t s, bool tables = false, int seg_unit = 0);
-// The same in one launch, for prefill calls of few layers.
+// The same in one launch, for prefill calls of few layers.  release: the kernel launched behind it starts at once and has to
+// wait for it at its end (see chain_release).
 bool segment_in_one(const DevCtx& c, int layer_count);
 cudaError_t launch_segment_in_one(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start, int slot,
-                                  long long theta_q_abs, int n, int t0, const __nv_bfloat16* q, cudaStream_t s);
+                                  long long theta_q_abs, int n, int t0, const __nv_bfloat16* q, bool release, cudaStream_t s);
 cudaError_t launch_score_prefill(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s);
 // tensor-core version of launch_score_prefill (split-bf16 representatives)
 cudaError_t launch_score_prefill_mma(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s);
@@ -222,7 +223,13 @@ cudaError_t launch_attn_prefill_tc(const DevCtx& c, const PrefillArgs& a, int ph
                                    cudaStream_t s);
 bool tc_attention_supported(const DevCtx& c);
 bool tc_encode_kv_maps(const DevCtx& c, void* out_bytes);
-cudaError_t launch_map_pass_tc(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, cudaStream_t s);
+// Which keys a launch of the map pass covers: all, those of the call itself (which the segmenter waits for), or those before
+// the call (whose votes nothing in the call reads).  late_wait: the kernel in front has released this one (see
+// chain_release), which waits for it at its end.
+enum MapPart { kMapAll, kMapOwn, kMapBefore };
+bool map_pass_splits(const DevCtx& c, const PrefillArgs& a);  // whether the second part is worth a launch of its own
+cudaError_t launch_map_pass_tc(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, MapPart part, bool late_wait,
+                               cudaStream_t s);
 // tcgen05 version of the prefill scores; returns cudaErrorNotSupported when the query-span count does not fit
 cudaError_t launch_score_prefill_tc(const DevCtx& c, const PrefillArgs& a, int span_bound, const void* kv_maps,
                                     cudaStream_t s);
@@ -254,10 +261,10 @@ cudaError_t launch_wait_probe(const DevCtx& c, long long short_limit, cudaStream
 // instead of 0.225 ms per step).  Launched the ordinary way, chain_wait() does nothing.
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Lets the kernel launched behind this one start now instead of when this grid has finished.  Used in one place only:
-// the eviction kernel (a few CTAs) releases the call's append kernel, which does not depend on it and whose threads
-// wait for the eviction kernel at their end instead of their beginning, so that the two run side by side and
-// everything behind the append kernel still follows both.
+// Lets the kernel launched behind this one start now instead of when this grid has finished.  Used where a kernel of a few
+// CTAs is followed by one that does not depend on it: the eviction kernel releases the call's append kernel, and the
+// one-launch segmenter the map pass over the keys before the call.  The released kernel waits for its predecessor at its
+// end instead of its beginning, so that the two run side by side and everything behind it still follows both.
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Dynamic shared memory that `fn` may ask for at a launch; bytes < 0: all that its static arrays leave of a block's limit.

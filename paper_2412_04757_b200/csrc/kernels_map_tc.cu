@@ -55,7 +55,13 @@ constexpr int kMapKT = 4;
 template <int G, bool FIT>
 __global__ void __launch_bounds__(kMapThreads, 1)
     k_map_tc(DevCtx c, PrefillArgs a, int n_local_groups, int n_local_tiles, int n_cur_tiles, int fit_tiles, int fit_splits,
-             const __grid_constant__ MapMaps maps) {
+             int late_wait, const __grid_constant__ MapMaps maps) {
+  // late_wait: the kernel in front of this one has released it (see chain_release): everything older is complete and visible,
+  // the two touch different data, and the last CTA waits for that kernel before it exits, so that whatever follows this one
+  // follows both.  (Only the last CTA: the grid is not complete before it is, and CTAs that sat waiting would keep the rest of
+  // the grid from starting.)
+  const bool holds_back =
+      late_wait && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1;
   extern __shared__ unsigned char smem_raw[];
   // KFULL[4] | QFULL[2] QEMPTY[2] | SFULL[4] SEMPTY[4]
   __shared__ __align__(8) unsigned long long bars[4 + 4 + 8];
@@ -70,7 +76,10 @@ __global__ void __launch_bounds__(kMapThreads, 1)
   int rh = -1;
   if (c.ret_head) {  // (a table in global memory, written once at ltri_create: older than any predecessor in the chain)
     rh = c.ret_head[layer];
-    if (rh >= 0 && g != rh / G) return;
+    if (rh >= 0 && g != rh / G) {
+      if (holds_back) chain_wait();
+      return;
+    }
   }
   const int group_tiles = FIT ? fit_tiles : kMapKT, splits = FIT ? fit_splits : 1;
   const int group = (int)blockIdx.x / splits, split = (int)blockIdx.x % splits;
@@ -85,7 +94,10 @@ __global__ void __launch_bounds__(kMapThreads, 1)
   const int all_blocks = (a.n + TPB - 1) / TPB, bfirst = blk0_of(0);
   const int per_split = (all_blocks - bfirst + splits - 1) / splits;
   const int bmin = bfirst + split * per_split, nblocks = min(all_blocks, bmin + per_split);
-  if (bmin >= nblocks) return;
+  if (bmin >= nblocks) {
+    if (holds_back) chain_wait();
+    return;
+  }
   int ntile = min(group_tiles, (is_cur ? n_cur_tiles : n_local_tiles) - tile0);
   while (ntile > 1 && blk0_of(ntile - 1) >= nblocks) --ntile;
 
@@ -130,7 +142,7 @@ __global__ void __launch_bounds__(kMapThreads, 1)
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = s_tmem_base;
-  chain_wait();  // everything above set up shared memory, barriers and TMEM only
+  if (!late_wait) chain_wait();  // everything above set up shared memory, barriers and TMEM only
 
   if (warp == 16) {
     // Every key tile has its own barrier, and the first one is asked for before anything else, the others behind the
@@ -352,6 +364,7 @@ __global__ void __launch_bounds__(kMapThreads, 1)
   fence_after_sync();
   if (warp == 16) tmem_dealloc(tmem, 512);
   if (tid == 0 && s_abort) set_status(c, -6, 5000 + (int)blockIdx.x);
+  if (holds_back) chain_wait();
 }
 
 typedef CUresult (*EncodeFnM)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -361,7 +374,8 @@ typedef CUresult (*EncodeFnM)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
 constexpr int kMapSmem = kMapKT * 32768 + 65536 + 3 * 4096 + 1024;  // key tiles, two query stages, the offset tiles
 
 template <int G>
-static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, cudaStream_t s) {
+static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, MapPart part, bool late_wait,
+                                   cudaStream_t s) {
   static EncodeFnM enc = nullptr;
   if (!enc) {
     void* p = nullptr;
@@ -383,27 +397,33 @@ static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const 
     return cudaErrorInvalidValue;
   // (the region maps, which the kernel accumulates into with integer reductions, were cleared by the call's append
   // kernel)
-  const int nloc = (a.loc_begin >= c.Ls) ? (a.t0 - a.loc_begin + 127) / 128 : 0;
-  const int ncur = (a.n + 127) / 128;
+  const int nloc = part != kMapOwn && a.loc_begin >= c.Ls ? (a.t0 - a.loc_begin + 127) / 128 : 0;
+  const int ncur = part != kMapBefore ? (a.n + 127) / 128 : 0;
   // Key tiles per CTA and splits of the query blocks.  With enough CTAs for several waves: four tiles, no split (the
-  // queries are re-read least).  Otherwise the pair that finishes first by a small model, in units of one product of a key
-  // tile with a query block; a CTA starts and ends in six of them.  One layer, 36 tiles, 8 KV heads: 72 CTAs of four tiles
-  // took 57 us, 144 CTAs of four tiles and half the blocks take 43.  The model ranks, it does not predict: against the best
-  // of the sixteen pairs, over 1 to 16 layers and 1 to 8 query heads per KV head, its choice is within 14% for calls of up to
-  // 512 tokens and up to 36% behind for 1024 tokens over a full window (one layer of 32 heads: 104 us against 80 with three
-  // tiles and four splits; 127 unsplit).  The map and the votes are integer sums, so the results do not depend on the choice.
+  // queries are re-read least).  Otherwise the pair that finishes first by a model of the launch in tenths of a microsecond: a
+  // CTA starts and ends in 45 and takes 6.6 for a product of a key tile with a query block (a CTA of four tiles and 16 blocks
+  // lives 45 us); beside the segmenter its 16 SMs per layer join in when it is through.  The map and the votes are integer
+  // sums, so the results do not depend on the choice.
   const int nblk = (a.n + 128 / G - 1) / (128 / G);
   int kt = kMapKT, qs = 1;
   const int heads = c.Hkv * a.layer_count;
   auto ctas_of = [&](int k, int q) { return ((nloc + k - 1) / k + (ncur + k - 1) / k) * q * heads; };
-  if (ctas_of(kMapKT, 1) <= 3 * c.sms) {
-    long long best = -1;
+  const bool beside = part == kMapBefore;
+  if (ctas_of(kMapKT, 1) <= (beside ? 6 : 3) * c.sms) {
+    const int late = beside ? min(kSegSms * a.layer_count, c.sms - 1) : 0, now = c.sms - late;
+    const int from = 150 + a.n * 2 / 5;  // when the segmenter is through (about 35 us for 512 tokens)
+    int best = 0;
     for (int k = kMapKT; k >= 1; --k)
-      for (int q = 1; q <= 8 && q <= nblk; q *= 2) {
-        const long long waves = (ctas_of(k, q) + c.sms - 1) / c.sms;
-        const long long cost = waves * (6 + k * ((nblk + q - 1) / q));
-        if (best < 0 || cost < best) {
-          best = cost;
+      for (int q = 1; q <= 8 && q <= nblk; ++q) {
+        const int n = ctas_of(k, q), d = 45 + (66 * k * ((nblk + q - 1) / q) + 9) / 10;
+        // the first moment at which `now` CTAs at a time since the start and `late` at a time since `from` come to n
+        int t = (n + now - 1) / now * d;
+        for (int w = 1; late > 0 && from + w * d < t; ++w)
+          if ((from + w * d) / d * now + w * late >= n) t = from + w * d;
+        for (int w = 1; late > 0 && w * d < t; ++w)
+          if (w * now + max(w * d - from, 0) / d * late >= n) t = w * d;
+        if (best == 0 || t < best) {
+          best = t;
           kt = k;
           qs = q;
         }
@@ -412,7 +432,7 @@ static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const 
   const int gloc = (nloc + kt - 1) / kt, gcur = (ncur + kt - 1) / kt;
   return launch_chained(kt < kMapKT || qs > 1 ? k_map_tc<G, true> : k_map_tc<G, false>,
                         dim3((gloc + gcur) * qs, c.Hkv, a.layer_count), dim3(kMapThreads), kMapSmem, s, c, a, gloc, nloc, ncur,
-                        kt, qs, maps);
+                        kt, qs, late_wait ? 1 : 0, maps);
 }
 
 template <int G>
@@ -430,12 +450,21 @@ cudaError_t prepare_map_tc(const DevCtx& c) {
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_map_pass_tc(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, cudaStream_t s) {
+// The keys before the call take four products of a key tile with a query block per SM, or more.  (256 tokens over 576 of one
+// layer with two KV heads, 80 products: 803 us a request of eight calls in one launch, 813 in two; 512 tokens over 1024 with
+// eight, 1024 products: 5 us a call gained.)
+bool map_pass_splits(const DevCtx& c, const PrefillArgs& a) {
+  const long long tiles = (a.t0 - a.loc_begin + 127) / 128, blocks = ((long long)a.n * c.G + 127) / 128;
+  return tiles * blocks * c.Hkv * a.layer_count >= 4ll * c.sms;
+}
+
+cudaError_t launch_map_pass_tc(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, MapPart part, bool late_wait,
+                                   cudaStream_t s) {
   switch (c.G) {
-    case 1: return launch_map_tc_g<1>(c, a, kv_maps, s);
-    case 2: return launch_map_tc_g<2>(c, a, kv_maps, s);
-    case 4: return launch_map_tc_g<4>(c, a, kv_maps, s);
-    case 8: return launch_map_tc_g<8>(c, a, kv_maps, s);
+    case 1: return launch_map_tc_g<1>(c, a, kv_maps, part, late_wait, s);
+    case 2: return launch_map_tc_g<2>(c, a, kv_maps, part, late_wait, s);
+    case 4: return launch_map_tc_g<4>(c, a, kv_maps, part, late_wait, s);
+    case 8: return launch_map_tc_g<8>(c, a, kv_maps, part, late_wait, s);
   }
   return cudaErrorInvalidValue;
 }

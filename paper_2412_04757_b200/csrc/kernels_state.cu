@@ -1000,6 +1000,7 @@ struct SegArgs {
   NmsArgs nms;
   int theta_mode;         // 1: quantile (of rank `rank`), otherwise the threshold is given
   int bh;                 // rows of a block: m / 32, rounded up
+  int release;            // lets the kernel launched behind this one start at once
   long long rank, thq, thq1;
 };
 
@@ -1021,6 +1022,7 @@ static size_t seg_smem(int m, int bh) {  // (two row strides, each rounded up by
 template <typename PT>
 __global__ void __launch_bounds__(kSegThreads, 1) k_segment(DevCtx c, SegArgs a) {
   chain_wait();
+  if (a.release) chain_release();
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   const int part = (int)cluster.block_rank(), lidx = blockIdx.x / kSegCluster, layer = a.nms.layer_begin + lidx;
@@ -1307,11 +1309,12 @@ int segment_wide_clusters(const DevCtx& c) {
 bool segment_in_one(const DevCtx& c, int layer_count) { return layer_count <= c.seg_wide; }
 
 cudaError_t launch_segment_in_one(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start, int slot,
-                                  long long theta_q_abs, int n, int t0, const __nv_bfloat16* q, cudaStream_t s) {
+                                  long long theta_q_abs, int n, int t0, const __nv_bfloat16* q, bool release, cudaStream_t s) {
   SegArgs a;
   a.nms = NmsArgs{seq, layer_begin, m, reg_start, slot, c.C, n, t0, q, 1, c.seg_unit};
   a.theta_mode = c.theta_mode;
   a.bh = (m + kSegBlocks - 1) / kSegBlocks;
+  a.release = release ? 1 : 0;
   a.rank = quantile_rank(c.theta, m);
   a.thq = theta_q_abs;
   a.thq1 = (long long)nearbyint((double)c.theta * (double)kQScale);

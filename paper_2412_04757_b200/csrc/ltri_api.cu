@@ -757,15 +757,27 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
       LTRI_CUDA(ctx, ctx->use_tc ? launch_attn_prefill_tc(d, ag, 0, !has_index, ctx->kv_maps, st)
                                  : launch_attn_prefill(d, ag, 0, !has_index, st));
     }
+    // Few layers: the segmenter is one launch of 16 CTAs per layer that needs the map of the call's own keys only, so that
+    // part of the map pass goes first and the rest, most of it, runs beside the segmenter on the other SMs.
+    const bool before = a.loc_begin >= d.Ls && a.t0 > a.loc_begin;  // keys before the call are voted for
+    const bool seg_one = m > 0 && segment_in_one(d, ag.layer_count);
+    const bool own_first = seg_one && ctx->use_tc && before && map_pass_splits(d, ag);
     {
       // (the tensor-core pass is one kernel; the warp-MMA fallback has one for the local keys and one for the call's own)
-      Scope sc(ctx, st, LTRI_K_MAP, ctx->use_tc ? 1 : ((a.t0 - a.loc_begin > 0 && a.loc_begin >= d.Ls) ? 2 : 1));
-      LTRI_CUDA(ctx, ctx->use_tc ? launch_map_pass_tc(d, ag, ctx->kv_maps, st) : launch_map_pass(d, ag, st));
+      Scope sc(ctx, st, LTRI_K_MAP, ctx->use_tc || !before ? 1 : 2);
+      LTRI_CUDA(ctx, ctx->use_tc ? launch_map_pass_tc(d, ag, ctx->kv_maps, own_first ? kMapOwn : kMapAll, false, st)
+                                 : launch_map_pass(d, ag, st));
     }
-    if (m > 0 && segment_in_one(d, ag.layer_count)) {
-      Scope sc(ctx, st, LTRI_K_SEGMENT, 1);
-      LTRI_CUDA(ctx, launch_segment_in_one(d, seq, ag.layer_begin, ag.layer_count, m, reg_start, slot, thq_abs, n_tokens, t0,
-                                           ag.q, st));
+    if (seg_one) {
+      {
+        Scope sc(ctx, st, LTRI_K_SEGMENT, 1);
+        LTRI_CUDA(ctx, launch_segment_in_one(d, seq, ag.layer_begin, ag.layer_count, m, reg_start, slot, thq_abs, n_tokens,
+                                             t0, ag.q, own_first, st));
+      }
+      if (own_first) {
+        Scope sc(ctx, st, LTRI_K_MAP, 1);
+        LTRI_CUDA(ctx, launch_map_pass_tc(d, ag, ctx->kv_maps, kMapBefore, true, st));
+      }
     } else if (m > 0) {
       Scope sc(ctx, st, LTRI_K_SEGMENT, 4);
       LTRI_CUDA(ctx, launch_segment(d, seq, ag.layer_begin, ag.layer_count, m, reg_start, slot, d.theta_mode, d.theta,
