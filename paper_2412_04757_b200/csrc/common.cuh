@@ -150,7 +150,7 @@ struct EvictArgs {
   int nslots;
   int slot[8];
   long long shift;  // sliding slabs: token - shift = row
-  int release;      // let the kernel launched behind this one (the call's append kernel) start at once
+  int release;      // let the kernel launched behind this one (the call's map pass) start at once
 };
 
 struct PrefillArgs {
@@ -183,7 +183,7 @@ cudaError_t prepare_state();
 cudaError_t prepare_decode(const DevCtx& c);
 cudaError_t prepare_dec_step(const DevCtx& c);
 cudaError_t launch_init(const DevCtx& c, int seq /* -1: all */, cudaStream_t s);
-cudaError_t launch_append_prefill(const DevCtx& c, const PrefillArgs& a, bool clear_maps, bool late_wait, cudaStream_t s);
+cudaError_t launch_append_prefill(const DevCtx& c, const PrefillArgs& a, bool clear_maps, cudaStream_t s);
 cudaError_t launch_append_decode(const DevCtx& c, const DecBatch& b, int layer_begin, int layer_count, int n_seqs_total,
                                  const __nv_bfloat16* k, const __nv_bfloat16* v, cudaStream_t s);
 cudaError_t launch_evict_index(const DevCtx& c, const EvictArgs& a, int layer_count, cudaStream_t s);
@@ -262,8 +262,8 @@ cudaError_t launch_wait_probe(const DevCtx& c, long long short_limit, cudaStream
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the kernel launched behind this one start now instead of when this grid has finished.  Used where a kernel of a few
-// CTAs is followed by one that does not depend on it: the eviction kernel releases the call's append kernel, and the
-// one-launch segmenter the map pass over the keys before the call.  The released kernel waits for its predecessor at its
+// CTAs is followed by one that does not depend on it: the eviction kernel releases the call's map pass, and the one-launch
+// segmenter the map pass over the keys before the call.  The released kernel waits for its predecessor at its
 // end instead of its beginning, so that the two run side by side and everything behind it still follows both.
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

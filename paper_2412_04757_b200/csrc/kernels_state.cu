@@ -58,11 +58,8 @@ cudaError_t launch_init(const DevCtx& c, int seq, cudaStream_t s) {
 // (zero_vec of them, 16 bytes each) clear the region maps of the call's layers, which the tensor-core map pass
 // accumulates into with integer reductions: nothing reads a layer's map between the segmenter of the layer's previous
 // call and that pass, so clearing it here, in the first kernel of the call, keeps a memset out of the kernel chain.
-__global__ void k_append_prefill(DevCtx c, PrefillArgs a, unsigned long long zero_vec, int late_wait) {
-  // late_wait: the kernel in front of this one is the call's eviction kernel, which has released this one (see
-  // chain_release): everything older is complete and visible, the two kernels touch different data, and this one
-  // waits for the eviction kernel at its end (in its last CTA), so that whatever follows it follows both.
-  if (!late_wait) chain_wait();
+__global__ void k_append_prefill(DevCtx c, PrefillArgs a, unsigned long long zero_vec) {
+  chain_wait();
   const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int c16 = gid & 15;
   size_t row = gid >> 4;  // over [layer_count][n][Hkv]
@@ -94,17 +91,12 @@ __global__ void k_append_prefill(DevCtx c, PrefillArgs a, unsigned long long zer
       if (g == 0 && c16 == 0) c.votes[unit * c.Tpad + a.t0 + r] = 0;
     }
   }
-  // (only the last CTA waits: the grid is not complete before it is, and CTAs that sat waiting in every slot of an SM
-  // would keep the rest of the grid from starting)
-  if (late_wait && blockIdx.x == gridDim.x - 1) chain_wait();
 }
 
-cudaError_t launch_append_prefill(const DevCtx& c, const PrefillArgs& a, bool clear_maps, bool late_wait,
-                                  cudaStream_t s) {
+cudaError_t launch_append_prefill(const DevCtx& c, const PrefillArgs& a, bool clear_maps, cudaStream_t s) {
   const unsigned long long zero_vec = clear_maps ? (unsigned long long)a.layer_count * c.chunk * c.chunk / 4 : 0ull;
   const size_t threads = (size_t)a.layer_count * a.n * c.Hkv * 16 + zero_vec;
-  return launch_chained(k_append_prefill, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, s, c, a, zero_vec,
-                        late_wait ? 1 : 0);
+  return launch_chained(k_append_prefill, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, s, c, a, zero_vec);
 }
 
 __global__ void k_append_decode(DevCtx c, DecBatch b, int layer_begin, int layer_count,

@@ -692,23 +692,23 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
   }
   const long long shift = d.paged ? s0.base - d.Lsp : 0;
   a.shift = shift;
-  // The eviction kernel (eight small CTAs per layer) goes first and releases the append kernel behind it at once: the two
-  // touch different data and run side by side; the append kernel waits for the eviction kernel at its end.  They are
-  // timed together (class LTRI_K_EVICT); a call that evicts nothing times its append kernel alone (LTRI_K_APPEND).
-  {
-    const int n_ev = (int)((ev.size() + 7) / 8);
-    Scope sc(ctx, st, n_ev > 0 ? LTRI_K_EVICT : LTRI_K_APPEND, n_ev + 1);
+  auto evict = [&](int lb, int layers, bool release) -> cudaError_t {
     for (size_t i = 0; i < ev.size(); i += 8) {
       EvictArgs ea;
       ea.seq = seq;
       ea.shift = shift;
-      ea.layer_begin = layer_begin;
+      ea.layer_begin = lb;
       ea.nslots = (int)std::min<size_t>(8, ev.size() - i);
-      ea.release = i + 8 >= ev.size() ? 1 : 0;
+      ea.release = release && i + 8 >= ev.size() ? 1 : 0;
       for (int j = 0; j < ea.nslots; ++j) ea.slot[j] = ev[i + j].slot;
-      LTRI_CUDA(ctx, launch_evict_index(d, ea, layer_count, st));
+      if (const cudaError_t e = launch_evict_index(d, ea, layers, st); e != cudaSuccess) return e;
     }
-    LTRI_CUDA(ctx, launch_append_prefill(d, a, /*clear_maps=*/ctx->use_tc, /*late_wait=*/n_ev > 0, st));
+    return cudaSuccess;
+  };
+  const int n_ev = (int)((ev.size() + 7) / 8);
+  {
+    Scope sc(ctx, st, LTRI_K_APPEND, 1);
+    LTRI_CUDA(ctx, launch_append_prefill(d, a, /*clear_maps=*/ctx->use_tc, st));
   }
   if (d.host_kv && !ev.empty()) {
     // mirror the rows that just left the window to the host: one strided copy for K and one for V per region (the
@@ -762,10 +762,17 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
     const bool before = a.loc_begin >= d.Ls && a.t0 > a.loc_begin;  // keys before the call are voted for
     const bool seg_one = m > 0 && segment_in_one(d, ag.layer_count);
     const bool own_first = seg_one && ctx->use_tc && before && map_pass_splits(d, ag);
+    // The spans that leave the window are indexed before the scores are taken, no sooner: the eviction kernel (eight small
+    // CTAs per layer, 7 us in front of the attention otherwise) goes in front of the map pass and releases it at once; the two
+    // touch different data and run side by side, and the map pass waits for the eviction kernel at its end.
+    if (n_ev > 0) {
+      Scope sc(ctx, st, LTRI_K_EVICT, n_ev);
+      LTRI_CUDA(ctx, evict(ag.layer_begin, ag.layer_count, ctx->use_tc));
+    }
     {
       // (the tensor-core pass is one kernel; the warp-MMA fallback has one for the local keys and one for the call's own)
       Scope sc(ctx, st, LTRI_K_MAP, ctx->use_tc || !before ? 1 : 2);
-      LTRI_CUDA(ctx, ctx->use_tc ? launch_map_pass_tc(d, ag, ctx->kv_maps, own_first ? kMapOwn : kMapAll, false, st)
+      LTRI_CUDA(ctx, ctx->use_tc ? launch_map_pass_tc(d, ag, ctx->kv_maps, own_first ? kMapOwn : kMapAll, n_ev > 0, st)
                                  : launch_map_pass(d, ag, st));
     }
     if (seg_one) {
