@@ -28,15 +28,15 @@ constexpr int kStWarps = kStThreads / 32;
 constexpr int kStTileBytes = 2 * kDTile * 256;  // K and V rows of a 16-token tile
 constexpr int kStRing = kStWarps * kStTileBytes;
 constexpr int kStMaxCluster = 16;
-constexpr int kStList = 512;          // candidates of a cluster: room for kStList / S per CTA
+constexpr int kStList = 1024;         // candidates of a cluster: room for kStList / S per CTA
 constexpr int kStCand = kStThreads;   // candidates ranked against each other, one per thread
 constexpr int kStAhead = 4;           // batches of index rows requested ahead of the scan
 constexpr int kStMaxSlots = 5120;     // order keys a CTA can keep (20 KB)
 static_assert(kStRing >= (int)(kStWarps * 8 * (kD + 2) * sizeof(float)), "the warps' partials reuse the ring");
-static_assert(kStMaxCluster * kMaxTopK * 8 <= kStList * 16, "the lists of the general select reuse the candidates'");
+static_assert(kStMaxCluster * kMaxTopK <= kStList, "the lists of the general select reuse the candidates'");
 
 // dynamic shared memory: K/V ring | candidates | order keys
-static int dec_step_smem(int key_slots) { return kStRing + kStList * 16 + key_slots * 4; }
+static int dec_step_smem(int key_slots) { return kStRing + kStList * 8 + key_slots * 4; }
 
 template <int G>
 __global__ void __launch_bounds__(kStThreads, 2)
@@ -44,12 +44,14 @@ __global__ void __launch_bounds__(kStThreads, 2)
                const __nv_bfloat16* __restrict__ knew, const __nv_bfloat16* __restrict__ vnew,
                __nv_bfloat16* __restrict__ out, int key_slots) {
   extern __shared__ __align__(1024) unsigned char dsm[];
-  int4* s_list = reinterpret_cast<int4*>(dsm + kStRing);  // [S][kStList / S] (key, id, start, length) of the candidates
+  // [S][kStList / S] (key, id) of the candidates, larger key first, then lower id: one descending order
+  unsigned long long* s_list = reinterpret_cast<unsigned long long*>(dsm + kStRing);
   unsigned* g_key = reinterpret_cast<unsigned*>(s_list);  // general select: the cluster's lists, keys then ids
   int* g_id = reinterpret_cast<int*>(g_key + kStMaxCluster * kMaxTopK);
-  unsigned* sck = reinterpret_cast<unsigned*>(dsm + kStRing + kStList * 16);  // [key_slots] this CTA's order keys
+  unsigned* sck = reinterpret_cast<unsigned*>(dsm + kStRing + kStList * 8);  // [key_slots] this CTA's order keys
   __shared__ float su[kD];
   __shared__ unsigned hist[256];
+  __shared__ unsigned r_hist[256];  // added up by the CTAs of the cluster: the histogram over all their keys
   __shared__ unsigned s_prefix, s_need;
   __shared__ int s_ids[kMaxTopK], s_cnt, s_cut;
   __shared__ int s_scan[64 + kSelCand];
@@ -93,35 +95,40 @@ __global__ void __launch_bounds__(kStThreads, 2)
   const __nv_bfloat16* Vslab = c.Vc + (unit * c.Hkv + g) * (size_t)c.SR * kD;
   const uint32_t sk = smem_u32(dsm) + warp * kStTileBytes, sv = sk + kDTile * 256;  // this warp's tile: K rows, V rows
   const int ch = lane & 15;
-  // this lane copies rows (lane >> 4) + 2i of a tile, 16 bytes at chunk ch; the new token's row comes from the
-  // caller's tensors (its copy in the cache is written by another CTA of the cluster)
-  auto issue_a = [&](int t, bool values) {
-    const __nv_bfloat16* slab = values ? Vslab : Kslab;
-    const __nv_bfloat16* fresh = (values ? vnew : knew) + nrow * kD;
-    const uint32_t dst = values ? sv : sk;
+  // A tile is copied in two steps: every lane finds the row of one of its tokens (lane & 15), then copies 16 bytes at chunk ch
+  // of the rows (lane >> 4) + 2i, whose numbers it gets from the lanes that found them.  (A kernel this short fetches each of
+  // its instructions once, at some ten cycles apiece, so what counts on the way is their number: with every lane working out
+  // eight addresses for the keys and eight for the values at each place, requesting a tile took 3K cycles.)
+  constexpr int kNoRow = -1, kNewRow = -2;  // the new token's row comes from the caller's tensors: another CTA stores it
+  auto known_row = [&](int t) {
+    const int v = tA0 + t * kDTile + ch, tok = v < a0 ? v : rb + (v - a0);
+    return v >= tA1 ? kNoRow : tok == pos ? kNewRow : (int)slab_row(c, tok, b.shift[bi]);
+  };
+  auto copy_rows = [&](int rows, const __nv_bfloat16* base, const __nv_bfloat16* fresh, uint32_t dst) {
 #pragma unroll
     for (int i = 0; i < kDTile / 2; ++i) {
-      const int row = 2 * i + (lane >> 4);
-      const int v = tA0 + t * kDTile + row;
-      const bool ok = v < tA1;
-      const int tok = ok ? (v < a0 ? v : rb + (v - a0)) : 0;
-      const __nv_bfloat16* src = ok && tok == pos ? fresh : slab + (size_t)slab_row(c, tok, b.shift[bi]) * kD;
-      cp_async16(dst + tile_off(row, ch), src + ch * 8, ok ? 16 : 0);
+      const int row = 2 * i + (lane >> 4), r = __shfl_sync(0xffffffffu, rows, row);
+      const __nv_bfloat16* src = r == kNewRow ? fresh : base + (size_t)max(r, 0) * kD;
+      cp_async16(dst + tile_off(row, ch), src + ch * 8, r == kNoRow ? 0 : 16);
     }
   };
   const bool early = warp < ntA;  // this warp's first tile is requested before the retrieval
   if (early) {
-    issue_a(warp, false);
-    cp_async_commit();
-    issue_a(warp, true);
-    cp_async_commit();
+    const int rows = known_row(warp);
+#pragma unroll 1
+    for (int kv = 0; kv < 2; ++kv) {
+      copy_rows(rows, kv ? Vslab : Kslab, (kv ? vnew : knew) + nrow * kD, kv ? sv : sk);
+      cp_async_commit();
+    }
   }
-  if (rank == 0) append_decode_row(c, b, bi, l, layer_count, unit, g, knew, vnew);
+  // the new token's rows go to the cache at the end: their load is not waited for on the way (by the CTA with the fewest tokens)
+  const bool appends = rank == S - 1 && warp == kStWarps - 1;
+  uint4 new_row = make_uint4(0u, 0u, 0u, 0u);
+  if (appends) new_row = *reinterpret_cast<const uint4*>((lane < 16 ? knew : vnew) + nrow * kD + ch * 8);
 
   // ---- retrieval
   int nall = 0;
   const int* ids_all = s_ids;
-  bool extents = false;  // s_sst / s_sln already hold the selected spans' extents
   uint32_t qa[8][2];     // query fragments: rows 0..G-1 of the 16-row A operand are the heads of the group
   const int r = lane >> 2, qd = lane & 3;
   auto load_q = [&]() {
@@ -175,6 +182,7 @@ __global__ void __launch_bounds__(kStThreads, 2)
     }
     if (tid == 0) s_cnt = 0;
     hist[tid] = 0;
+    r_hist[tid] = 0;
     __syncthreads();
     unsigned kmax = 0u;
     {
@@ -266,7 +274,7 @@ __global__ void __launch_bounds__(kStThreads, 2)
     if (U == 0) {
       const int K = min(c.topk, nsp);
       const int cap = kStList / S;
-      unsigned bcut = 0xffffu, M16 = 0xffffu;  // (K == nsp: every span is a candidate)
+      unsigned bcut = 255u, M16 = 0xffffu;  // (K == nsp: every span is a candidate)
       bool general = false;
       if (K < nsp) {
         if (tid < S) {
@@ -279,17 +287,18 @@ __global__ void __launch_bounds__(kStThreads, 2)
         unsigned m = 0u;
         for (int t = 0; t < S; ++t) m = max(m, r_max[t]);
         M16 = m >> 16;
-        // how far the upper 16 bits of the keys lie below those of the largest; only the nearest 255 steps count
+        // how far the upper 16 bits of the keys lie below those of the largest (dist_bin), counted here and added to every
+        // CTA's total; few bins hold anything
         for (int s = tid; s < nloc; s += nt) {
-          const unsigned dist = M16 - (sck[s] >> 16);
-          if (dist < 255u) atomicAdd(&hist[dist], 1u);
+          const unsigned d = dist_bin(M16 - (sck[s] >> 16));
+          if (d < 255u) atomicAdd(&hist[d], 1u);
         }
         if (tid == 0) s_cut = 255;
+        __syncthreads();
+        if (const unsigned n = hist[tid])
+          for (int t = 0; t < S; ++t) atomicAdd(cluster.map_shared_rank(&r_hist[tid], t), n);
         cluster.sync();
-        unsigned tot = 0;
-#pragma unroll
-        for (int t = 0; t < kStMaxCluster; ++t)
-          if (t < S) tot += cluster.map_shared_rank(hist, t)[tid];
+        const unsigned tot = r_hist[tid];
         // the first bin at which the running count reaches K
         unsigned inc = tot;
 #pragma unroll
@@ -306,14 +315,14 @@ __global__ void __launch_bounds__(kStThreads, 2)
         general = bcut >= 255u;  // the K-th key lies further below (the same decision in every CTA)
       }
       if (!general) {
-        // the candidates go to every CTA of the cluster, with their extents
+        // the candidates go to every CTA of the cluster
+        const unsigned dcut = dist_last(bcut);
         for (int s = tid; s < nloc; s += nt) {
           const unsigned key = sck[s];
-          if (M16 - (key >> 16) <= bcut) {
+          if (M16 - (key >> 16) <= dcut) {
             const int j = atomicAdd(&s_cnt, 1);
             if (j < cap) {
-              const int4 e = make_int4((int)key, lo + s, c.span_start[unit * c.cap + lo + s],
-                                       c.span_len[unit * c.cap + lo + s]);
+              const unsigned long long e = ((unsigned long long)key << 32) | (unsigned)~(lo + s);
               for (int t = 0; t < S; ++t) cluster.map_shared_rank(s_list, t)[rank * cap + j] = e;
             }
           }
@@ -329,36 +338,27 @@ __global__ void __launch_bounds__(kStThreads, 2)
         }
         general = most > cap || nc > kStCand;  // many equal scores
         if (!general) {
-          for (int i = tid; i < S * cap; i += nt) {
-            const int t = i / cap, j = i - t * cap;
-            if (j < r_cnt[t]) {
-              int at = j;
-              for (int w = 0; w < t; ++w) at += r_cnt[w];
-              const int4 e = s_list[i];
-              // larger key first, then lower id: one descending order; the list position rides along
-              s_rank[at] = ((unsigned long long)(unsigned)e.x << 32) | (unsigned)(~e.y);
-              s_ckey[at] = (unsigned)i;
-            }
+          for (int t = warp; t < S; t += kStWarps) {  // the lists behind each other
+            int at = 0;
+            for (int w = 0; w < t; ++w) at += r_cnt[w];
+            for (int j = lane; j < r_cnt[t]; j += 32) s_rank[at + j] = s_list[t * cap + j];
           }
           __syncthreads();
           int rk = 0x7fffffff;
-          int4 e = make_int4(0, 0, 0, 0);
+          unsigned long long mine = 0;
           if (tid < nc) {
-            const unsigned long long mine = s_rank[tid];
-            e = s_list[s_ckey[tid]];
+            mine = s_rank[tid];
             rk = 0;
             for (int i = 0; i < nc; ++i) rk += s_rank[i] > mine;
-            if (rk < K) s_scan[rk] = e.y;
           }
+          const int id = (int)~(unsigned)mine;
+          if (rk < K) s_scan[rk] = id;
           __syncthreads();
           if (rk < K) {
             int at = 0;
-            for (int i = 0; i < K; ++i) at += s_scan[i] < e.y;
-            s_ids[at] = e.y;
-            s_sst[at] = e.z;
-            s_sln[at] = e.w;
+            for (int i = 0; i < K; ++i) at += s_scan[i] < id;
+            s_ids[at] = id;
           }
-          extents = true;
           cnt = K;
         }
       }
@@ -423,16 +423,15 @@ __global__ void __launch_bounds__(kStThreads, 2)
     }
     __syncthreads();
     nall = cnt;
-    if (rank == 0) {
+    if (rank == S - 1) {
       int* sel = c.sel + (unit * c.Hkv + g) * (size_t)c.topk;
       for (int t = tid; t < c.topk; t += nt) sel[t] = t < cnt ? s_ids[t] : -1;
     }
     if (c.persist) {
       nall = union_with_persistent(c, unit, g, s_ids, cnt, s_scan, s_all, &s_nall);
       ids_all = s_all;
-      extents = false;
     }
-    if (tid < nall && !extents) {
+    if (tid < nall) {
       if (U > 0) {  // the unit's tokens inside the indexed range
         const int st = max(ids_all[tid] * U, c.Ls);
         s_sst[tid] = st;
@@ -444,7 +443,7 @@ __global__ void __launch_bounds__(kStThreads, 2)
     }
   } else {
     load_q();
-    if (rank == 0) {
+    if (rank == S - 1) {
       int* sel = c.sel + (unit * c.Hkv + g) * (size_t)c.topk;
       for (int t = tid; t < c.topk; t += nt) sel[t] = -1;
     }
@@ -466,9 +465,11 @@ __global__ void __launch_bounds__(kStThreads, 2)
     cluster.sync();  // (orders the pulled rows before the cluster's reads)
   }
   // ranges of the selected tokens and the prefix of their lengths
-  if (warp == 0) {
+  if (nall == 0) {  // (the same in every CTA)
+    if (tid == 0) s_rp[0] = s_nr = 0;
+  } else if (warp == 0) {
     int nr = nall;
-    if (U == 0 && (c.phi_milli > 0 || c.phi_l) && nall > 0) {  // kept spans may overlap: every token once
+    if (U == 0 && (c.phi_milli > 0 || c.phi_l)) {  // kept spans may overlap: every token once
       nr = merge_ranges_warp(
           nall,
           [&](int i, int& st, int& ln) {
@@ -502,13 +503,13 @@ __global__ void __launch_bounds__(kStThreads, 2)
       s_rp[nr] = run;
       s_nr = nr;
     }
-    if (rank == 0) {
-      long long tokens = 0;
-      for (int t = lane; t < nall; t += 32) tokens += s_sln[t];
+  }
+  if (rank == S - 1 && warp == 1) {
+    long long tokens = 0;
+    for (int t = lane; t < nall; t += 32) tokens += s_sln[t];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) tokens += shfl_xor_ll(tokens, o);
-      if (lane == 0) c.sel_tokens[unit * c.Hkv + g] = tokens;  // (summed over the KV heads by ltri_get_stats)
-    }
+    for (int o = 16; o > 0; o >>= 1) tokens += shfl_xor_ll(tokens, o);
+    if (lane == 0) c.sel_tokens[unit * c.Hkv + g] = tokens;  // (summed over the KV heads by ltri_get_stats)
   }
   __syncthreads();
 
@@ -518,40 +519,28 @@ __global__ void __launch_bounds__(kStThreads, 2)
   const int ntiles = ntA + (tB1 - tB0 + kDTile - 1) / kDTile;
   const __nv_bfloat16* Ksel = c.host_kv ? c.Kcache : Kslab;  // what the ranges' rows are counted from
   const __nv_bfloat16* Vsel = c.host_kv ? c.Vcache : Vslab;
-  int rik = 0, riv = 0;  // ranges of this lane's last K and V row (a warp's tiles ascend)
-  auto issue = [&](int t, bool values) {
-    if (t < ntA) {
-      issue_a(t, values);
-      return;
-    }
-    const uint32_t dst = values ? sv : sk;
-    const __nv_bfloat16* base = values ? Vsel : Ksel;
-    int ri = values ? riv : rik;
-#pragma unroll
-    for (int i = 0; i < kDTile / 2; ++i) {
-      const int row = 2 * i + (lane >> 4);
-      const int v = tB0 + (t - ntA) * kDTile + row;
-      const bool ok = v < tB1;
-      size_t tok = 0;
-      if (ok) {
-        while (v >= s_rp[ri + 1]) ++ri;
-        tok = (size_t)(s_rs[ri] + (v - s_rp[ri]));
-      }
-      cp_async16(dst + tile_off(row, ch), base + tok * kD + ch * 8, ok ? 16 : 0);
-    }
-    if (values)
-      riv = ri;
-    else
-      rik = ri;
+  int ri = 0;  // range of this lane's last row (a warp's tiles ascend)
+  auto any_row = [&](int t) {
+    if (t < ntA) return known_row(t);
+    const int v = tB0 + (t - ntA) * kDTile + ch;
+    if (v >= tB1) return kNoRow;
+    while (v >= s_rp[ri + 1]) ++ri;
+    return s_rs[ri] + (v - s_rp[ri]);
+  };
+  auto issue = [&](int t, int rows, bool values) {
+    copy_rows(rows, t < ntA ? (values ? Vslab : Kslab) : (values ? Vsel : Ksel), (values ? vnew : knew) + nrow * kD,
+              values ? sv : sk);
   };
   // One tile buffer per warp: the next K rows are requested as soon as the tile's logits are formed, the next V rows
   // after its P.V product, so that one of the two is always on its way (a second buffer would cost the second CTA).
   const int my_tiles = ntiles > warp ? (ntiles - warp + kStWarps - 1) / kStWarps : 0;
   if (!early && my_tiles > 0) {
-    issue(warp, false);
-    cp_async_commit();
-    issue(warp, true);
-    cp_async_commit();
+    const int rows = any_row(warp);
+#pragma unroll 1
+    for (int kv = 0; kv < 2; ++kv) {
+      issue(warp, rows, kv != 0);
+      cp_async_commit();
+    }
   }
   const float c2 = c.scale * kLog2eD;
   DecAcc acc;
@@ -564,7 +553,11 @@ __global__ void __launch_bounds__(kStThreads, 2)
     float Sl[2][4];
     dec_tile_logits(Sl, qa, sk, lane);
     __syncwarp();
-    if (next < ntiles) issue(next, false);
+    int rows = kNoRow;
+    if (next < ntiles) {
+      rows = any_row(next);
+      issue(next, rows, false);
+    }
     cp_async_commit();
     uint32_t pa[4];
     dec_tile_softmax(acc, Sl, pa, left, c2, lane);
@@ -572,7 +565,7 @@ __global__ void __launch_bounds__(kStThreads, 2)
     __syncwarp();
     dec_tile_values(acc, pa, sv, lane);
     __syncwarp();
-    if (next < ntiles) issue(next, true);
+    if (next < ntiles) issue(next, rows, true);
     cp_async_commit();
   }
   cp_async_wait<0>();
@@ -609,6 +602,17 @@ __global__ void __launch_bounds__(kStThreads, 2)
     const int to = idx / share;
     cluster.map_shared_rank(r_o, to)[rank * share + idx - to * share] = ot;
     if (e < S) *cluster.map_shared_rank(&r_ml[rank][hh], e) = make_float2(mx, lt);
+  }
+  if (appends) {
+    const long long wrow = c.paged ? pos - b.shift[bi] : pos;
+    __nv_bfloat16* slab = (lane < 16 ? c.Kc : c.Vc) + (unit * c.Hkv + g) * (size_t)c.SR * kD + ch * 8;
+    if (wrow < 0 || wrow >= c.SR) {  // cannot happen: the host keeps the window inside the slab
+      set_status(c, -2, pos);
+    } else {
+      *reinterpret_cast<uint4*>(slab + wrow * kD) = new_row;
+      if (c.paged && pos < c.Ls) *reinterpret_cast<uint4*>(slab + (size_t)pos * kD) = new_row;  // the sink's permanent row
+    }
+    if (g == 0 && lane == 0) c.votes[unit * c.Tpad + pos] = 0;
   }
   cluster.sync();  // (from here on a CTA reads its own shared memory only)
   for (int i = tid; i < share; i += nt) {

@@ -147,6 +147,19 @@ __device__ __forceinline__ unsigned order_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// Bin (0..254, 255: further away) of how far the upper 16 bits of a key lie below those of the largest key.  The upper 16 bits
+// have 128 steps per power of two: one step per bin for the nearest 128, then 4, 16 and 64, so that a K-th score
+// 2^22 times smaller than the best is still found by one histogram (with one step per bin throughout, two powers of two, the
+// planted streams of 128K tokens sent every other retrieval to the passes of the general select: 28K cycles instead of 9K).
+__device__ __forceinline__ unsigned dist_bin(unsigned d) {
+  // bins 0..127 | 128..191 from d = 128 | 192..223 from 384 | 224..254 from 896 | 255 from 2880
+  return min(min(d, 96u + (d >> 2)), min(min(168u + (d >> 4), 210u + (d >> 6)), 255u));
+}
+// the largest distance that falls into bin b
+__device__ __forceinline__ unsigned dist_last(unsigned b) {
+  return b < 128u ? b : b < 192u ? 4u * b - 381u : b < 224u ? 16u * b - 2673u : b < 255u ? 64u * b - 13377u : 0xffffffffu;
+}
+
 // Radix select of the K largest keys among KEY(0..N) (ties: lower index first), one 8-bit digit per pass from the top.
 // Writes the chosen indices, unordered, to s_ids and their number to *s_cnt (which the caller has zeroed).  Called by
 // every thread of the CTA; K < N.  R > 0 (keys that are expensive to read, 32-bit): up to R keys per thread are read
@@ -196,12 +209,12 @@ __device__ __forceinline__ void radix_select_top(KeyF&& KEY, int N, int K, unsig
     }
   };
   if (sizeof(KT) == 4 && s_ckey != nullptr) {
-    // Short cut for 32-bit keys (K is small against N): with the block's largest key M known, one histogram
-    // of how far a key's upper 16 bits lie below M's (256 bins; further away: the last bin) gives the smallest
-    // distance b within which at least K keys lie; those keys -- usually a few more than K -- are listed in shared
-    // memory and ranked against each other (key, then lower index).  Four barriers instead of twelve and about a
-    // third of the instructions of the four radix passes.  The radix passes below remain for the cases this does not
-    // cover: the K-th key more than 255 bins below M, or more than kSelCand keys within b (many equal keys).
+    // Short cut for 32-bit keys (K is small against N): with the block's largest key M known, one histogram of how far a
+    // key's upper 16 bits lie below M's (dist_bin) gives the smallest bin b within which at least K keys lie; those keys --
+    // usually a few more than K -- are listed in shared memory and ranked against each other (key, then lower index).  Four
+    // barriers instead of twelve and about a third of the instructions of the four radix passes.  The radix passes below
+    // remain for the cases this does not cover: the K-th key in the last bin, or more than kSelCand keys within b (many
+    // equal keys).
     int* s_cid = s_scan + 64;  // (s_scan[32..34]: scratch words)
     const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
     unsigned m = 0;
@@ -214,7 +227,7 @@ __device__ __forceinline__ void radix_select_top(KeyF&& KEY, int N, int K, unsig
     m = __reduce_max_sync(0xffffffffu, (unsigned)s_scan[lane < nw ? lane : 0]);
     const unsigned M16 = m >> 16;
     DigitRuns dr;
-    for_each_key([&](int, KT key) { dr.add(hist, (int)min(M16 - ((unsigned)key >> 16), 255u)); });
+    for_each_key([&](int, KT key) { dr.add(hist, (int)dist_bin(M16 - ((unsigned)key >> 16))); });
     dr.flush(hist);
     __syncthreads();
     if (tid < 32) {
@@ -225,8 +238,9 @@ __device__ __forceinline__ void radix_select_top(KeyF&& KEY, int N, int K, unsig
     __syncthreads();
     const unsigned bcut = (unsigned)s_scan[33];
     if (bcut < 255u) {
+      const unsigned dcut = dist_last(bcut);
       for_each_key([&](int s, KT key) {
-        if (M16 - ((unsigned)key >> 16) <= bcut) {
+        if (M16 - ((unsigned)key >> 16) <= dcut) {
           const int j = atomicAdd(&s_scan[34], 1);
           if (j < kSelCand) {
             s_ckey[j] = (unsigned)key;
