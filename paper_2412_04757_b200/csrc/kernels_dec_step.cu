@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kStThreads, 2)
   __shared__ int l_id[kMaxTopK];
   __shared__ unsigned r_max[kStMaxCluster];  // written by the other CTAs: their largest keys, their candidate counts
   __shared__ int r_cnt[kStMaxCluster];
-  __shared__ int s_all[2 * kMaxTopK], s_nall;
+  __shared__ int s_all[2 * kMaxTopK];
   __shared__ int s_sst[2 * kMaxTopK], s_sln[2 * kMaxTopK];
   __shared__ int s_rs[kMaxRanges], s_rl[kMaxRanges], s_rp[kMaxRanges + 1], s_nr;
   // host-memory pager: the unit cache as the first CTA sees it, the named units' slots
@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(kStThreads, 2)
       for (int t = tid; t < c.topk; t += nt) sel[t] = t < cnt ? s_ids[t] : -1;
     }
     if (c.persist) {
-      nall = union_with_persistent(c, unit, g, s_ids, cnt, s_scan, s_all, &s_nall);
+      nall = union_with_persistent(c, unit, g, s_ids, cnt, s_scan, s_all);
       ids_all = s_all;
     }
     if (tid < nall) {

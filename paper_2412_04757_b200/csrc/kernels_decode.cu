@@ -34,14 +34,27 @@ __global__ void __launch_bounds__(kDecThreads, kDecCtasPerSm) k_decode_attn(DevC
   const size_t unit = unit_of(c, b.seq[bi], layer);
   const size_t rb = (unit * c.Hkv + g) * (size_t)c.rcap;
   const int nr = min(c.rng_cnt[unit * c.Hkv + g], c.rcap);
-  if (tid == 0) {
+  // (a warp reads 32 ranges at a time and adds up their lengths: one thread reading one range after the other took as long as
+  // several tiles, in every CTA)
+  if (warp == 0) {
     int run = 0;
-    for (int i = 0; i < nr; ++i) {
-      rs[i] = c.host_kv ? (int)c.rng_koff[rb + i] : c.rng_start[rb + i];
-      rp[i] = run;
-      run += c.rng_len[rb + i];
+    for (int base = 0; base < nr; base += 32) {
+      const int i = base + lane;
+      const int start = i < nr ? (c.host_kv ? (int)c.rng_koff[rb + i] : c.rng_start[rb + i]) : 0;
+      const int len = i < nr ? c.rng_len[rb + i] : 0;
+      int inc = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      if (i < nr) {
+        rs[i] = start;
+        rp[i] = run + inc - len;
+      }
+      run += __shfl_sync(0xffffffffu, inc, 31);
     }
-    rp[nr] = run;
+    if (lane == 0) rp[nr] = run;
   }
   __syncthreads();
   const int total = rp[nr];
@@ -69,7 +82,10 @@ __global__ void __launch_bounds__(kDecThreads, kDecCtasPerSm) k_decode_attn(DevC
   const float c2 = c.scale * kLog2eD;
 
   // this lane copies rows (lane>>4) + 2i of every tile, 16 bytes at chunk (lane&15)
-  int ri = 0;
+  int ri = 0;  // range of this lane's last row: at first that of the warp's first token
+  for (int base = 0; base < nr; base += 32)
+    ri += __popc(__ballot_sync(0xffffffffu, base + lane < nr && rp[base + lane + 1] <= v0 + warp * kDTile));
+  ri = min(ri, max(nr - 1, 0));
   const int ch = lane & 15;
   auto issue = [&](int t, int stage) {
     const uint32_t sk = wbase + stage * (2 * kDTile * 256), sv = sk + kDTile * 256;

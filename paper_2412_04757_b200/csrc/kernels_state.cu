@@ -1492,7 +1492,7 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
   __shared__ unsigned s_ckey[kSelCand];
   __shared__ int s_rs[kMaxRanges], s_rl[kMaxRanges], s_pre[kMaxRanges + 1], s_nr;  // merged ranges, packed-row prefix
   __shared__ int s_sst[2 * kMaxTopK], s_sln[2 * kMaxTopK];  // extents of the selected spans
-  __shared__ int s_all[2 * kMaxTopK], s_nall;            // decode: this step's selection united with the persistent one
+  __shared__ int s_all[2 * kMaxTopK];            // decode: this step's selection united with the persistent one
   __shared__ int s_ko[kMaxRanges];  // pager, decode: first K row of every range, counted from the start of the K slabs
   // `parts` CTAs make the same selection for a (layer, KV head) and share the rows to be packed; the first one stores it
   const int g = blockIdx.x / parts, my_part = blockIdx.x % parts;
@@ -1526,10 +1526,21 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
     N = Eend > c.Ls ? (Eend + U - 1) / U - u0 : 0;
     for (int i = tid; i < N; i += nt) ukey[i] = 0u;  // below the key of every real score
     __syncthreads();
-    for (int s = tid; s < nspans; s += nt) {
-      const int st = c.span_start[unit * c.cap + s], ln = c.span_len[unit * c.cap + s];
-      const unsigned key = order_key(sc[s]);
-      for (int u = st / U; u <= (st + ln - 1) / U; ++u) atomicMax(&ukey[u - u0], key);
+    // (four spans a thread in flight)
+    for (int base = tid; base < nspans; base += 4 * nt) {
+      int st[4], ln[4];
+      float v[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int s = base + t * nt;
+        st[t] = s < nspans ? c.span_start[unit * c.cap + s] : 0;
+        ln[t] = s < nspans ? c.span_len[unit * c.cap + s] : 0;
+        v[t] = s < nspans ? sc[s] : 0.f;
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (base + t * nt < nspans)
+          for (int u = st[t] / U; u <= (st[t] + ln[t] - 1) / U; ++u) atomicMax(&ukey[u - u0], order_key(v[t]));
     }
     __syncthreads();
   }
@@ -1604,7 +1615,7 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
   const int* ids_all = s_ids;
   int nall = cnt;
   if (DECODE && c.persist) {
-    nall = union_with_persistent(c, unit, g, s_ids, cnt, s_scan, s_all, &s_nall);
+    nall = union_with_persistent(c, unit, g, s_ids, cnt, s_scan, s_all);
     ids_all = s_all;
   }
   if (tid < nall) {
@@ -1905,7 +1916,7 @@ __global__ void __launch_bounds__(1024) k_dec_retrieve(DevCtx c, int layer_begin
   __shared__ int s_scan[1024];
   __shared__ unsigned s_ckey[kSelCand];
   __shared__ int s_rs[kMaxRanges], s_rl[kMaxRanges], s_nr, s_sst[2 * kMaxTopK], s_sln[2 * kMaxTopK];
-  __shared__ int s_all[2 * kMaxTopK], s_nall;
+  __shared__ int s_all[2 * kMaxTopK];
   const int g = blockIdx.x;
   const int bi = blockIdx.y / layer_count, l = blockIdx.y % layer_count, layer = layer_begin + l;
   const int sq = b.seq[bi], pos = b.pos[bi], loc_begin = b.loc_begin[bi];
@@ -1989,7 +2000,7 @@ __global__ void __launch_bounds__(1024) k_dec_retrieve(DevCtx c, int layer_begin
   const int* ids_all = s_ids;
   int nall = cnt;
   if (c.persist) {
-    nall = union_with_persistent(c, unit, g, s_ids, cnt, s_scan, s_all, &s_nall);
+    nall = union_with_persistent(c, unit, g, s_ids, cnt, s_scan, s_all);
     ids_all = s_all;
   }
   if (tid < nall) {
@@ -2060,7 +2071,7 @@ __global__ void __cluster_dims__(kRetCluster, 1, 1) __launch_bounds__(kRetThread
   __shared__ int s_loc[kMaxTopK]; // this CTA's selected ids
   __shared__ int s_scan[kRetThreads];
   __shared__ int s_rs[kMaxRanges], s_rl[kMaxRanges], s_nr, s_sst[2 * kMaxTopK], s_sln[2 * kMaxTopK];
-  __shared__ int s_all[2 * kMaxTopK], s_nall;
+  __shared__ int s_all[2 * kMaxTopK];
   const int rank = (int)cluster.block_rank();
   const int g = blockIdx.x / kRetCluster;
   const int bi = blockIdx.y / layer_count, l = blockIdx.y % layer_count, layer = layer_begin + l;
@@ -2225,7 +2236,7 @@ __global__ void __cluster_dims__(kRetCluster, 1, 1) __launch_bounds__(kRetThread
   const int* ids_all = s_ids;
   int nall = cnt;
   if (c.persist) {
-    nall = union_with_persistent(c, unit, g, s_ids, cnt, s_scan, s_all, &s_nall);
+    nall = union_with_persistent(c, unit, g, s_ids, cnt, s_scan, s_all);
     ids_all = s_all;
   }
   if (tid < nall) {

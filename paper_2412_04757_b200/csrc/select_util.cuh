@@ -117,29 +117,27 @@ __device__ __forceinline__ int warp0_exclusive_scan(int* s_scan, int nt) {
 // persist_sel (ascending, -1 padded): the persistent mechanism of Sec. 3.5.  Writes the ascending, duplicate-free id
 // list to s_all and returns its length.  Called by every thread of the CTA; s_tmp has room for kMaxTopK ints.
 __device__ __forceinline__ int union_with_persistent(const DevCtx& c, size_t unit, int g, const int* s_ids, int cnt,
-                                                     int* s_tmp, int* s_all, int* s_nall) {
-  const int tid = threadIdx.x;
-  if (tid < c.topk) s_tmp[tid] = c.persist ? c.persist_sel[(unit * c.Hkv + g) * (size_t)c.topk + tid] : -1;
-  __syncthreads();
-  if (tid == 0) {
-    int a = 0, b = 0, n = 0;
-    while (b < c.topk && s_tmp[b] < 0) ++b;  // (-1 padding sits at the end, but tolerate it anywhere)
-    while (a < cnt || b < c.topk) {
-      const int va = a < cnt ? s_ids[a] : 0x7fffffff;
-      const int vb = b < c.topk && s_tmp[b] >= 0 ? s_tmp[b] : 0x7fffffff;
-      if (va == 0x7fffffff && vb == 0x7fffffff) break;
-      const int v = va < vb ? va : vb;
-      s_all[n++] = v;
-      if (va == v) ++a;
-      if (vb == v) {
-        ++b;
-        while (b < c.topk && s_tmp[b] < 0) ++b;
-      }
-    }
-    *s_nall = n;
+                                                     int* s_tmp, int* s_all) {
+  // an element's place is the number of smaller ones in both lists, a thread each (walking the two lists with one thread took
+  // some 6K cycles of every decode step)
+  const int tid = threadIdx.x, b = tid - kMaxTopK;  // threads 0..63: this step's ids, 64..127: the kept ones
+  const bool kept = b >= 0 && b < c.topk;
+  int v = -1;
+  if (tid < min(cnt, kMaxTopK)) v = s_ids[tid];
+  if (kept) {
+    v = c.persist ? c.persist_sel[(unit * c.Hkv + g) * (size_t)c.topk + b] : -1;
+    for (int i = 0; i < cnt; ++i) v = s_ids[i] == v ? -1 : v;  // (named by both: counted once)
+    s_tmp[b] = v;
+  }
+  const int n = __syncthreads_count(v >= 0);
+  if (v >= 0) {
+    int at = 0;
+    for (int i = 0; i < cnt; ++i) at += s_ids[i] < v;
+    for (int i = 0; i < c.topk; ++i) at += s_tmp[i] >= 0 && s_tmp[i] < v;
+    s_all[at] = v;
   }
   __syncthreads();
-  return *s_nall;
+  return n;
 }
 
 __device__ __forceinline__ unsigned order_key(float f) {
