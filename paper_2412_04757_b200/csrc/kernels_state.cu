@@ -1774,11 +1774,13 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
     uint4* Kdst = reinterpret_cast<uint4*>(c.Kg + gslab * kD);
     uint4* Vdst = reinterpret_cast<uint4*>(c.Vg + gslab * kD);
     const int ch = tid & 15, rpp = nt >> 4;  // 16-byte chunk of the row, rows per pass
-    for (int r0 = my_part * 4 * rpp + (tid >> 4); r0 < Rz; r0 += parts * 4 * rpp) {
+    // (rows dealt to the CTAs rpp at a time, so that few rows reach all of them)
+    const int step = parts * rpp;
+    for (int r0 = my_part * rpp + (tid >> 4); r0 < Rz; r0 += 4 * step) {
       uint4 kv[4], vv[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int r = r0 + i * rpp;
+        const int r = r0 + i * step;
         kv[i] = vv[i] = make_uint4(0u, 0u, 0u, 0u);
         if (r < R) {
           int lo = 0, hi = nr - 1;  // last range whose first packed row is <= r
@@ -1793,7 +1795,7 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int r = r0 + i * rpp;
+        const int r = r0 + i * step;
         if (r < Rz) {
           Kdst[(size_t)r * 16 + ch] = kv[i];
           Vdst[(size_t)r * 16 + ch] = vv[i];
