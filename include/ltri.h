@@ -299,8 +299,8 @@ enum {
   LTRI_BUF_CACHE_STATS = 12,  /* int64 [2]: units found in the cache / pulled from the host so far (all KV heads) */
   LTRI_BUF_BALLOT = 9,   /* int32 [top_k]: the layer's own ballot under LTRI_FLAG_COLLAB_VOTE (ascending unit numbers,
                             -1 padded; all -1 for a layer without a retrieval head) */
-  LTRI_BUF_ROWSTAT = 7   /* float [chunk][n_q_heads][2]: reference maximum m (logits * scale * log2(e); may lag the true
-                            row maximum by up to 8) and the matching row sum of exp2(logit - m) of the local softmax
+  LTRI_BUF_ROWSTAT = 7   /* float [chunk][n_q_heads][2]: reference maximum m (logits * scale * log2(e); may lie below the
+                            true row maximum by up to 24) and the matching row sum of exp2(logit - m) of the local softmax
                             of the last prefill call */
 };
 /* Copy an internal buffer of (seq, layer) to HOST memory `dst`; *bytes_out = full size.  Synchronises. */

@@ -256,9 +256,9 @@ cudaError_t launch_wait_probe(const DevCtx& c, long long short_limit, cudaStream
 // The kernels of a prefill call and of a decode step form a chain on one stream.  Launched through launch_chained,
 // a kernel's launch is prepared while its predecessor is still running and its CTAs start as soon as the predecessor
 // grid has finished; it touches global memory only after chain_wait(), which returns once that grid's writes are
-// visible.  No kernel releases its successor early: with one large CTA per SM (or a tuned number of them) the
-// successor's CTAs would only take resources away from the kernel that is still working (measured: decode 0.250
-// instead of 0.225 ms per step).  Launched the ordinary way, chain_wait() does nothing.
+// visible.  Kernels do not release their successors early (but see chain_release): with one large CTA per SM (or a tuned
+// number of them) the successor's CTAs would only take resources away from the kernel that is still working (measured: decode
+// 0.250 instead of 0.225 ms per step).  Launched the ordinary way, chain_wait() does nothing.
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the kernel launched behind this one start now instead of when this grid has finished.  Used where a kernel of a few
