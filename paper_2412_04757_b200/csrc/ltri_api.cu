@@ -915,18 +915,17 @@ constexpr int kStepSpans = 2560;
 // in three; 24 units, 639K rows, 52.9 and 56.9).
 constexpr int kOneCtaSpans = 12288;
 constexpr long long kStepRows = 768 * 1024;
-// With unit-granular retrieval a step may attend over thousands of scattered tokens per unit, which the split-KV kernel with
-// three CTAs per SM streams faster than a CTA that keeps one 16-token tile per warp on the way (12.7K tokens per unit, 64
-// units: 124 us a step against 130 us as clusters of four).  Spans are few tokens beside the recent ones, and the recent
-// ones stream well either way (64 units, 3K to 15K recent tokens: 46 to 101 us a step as clusters of four, 59 to 116 us as
-// separate launches).
-constexpr int kStepTokens = 1536;
+// With unit-granular retrieval a step may attend over thousands of scattered tokens per unit.  In clusters of four or more the one
+// launch is faster up to the longest steps measured (64 units, clusters of four: 12.5K tokens a unit 95 us a step against 112
+// separately, 20.7K tokens 127 and 146; 32 units, clusters of eight: 60 and 82, 80 and 103); in clusters of two a CTA keeps too few
+// bytes on the way (128 units would; 64 units forced to two: 117 and 112, 163 and 146).
+constexpr int kStepTokens = 5120, kStepTokensTwo = 1536;
 // A small index of which every unit is fetched costs the separate launches no selection and leaves them one range of tokens
 // (48 units, clusters of four: 5.7K tokens a unit, 51 us a step in one launch and 45 separately; 4.2K tokens, 39 and 41.  96
 // units, clusters of two: 2.6K tokens 49 and 46, 2.1K tokens 40 and 40.  16 units, clusters of eight: 8.8K tokens 41.5 and
 // 40.0, 6.7K tokens 33 and 33.  8 units, and 32 as clusters of eight, are faster in one launch up to 8.8K tokens.)
 static int step_tokens_all(int cluster, int units) {
-  return cluster <= 4 ? 1088 : cluster == 8 && units < 24 ? 864 : kStepTokens;
+  return cluster <= 4 ? 1088 : cluster == 8 && units < 24 ? 864 : kStepTokensTwo;
 }
 static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, long long ub) {
   const DevCtx& d = ctx->d;
@@ -945,7 +944,7 @@ static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, 
   for (int i = 4; i >= 1; --i) {
     const int cl = 1 << i;
     if (automatic ? known / cl < 64 && cl > 2 : cl != ctx->step_cluster) continue;
-    if (automatic && (d.unit > 0 ? tokens > kStepTokens * cl : ub > (long long)kStepSpans * cl)) continue;
+    if (automatic && (d.unit > 0 ? tokens > (long long)(cl > 2 ? kStepTokens : kStepTokensTwo) * cl : ub > (long long)kStepSpans * cl)) continue;
     if ((long long)units * cl > ctx->step_cap[i] || !dec_step_fits(d, (int)ub, e_max, cl)) continue;
     return automatic && all && tokens > step_tokens_all(cl, units) * cl ? 0 : cl;
   }
