@@ -1808,15 +1808,19 @@ __global__ void __launch_bounds__(512) k_topk(DevCtx c, int seq, int layer_begin
 // Host-memory pager (Sec. 3.4), data movement of a prefill call.  A task = one (named unit, KV head, layer): bring
 // the unit's rows to the slab the retrieved attention reads (a5 gather) -- from its cache slot, or over the bus from
 // the host mirror, in which case the rows also go into the slot the top-k kernel chose for the unit (unless the unit
-// is the one the indexed range ends in and still grows: that one is never cached).  A few small persistent CTAs
-// (128 threads, few registers, no dynamic shared memory) walk the tasks: small and few on purpose, so that each fits
-// onto an SM beside the one large CTA of the attention and map kernels and the bus transfer really runs under the
-// computation of the call's other layers instead of taking SMs away from it.  Eight 16-byte loads per thread are in
-// flight on the bus at a time, which keeps the bus busy with far fewer threads than the GPU has.
+// is the one the indexed range ends in and still grows: that one is never cached).  A few small persistent CTAs walk the tasks:
+// small and few on purpose, so that each fits onto an SM beside the one large CTA of the attention and map kernels and the
+// bus transfer really runs under the computation of the call's other layers instead of taking SMs away from it.
+// Registers decide whether one fits: those kernels' 18 warps of 96 leave 1024 free on two of an SM's four partitions, which is
+// a warp of 32 registers a thread.  With 64 a thread a CTA found room only where a large one had just left, and all of them
+// crowded onto four to eight SMs, which takes twice as long.  Four 16-byte loads per thread in flight, K rows first, then V rows.
+// 512-token calls of 8 / 12 / 16 / 32 layers, 32 CTAs of 64 registers a thread: 1.32 / 2.58 / 3.72 / 8.26 ms, 64 of 32: 1.29 /
+// 1.89 / 2.42 / 4.86.
 constexpr int kPullThreads = 128;
-constexpr int kPullCtas = 32;
+constexpr int kPullCtas = 64;
 
-__global__ void __launch_bounds__(kPullThreads) k_pull_pack(DevCtx c, int seq, int layer_begin, int layer_count, int max_units) {
+__global__ void __launch_bounds__(kPullThreads, 65536 / (kPullThreads * 32))
+    k_pull_pack(DevCtx c, int seq, int layer_begin, int layer_count, int max_units) {
   __shared__ int s_off;
   const int tid = threadIdx.x;
   const int ntasks = max_units * c.Hkv * layer_count;
@@ -1841,43 +1845,29 @@ __global__ void __launch_bounds__(kPullThreads) k_pull_pack(DevCtx c, int seq, i
   const size_t gslab = ((size_t)layer * c.Hkv + g) * (size_t)c.Rcap + s_off;
   uint4* Kdst = reinterpret_cast<uint4*>(c.Kg + gslab * kD);
   uint4* Vdst = reinterpret_cast<uint4*>(c.Vg + gslab * kD);
-  const uint4 *Ksrc, *Vsrc;
-  uint4 *Kslot = nullptr, *Vslot = nullptr;
-  const size_t hslab = (unit * c.Hkv + g) * (size_t)c.Tpad;
-  if (src >= 0) {
-    const size_t row = ((unit * c.Hkv + g) * (size_t)c.cache_units + (src & 0xffff)) * (size_t)U + (st - id * U);
-    Ksrc = reinterpret_cast<const uint4*>(c.Kcache + row * kD);
-    Vsrc = reinterpret_cast<const uint4*>(c.Vcache + row * kD);
-    if (src & 0x10000) {  // not there yet: over the bus, and into the slot as well
-      Kslot = reinterpret_cast<uint4*>(c.Kcache + row * kD);
-      Vslot = reinterpret_cast<uint4*>(c.Vcache + row * kD);
-      Ksrc = reinterpret_cast<const uint4*>(c.hostK + (hslab + st) * kD);
-      Vsrc = reinterpret_cast<const uint4*>(c.hostV + (hslab + st) * kD);
-    }
-  } else {
-    Ksrc = reinterpret_cast<const uint4*>(c.hostK + (hslab + st) * kD);
-    Vsrc = reinterpret_cast<const uint4*>(c.hostV + (hslab + st) * kD);
-  }
   const int n16 = ln * 16;
-  for (int i0 = tid; i0 < n16; i0 += 4 * kPullThreads) {
-    uint4 kv[4], vv[4];
+  const size_t hslab = (unit * c.Hkv + g) * (size_t)c.Tpad;
+  const size_t row = ((unit * c.Hkv + g) * (size_t)c.cache_units + (src & 0xffff)) * (size_t)U + (st - id * U);
+  const bool bus = src < 0 || (src & 0x10000);  // not in the cache: over the bus, and into its slot if it has one
+#pragma unroll 1
+  for (int kv = 0; kv < 2; ++kv) {
+    uint4* slot = src < 0 ? nullptr : reinterpret_cast<uint4*>((kv ? c.Vcache : c.Kcache) + row * kD);
+    const uint4* from = bus ? reinterpret_cast<const uint4*>((kv ? c.hostV : c.hostK) + (hslab + st) * kD) : slot;
+    uint4* to = kv ? Vdst : Kdst;
+    if (!bus) slot = nullptr;
+    for (int i0 = tid; i0 < n16; i0 += 4 * kPullThreads) {
+      uint4 v[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + u * kPullThreads;
-      if (i < n16) {
-        kv[u] = Ksrc[i];
-        vv[u] = Vsrc[i];
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * kPullThreads;
+        if (i < n16) v[u] = from[i];
       }
-    }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + u * kPullThreads;
-      if (i < n16) {
-        Kdst[i] = kv[u];
-        Vdst[i] = vv[u];
-        if (Kslot) {
-          Kslot[i] = kv[u];
-          Vslot[i] = vv[u];
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * kPullThreads;
+        if (i < n16) {
+          to[i] = v[u];
+          if (slot) slot[i] = v[u];
         }
       }
     }

@@ -42,3 +42,13 @@ def test_the_result_of_every_launch_is_looked_at(name):
     # a statement that begins with the launch drops its result, and the kernels behind it run on what it did not write
     text = open(os.path.join(CSRC, name)).read()
     assert not re.search(r"(^|[;{}]|\)|\belse)\s*\n\s*launch(_chained(_cluster)?)?\(", text), name
+
+
+def test_the_pull_kernel_fits_beside_the_large_kernels():
+    # 18 warps of 96 registers a thread leave 1024 registers on two of an SM's four partitions: a warp of 32 a thread.  What a
+    # kernel may use follows from its launch bounds: 65536 registers over the threads of the CTAs that an SM has to hold.
+    text = open(os.path.join(CSRC, "kernels_state.cu")).read()
+    threads = int(re.search(r"kPullThreads = (\d+);", text).group(1))
+    m = re.search(r"__launch_bounds__\(kPullThreads(?:, ([^;{}]*?))?\)\s+k_pull_pack\(", text)
+    ctas = eval((m.group(1) or "1").replace("kPullThreads", str(threads)).replace("/", "//"))
+    assert 65536 // (ctas * threads) <= 32
