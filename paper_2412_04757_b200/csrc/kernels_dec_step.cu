@@ -363,8 +363,8 @@ __global__ void __launch_bounds__(kStThreads, 2)
         }
       }
       if (general) {
-        // this CTA's best k of its slice in ascending id order, then the best k of the cluster's lists
-        cluster.sync();  // (the others are done with this CTA's histogram)
+        // this CTA's best k of its slice in ascending id order, then the best k of the cluster's lists, which take the place of
+        // the candidates' (their last remote writes lie before the cluster barrier that counted them)
         if (tid == 0) s_cnt = 0;
         __syncthreads();
         const int cf = min(c.topk, per);  // candidates of every full slice

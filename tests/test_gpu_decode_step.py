@@ -1,4 +1,7 @@
 """The one-launch decode step against the oracle, at the sizes where its splits and short cuts change."""
+import os
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -27,19 +30,33 @@ def test_one_launch_step(cluster, extra, monkeypatch):
     print(rep)
 
 
+STEP = open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "..", "paper_2412_04757_b200", "csrc",
+                         "kernels_dec_step.cu")).read()
+
+
+def step_constant(name):
+    return int(re.search(rf"constexpr int {name} = (\d+);", STEP).group(1))
+
+
 @pytest.mark.parametrize("cluster", [2, 4, 8, 16])
-@pytest.mark.parametrize("kind", ["thirds", "all", "one_slice", "far"])
+@pytest.mark.parametrize("kind", ["thirds", "all", "brim", "over", "one_slice", "far"])
 def test_selection_of_equal_and_of_distant_scores(kind, cluster, monkeypatch):
-    # The short cut of the cluster's select lists candidates near the largest score, 512 / cluster per CTA and 256 in all;
-    # beyond that the general select takes over.  700 loaded spans, ties go to the lower span:
+    # The short cut of the cluster's select lists candidates near the largest score, kStList / cluster per CTA and one per
+    # thread in all; beyond that the general select takes over.  Ties go to the lower span:
     #   thirds     three groups of 233 equal scores that cross all slices, the cut inside the first: the short cut
     #   all        700 equal scores
-    #   one_slice  the last CTA's whole slice equal and on top: more than its list holds
-    #   far        three scores more than 255 steps of the histogram above the others
+    #   brim       as many equal scores on top as the last CTA's list holds, or as are ranked in all: the short cut
+    #   over       one more
+    #   one_slice  the last CTA's whole slice equal and on top
+    #   far        three scores further above the others than the histogram reaches
+    limit = min(step_constant("kStList") // cluster, step_constant("kStThreads"))
+    N = 700 if kind in ("thirds", "all") else 1600
+    per = -(-N // cluster)
+    assert "kStCand = kStThreads;" in STEP and (kind != "one_slice" or per > step_constant("kStList") // cluster)
     monkeypatch.setenv("LTRI_DEC_CLUSTER", str(cluster))
-    L, hq, hkv, topk, N = 2, 8, 2, 5, 700
-    cfg = small_cfg(n_layers=L, n_q_heads=hq, n_kv_heads=hkv, context=1536, window=128, n_sink=16, top_k=topk,
-                    max_spans_per_region=64, decode_steps=1)
+    L, hq, hkv, topk = 2, 8, 2, 5
+    cfg = small_cfg(n_layers=L, n_q_heads=hq, n_kv_heads=hkv, context=1536 if N == 700 else 2048, window=128, n_sink=16,
+                    top_k=topk, max_spans_per_region=64, decode_steps=1)
     st = inputs.SyntheticStream(cfg, device="cuda:0")
     lts = [binding.Ltri(ph.params_of(cfg))]
     monkeypatch.setenv("LTRI_DEC_FUSED", "0")
@@ -64,13 +81,17 @@ def test_selection_of_equal_and_of_distant_scores(kind, cluster, monkeypatch):
             idx = top.clone()
         else:
             on_top = torch.zeros(N, dtype=torch.bool)
-            if kind == "one_slice":
-                on_top[-(-N // cluster) * (cluster - 1):] = True
-            else:
+            first = per * (cluster - 1)                # of the last CTA's slice
+            if kind == "far":
                 on_top[[3, 350, 699]] = True
+                low *= 2.0 ** -24
+            else:
+                on_top[first:first + {"brim": limit, "over": limit + 1, "one_slice": N}[kind]] = True
             idx = torch.where(on_top[:, None], top, low)
         idx = idx.to(torch.bfloat16)
         sc = torch.einsum("gnd,gd->gn", idx.double(), u).numpy()
+        if kind == "far":                              # the histogram ends 22.5 octaves below the largest score
+            assert all(np.log2(sc[g].max() / np.sort(sc[g])[-topk]) > 23 for g in range(hkv))
         want.append([sorted(np.argsort(-sc[g], kind="stable")[:topk].tolist()) for g in range(hkv)])
         for lt in lts:
             lt.ltri_debug_load_index(0, layer, E, spans, inputs.bf16_bits(idx))
