@@ -4,6 +4,7 @@ One or two layers of eight query heads on two KV heads are four or eight work it
 how many CTAs share one: four tiles of 128 keys two, eight four, sixteen eight.
 """
 import dataclasses
+import math
 
 import pytest
 import torch
@@ -31,9 +32,9 @@ def test_shared_work_items(window, context, extra):
 
 
 @pytest.mark.parametrize("window", [700, 1500])
-def test_a_key_of_very_large_norm_sends_the_whole_cluster_through_the_second_launch(window):
-    # the logits of one tile exceed every earlier maximum by hundreds of log2 units: the CTA that walks this tile asks for
-    # the second launch, which has to run in all CTAs that share the item
+def test_a_key_of_very_large_norm_in_one_tile_of_a_shared_item(window):
+    # the logits of one tile exceed every other maximum by hundreds of log2 units: the CTA that walks this tile ends with a
+    # reference far above those of the others, whose parts the merge scales to nothing
     cfg = small_cfg(n_layers=1, context=2304, window=window, top_k=12, decode_steps=0)
     sp = ph.StreamPair(cfg, [0], deep=False)
     st = inputs.SyntheticStream(cfg)
@@ -45,6 +46,52 @@ def test_a_key_of_very_large_norm_sends_the_whole_cluster_through_the_second_lau
     assert sp.lt.ltri_sync_status() == 0
     sp.lt.close()
     print(sp.rep)
+
+
+@pytest.mark.parametrize("clusters", ["8", "1"])          # a work item shared by CTAs, and one CTA per item
+@pytest.mark.parametrize("big", [
+    {300: 23.0}, {300: 25.0},                             # one key 23 or 25 log2 units above all others
+    {300: 23.0, 700: 46.0}, {300: 25.0, 700: 50.0},       # a second one as far above the first
+    {5: 40.0, 700: 63.0}, {300: 12.0, 500: 23.0, 800: 35.0},
+])
+def test_growth_of_the_running_maximum_around_the_rescale_line(big, clusters, monkeypatch):
+    # A thread moves its reference maximum, and rescales what it has accumulated, when a tile's maximum lies more than 24 log2
+    # units above it.  softmax_scale = ln 2 makes a logit its own log2: every query is one along the first axis, where the
+    # named keys have the given values and all others none.  The values of the others are so large that they carry about half
+    # of an output, which a wrong scale would show.
+    monkeypatch.setenv("LTRI_MAX_CLUSTER", clusters)
+    n, calls, hq, hkv = 128, 8, 8, 2
+    lt = binding.Ltri(binding.make_params(n_layers=1, n_q_heads=hq, n_kv_heads=hkv, max_tokens=n * calls, chunk=n, window=2000,
+                                          n_sink=16, top_k=4, softmax_scale=math.log(2.0)))
+    g = torch.Generator(device="cuda").manual_seed(11)
+    q = 0.01 * torch.randn(n * calls, hq, 128, generator=g, device="cuda")
+    q[..., 0] = 1.0
+    k = torch.randn(n * calls, hkv, 128, generator=g, device="cuda")
+    k[..., 0] = 0.0
+    v = 2.0 ** (max(big.values()) - 9) * (1.0 + torch.randn(n * calls, hkv, 128, generator=g, device="cuda"))
+    for tok, value in big.items():
+        k[tok, :, 0] = value
+        v[tok] *= 2.0 ** (9 - value)
+    q, k, v = (x.to(torch.bfloat16) for x in (q, k, v))
+    for t0 in range(0, n * calls, n):
+        out = lt.ltri_prefill_chunk(0, 0, 1, *(x[None, t0:t0 + n].contiguous() for x in (q, k, v)))[0]
+        keys, vals = (x[:t0 + n].double().repeat_interleave(hq // hkv, 1) for x in (k, v))
+        x = torch.einsum("nhd,thd->nht", q[t0:t0 + n].double(), keys) * math.log(2.0)
+        pos = torch.arange(t0 + n, device="cuda")
+        x.masked_fill_((pos > pos[t0:, None])[:, None], -math.inf)
+        want = torch.einsum("nht,thd->nhd", torch.softmax(x, -1), vals)
+        # per row: probabilities and outputs in bf16, each within 2^-9 of itself
+        err = (out.double() - want).norm(dim=-1) / want.norm(dim=-1)
+        assert float(err.max()) <= ph.REL_FRO, t0
+    if clusters == "1":    # a row's reference: that of the last key that outgrew it
+        ref = 0.0
+        for tok in sorted(big):
+            ref = big[tok] if big[tok] > ref + 24.0 else ref
+        m = lt.ltri_debug_read(binding.BUF_ROWSTAT, 0, 0)[:n, :, 0]
+        first = max(big[t] for t in big if t < 16) if min(big) < 16 else 0.0      # (in the first tile: the sink's)
+        assert abs(m - max(ref, first)).max() < 1.0
+    assert lt.ltri_sync_status() == 0
+    lt.close()
 
 
 @pytest.mark.parametrize("n_layers", [9, 18])

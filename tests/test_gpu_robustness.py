@@ -1,4 +1,4 @@
-"""GPU paths that ordinary streams never reach: keys of very large norm (the attention kernel's second pass),
+"""GPU paths that ordinary streams never reach: keys of very large norm,
 an expiring device-side wait, a span index loaded from outside, and host-side limits that must leave the context
 unchanged.  Everything here is finite input and bounded waiting: nothing is expected to fault, trap or hang."""
 import dataclasses
@@ -23,12 +23,11 @@ def _decode_inputs(st, pos):
 def test_keys_of_very_large_norm_give_the_exact_softmax(gain, max_ctas, monkeypatch):
     # Sec. 3.4 step 3: exact softmax over sink | retrieved | local | current for ANY finite input.  Two keys of
     # KV head 0 are scaled up so that the logits of the queries that point at their segment exceed every earlier
-    # tile's maximum by hundreds of log2 units (gain 30 and 12: the kernel's first pass, whose softmax reference
-    # moves one tile late, notices and a second pass with the true maximum on every tile redoes the CTA's items) or
-    # by an amount the late reference still absorbs (gain 1.4).  The keys sit in a later tile of the local window
-    # while they are local and in the packed slab of the retrieved spans afterwards (their own votes make them their
-    # spans' representatives, so the spans are retrieved).  KV head 1 keeps ordinary keys, so one launch has CTAs
-    # that take the second pass and CTAs that do not; with three CTAs every CTA walks many items in both passes.
+    # tile's maximum by hundreds of log2 units (gain 30 and 12: what was accumulated before is rescaled to nothing) or
+    # by a few (gain 1.4; the line at which a reference moves is in test_gpu_prefill_split.py).  The keys sit in a later
+    # tile of the local window while they are local and in the packed slab of the retrieved spans afterwards (their own
+    # votes make them their spans' representatives, so the spans are retrieved).  KV head 1 keeps ordinary keys; with
+    # three CTAs every CTA walks many items of both kinds.
     # The map comparison is left to the ordinary tests: with logits of this size the fp32 rounding of a logit (on
     # both sides) is worth dozens of Q20 units at a probability near one, beyond the tolerance that is meant for
     # bf16-sized inputs; spans (with the oracle's tie rule), index, selections and outputs are compared as always.
