@@ -932,17 +932,24 @@ constexpr int kStepSpans = 2560;
 // in three; 24 units, 639K rows, 52.9 and 56.9).
 constexpr int kOneCtaSpans = 12288;
 constexpr long long kStepRows = 768 * 1024;
-// With unit-granular retrieval a step may attend over thousands of scattered tokens per unit.  In clusters of four or more the one
-// launch is faster up to the longest steps measured (64 units, clusters of four: 12.5K tokens a unit 95 us a step against 112
-// separately, 20.7K tokens 127 and 146; 32 units, clusters of eight: 60 and 82, 80 and 103); in clusters of two a CTA keeps too few
-// bytes on the way (128 units would; 64 units forced to two: 117 and 112, 163 and 146).
+// With unit-granular retrieval a step may attend over thousands of scattered tokens per unit.  Every measured step of
+// clusters of four or more is faster in one launch, up to these tokens a CTA and beyond them, so the line is on the safe
+// side (us a step in one launch and separately; clusters of four, 64 units: 12.5K tokens a unit 95 and 112, 20.7K 127 and
+// 146; eight, 32 units: 10.8K 52 and 96, 35K 105 and 204, 68K 173 and 335; sixteen, 8 units: 10.8K 32 and 80, 68K 90 and
+// 298, 133K 147 and 628).  In clusters of two a CTA keeps fewer bytes on the way: 64 units forced to two, 12.5K tokens 117
+// and 112, 20.7K 163 and 146; 128 units take 52 and 69 at 2.6K tokens, and beyond the line still 63 and 80 at 3.7K, 134 and
+// 153 at 9.8K.  Steps of the host-memory pager wait for their pulls either way (64 units of 8.8K tokens, 32 slots: 2.69 and
+// 2.71 ms; 8 units: 403 and 572 us).
 constexpr int kStepTokens = 5120, kStepTokensTwo = 1536;
 // A small index of which every unit is fetched costs the separate launches no selection and leaves them one range of tokens
 // (48 units, clusters of four: 5.7K tokens a unit, 51 us a step in one launch and 45 separately; 4.2K tokens, 39 and 41.  96
 // units, clusters of two: 2.6K tokens 49 and 46, 2.1K tokens 40 and 40.  16 units, clusters of eight: 8.8K tokens 41.5 and
-// 40.0, 6.7K tokens 33 and 33.  8 units, and 32 as clusters of eight, are faster in one launch up to 8.8K tokens.)
+// 40.0, 6.7K tokens 33 and 33.  8 units, and 32 as clusters of eight, are faster in one launch up to 8.8K tokens, and with few
+// known tokens, which leave the separate attention few CTAs, beyond the line too: 1.6K known, 32 units, 12.4K tokens 46 and 117;
+// 8 units, 24.6K tokens 41 and 204.)
+constexpr int kStepTokensAll = 1536;
 static int step_tokens_all(int cluster, int units) {
-  return cluster <= 4 ? 1088 : cluster == 8 && units < 24 ? 864 : kStepTokensTwo;
+  return cluster <= 4 ? 1088 : cluster == 8 && units < 24 ? 864 : kStepTokensAll;
 }
 static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, long long ub) {
   const DevCtx& d = ctx->d;
@@ -961,7 +968,8 @@ static int step_cluster_size(const ltri_ctx* ctx, const DecBatch& b, int units, 
   for (int i = 4; i >= 1; --i) {
     const int cl = 1 << i;
     if (automatic ? known / cl < 64 && cl > 2 : cl != ctx->step_cluster) continue;
-    if (automatic && (d.unit > 0 ? tokens > (long long)(cl > 2 ? kStepTokens : kStepTokensTwo) * cl : ub > (long long)kStepSpans * cl)) continue;
+    const long long most = d.unit > 0 ? (long long)(cl > 2 ? kStepTokens : kStepTokensTwo) * cl : (long long)kStepSpans * cl;
+    if (automatic && (d.unit > 0 ? tokens : ub) > most) continue;
     if ((long long)units * cl > ctx->step_cap[i] || !dec_step_fits(d, (int)ub, e_max, cl)) continue;
     return automatic && all && tokens > step_tokens_all(cl, units) * cl ? 0 : cl;
   }

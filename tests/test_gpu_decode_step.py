@@ -180,6 +180,48 @@ def test_route_of_steps_that_fetch_every_unit(seqs, context, one_launch, monkeyp
         lt.close()
 
 
+@pytest.mark.parametrize("seqs,layers,top_k,window,persist,one_launch", [
+    (1, 8, 64, 3072, True, True),      # 64 units as clusters of four: 16384 fetched and 3.6K known tokens a unit
+    (1, 8, 64, 4608, True, False),     # 20480 are the line
+    (2, 8, 8, 896, False, True),       # 128 units as clusters of two: 1024 fetched and 1.6K known tokens a unit
+    (2, 8, 8, 2496, False, False),     # 3072 are the line
+])
+def test_route_of_steps_that_fetch_some_units(seqs, layers, top_k, window, persist, one_launch, monkeypatch):
+    # an index of more units than are fetched, with and without the selection kept from the last prefill call
+    chunk = 512
+    context = 2 * 64 * 128 + window + 2 * chunk if top_k == 64 else 4096 + window
+    context += -context % chunk
+    cfg = small_cfg(n_layers=layers, n_q_heads=16, n_kv_heads=8, context=context, chunk=chunk, window=window, n_seqs=seqs,
+                    unit_tokens=128, top_k=top_k, decode_steps=2, persist_decode=persist, max_spans_per_region=8)
+    st = inputs.SyntheticStream(cfg, device="cuda:0")
+    lts = [binding.Ltri(ph.params_of(cfg))]
+    monkeypatch.setenv("LTRI_DEC_FUSED", "0")
+    lts.append(binding.Ltri(ph.params_of(cfg)))
+    for t0, n in st.prefill_chunks():
+        q, k, v = st.tokens(t0, n)
+        for lt in lts:
+            for s in range(seqs):
+                lt.ltri_prefill_chunk(s, 0, layers, q, k, v)
+    E = lts[0].ltri_get_stats(0, 0).evicted_end
+    known = cfg.n_sink + context + 1 - E
+    tokens = known + min(E, top_k * 128 * (2 if persist else 1))
+    assert (E - 1) // 128 >= top_k and (tokens <= (20480 if layers * seqs == 8 else 3072)) == one_launch
+    for step in range(cfg.decode_steps):
+        q, k, v = (x.permute(1, 0, 2, 3).expand(seqs, -1, -1, -1).contiguous() for x in st.tokens(context + step, 1, kind=1))
+        outs = []
+        for lt, one in zip(lts, (one_launch, False)):
+            before = lt.ltri_launch_count()
+            outs.append(lt.ltri_decode_step(list(range(seqs)), 0, layers, q, k, v))
+            assert (lt.ltri_launch_count() - before == 1) == one
+        for s in range(seqs):
+            for l in range(layers):
+                assert (lts[0].ltri_get_selected(s, l) == lts[1].ltri_get_selected(s, l)).all()
+        assert float((outs[0].float() - outs[1].float()).abs().max()) <= ph.MAX_ABS
+    for lt in lts:
+        assert lt.ltri_sync_status() == 0
+        lt.close()
+
+
 @pytest.mark.parametrize("seqs,one_launch", [(3, True), (4, False)])
 def test_route_of_steps_over_a_large_index(seqs, one_launch, monkeypatch):
     # 18K spans and 4.3K known tokens: 24 units read 639K rows, 32 read 851K; the line lies at 768K
