@@ -17,6 +17,7 @@ constexpr int kMaxDecSplit = 32;
 constexpr int kMaxRanges = 2 * kMaxTopK + 2;  // sink + local + the spans of this step's and of the persistent selection
 constexpr float kMapMargin = 0.0078125f;          // safety margin (in log2 units) of the map pass's skip test
 constexpr float kMapScale = 0.4972997117f;         // 2^-(1 + kMapMargin)
+constexpr long long kRowSumQ = (1 << 20) + 512;  // largest row sum of a head's map: one, and half a unit per entry
 constexpr int kSegSms = 16;            // SMs that a layer of the one-launch segmenter occupies
 constexpr int kSegPasses = 3, kSegHistBits = 12;  // its histograms: 7 bits behind the leading one, 12 more, 12 more
 constexpr int kTokPad = 128;          // rows of slack after every K/V slab so tile over-reads stay inside it
@@ -196,7 +197,8 @@ cudaError_t launch_segment(const DevCtx& c, int seq, int layer_begin, int layer_
 // wait for it at its end (see chain_release).
 bool segment_in_one(const DevCtx& c, int layer_count);
 cudaError_t launch_segment_in_one(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start, int slot,
-                                  long long theta_q_abs, int n, int t0, const __nv_bfloat16* q, bool release, cudaStream_t s);
+                                  int theta_mode, float theta, long long theta_q_abs, int max_spans, int n, int t0,
+                                  const __nv_bfloat16* q, bool release, cudaStream_t s, bool tables, int seg_unit);
 cudaError_t launch_score_prefill(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s);
 // tensor-core version of launch_score_prefill (split-bf16 representatives)
 cudaError_t launch_score_prefill_mma(const DevCtx& c, const PrefillArgs& a, int span_bound, cudaStream_t s);

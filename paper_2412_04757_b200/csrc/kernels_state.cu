@@ -621,9 +621,9 @@ __device__ __forceinline__ void spans_and_reps(const DevCtx& c, const NmsArgs& a
   // Greedy NMS without a sort: the candidate the sorted sweep would reach next is the best one that is still alive
   // (key larger, or equal key and smaller anti-diagonal), so every round takes the block-wide maximum over the alive
   // candidates, keeps it, and lets every thread strike out its own candidates that the new span suppresses (or whose
-  // unit is full).  At most max_spans rounds of two barriers each instead of sorting up to 2047 keys.
+  // unit is full).  At most max_spans rounds instead of sorting up to 2047 keys.
   // Candidate of anti-diagonal cd: key = (S << 10) | (1023 - len) > 0; x = (cd - len) / 2, y = x + len.
-  // The rounds run in the first 8 warps, one barrier each: the warps' best meet in one of two arrays that the rounds use in
+  // The rounds run in the first 8 warps, one barrier each (three where units fill up): the warps' best meet in one of two arrays that the rounds use in
   // turn.  A key is held as its upper 32 significant bits (of the largest key) and the rest, so that one warp-wide maximum
   // nearly always names the winner.  (Bound: latency of the chain suppress - warp maximum - barrier - maximum.  With three
   // warp-wide reductions per maximum and a branch per candidate a round took 1300 cycles, now 750.)
@@ -979,7 +979,7 @@ __global__ void __launch_bounds__(1024) k_seg_nms(DevCtx c, NmsArgs a) {
 // Both go through L2: gathered from the other CTAs' shared memory, 64 KB a CTA, they took 8K cycles each time.
 // Bound: latency, a dozen dependent steps.  As four launches, with the map and a 64-bit table of sums going through L2 between
 // them, a layer took 36 us (256 tokens), 45 (512) and 66 (1024); now 20, 30 and 55.
-// The map's entries are not negative and a row's sum over all heads is at most Hq * (2^20 + 512), so RS fits 32 bits; PT, the
+// The map's entries are not negative and a row's sum over all heads is at most Hq * kRowSumQ, so RS fits 32 bits; PT, the
 // type of a block's column sums (at most 32 rows), is 32 bits up to 64 heads.
 constexpr int kSegThreads = 1024, kSegCluster = kSegSms, kSegBlocks = 2 * kSegCluster;
 constexpr int kSegFrac = 7;                         // the first histogram has 2^7 bins per power of two,
@@ -1301,15 +1301,16 @@ int segment_wide_clusters(const DevCtx& c) {
 bool segment_in_one(const DevCtx& c, int layer_count) { return layer_count <= c.seg_wide; }
 
 cudaError_t launch_segment_in_one(const DevCtx& c, int seq, int layer_begin, int layer_count, int m, int reg_start, int slot,
-                                  long long theta_q_abs, int n, int t0, const __nv_bfloat16* q, bool release, cudaStream_t s) {
+                                  int theta_mode, float theta, long long theta_q_abs, int max_spans, int n, int t0,
+                                  const __nv_bfloat16* q, bool release, cudaStream_t s, bool tables, int seg_unit) {
   SegArgs a;
-  a.nms = NmsArgs{seq, layer_begin, m, reg_start, slot, c.C, n, t0, q, 1, c.seg_unit};
-  a.theta_mode = c.theta_mode;
+  a.nms = NmsArgs{seq, layer_begin, m, reg_start, slot, max_spans, n, t0, q, tables ? 1 : 0, seg_unit};
+  a.theta_mode = theta_mode;
   a.bh = (m + kSegBlocks - 1) / kSegBlocks;
   a.release = release ? 1 : 0;
-  a.rank = quantile_rank(c.theta, m);
+  a.rank = quantile_rank(theta, m);
   a.thq = theta_q_abs;
-  a.thq1 = (long long)nearbyint((double)c.theta * (double)kQScale);
+  a.thq1 = (long long)nearbyint((double)theta * (double)kQScale);
   return launch_chained_cluster(seg_wide_sums(c) ? k_segment<unsigned long long> : k_segment<unsigned>,
                                 dim3(layer_count * kSegCluster), dim3(kSegThreads), kSegCluster, seg_smem(m, a.bh), s, c, a);
 }

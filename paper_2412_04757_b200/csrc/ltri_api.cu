@@ -260,6 +260,7 @@ struct ltri_ctx {
   bool spilled = false;      // ev_spill has been recorded at least once
   cudaEvent_t ev_up[2][kHostGroups] = {}, ev_run[2][kHostGroups] = {}, ev_down[2][kHostGroups] = {};
   int call_layers = 0;     // > 0 while the host-buffer entry issues a call of that many layers in groups
+  bool debug_one = false;  // testing aid (LTRI_DEBUG_SEGMENT=one): ltri_debug_segment_map takes the one-launch segmenter
   int ret_phase = 2;       // retrieved attention: 2 merges with the stored local state, 1 continues from it (testing aid)
   bool grp_used[2][kHostGroups] = {};  // the events of (set, group) have been recorded at least once
   long long host_calls = 0;
@@ -449,6 +450,7 @@ int ltri_create(const ltri_params* p, void* cuda_stream, ltri_ctx** out) {
   // Clusters that need a whole GPC, or the shared memory of several SMs, are used up to the size that the device can run; those
   // of up to eight small CTAs (segmenter, index build, large-index retriever) always.  (Testing aid: LTRI_MAX_CLUSTER, the
   // largest size of the former to count on.)
+  if (const char* f = std::getenv("LTRI_DEBUG_SEGMENT")) ctx->debug_one = std::strcmp(f, "one") == 0;
   const char* mc = std::getenv("LTRI_MAX_CLUSTER");
   const int most = mc ? std::atoi(mc) : 16;
   if (ctx->dec_fused < 0 && !ctx->d.vote)
@@ -778,8 +780,8 @@ int ltri_prefill_chunk(ltri_ctx* ctx, int seq, int layer_begin, int layer_count,
     if (seg_one) {
       {
         Scope sc(ctx, st, LTRI_K_SEGMENT, 1);
-        LTRI_CUDA(ctx, launch_segment_in_one(d, seq, ag.layer_begin, ag.layer_count, m, reg_start, slot, thq_abs, n_tokens,
-                                             t0, ag.q, own_first, st));
+        LTRI_CUDA(ctx, launch_segment_in_one(d, seq, ag.layer_begin, ag.layer_count, m, reg_start, slot, d.theta_mode, d.theta,
+                                             thq_abs, d.C, n_tokens, t0, ag.q, own_first, st, /*tables=*/true, d.seg_unit));
       }
       if (own_first) {
         Scope sc(ctx, st, LTRI_K_MAP, 1);
@@ -1339,14 +1341,27 @@ int ltri_debug_segment_map(ltri_ctx* ctx, const int32_t* Mq, int m, int theta_mo
   const DevCtx& d = ctx->d;
   if (m < 1 || m > d.chunk || theta_mode < 0 || theta_mode > 2 || max_spans < 1 || max_spans > d.C) return LTRI_EINVAL;
   if (theta_mode == 1 && !(theta >= 0.f && theta <= 1.f)) return LTRI_EINVAL;
+  const bool one = ctx->debug_one && segment_in_one(d, 1);
+  if (one)  // which counts on what a map of the library's own is like (see k_segment)
+    for (int i = 0; i < m; ++i) {
+      long long sum = 0;
+      for (int x = 0; x <= i; ++x) {
+        if (Mq[(size_t)i * m + x] < 0) return LTRI_EINVAL;
+        sum += Mq[(size_t)i * m + x];
+      }
+      if (sum > d.Hq * kRowSumQ) return LTRI_EINVAL;
+    }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   LTRI_CUDA(ctx, cudaMemcpy2DAsync(d.Mq, (size_t)d.chunk * sizeof(int), Mq, (size_t)m * sizeof(int),
                                    (size_t)m * sizeof(int), m, cudaMemcpyHostToDevice, st));
   long long thq = theta_q;
   if (theta_mode == 0) thq = (long long)std::nearbyint((double)theta * (double)d.Hq * (double)kQScale);
   const int slot = d.slots - 1;
-  LTRI_CUDA(ctx, launch_segment(d, 0, 0, 1, m, 0, slot, theta_mode == 1 ? 1 : 0, theta, thq, max_spans, 0, 0, nullptr,
-                                st));
+  if (one)
+    LTRI_CUDA(ctx, launch_segment_in_one(d, 0, 0, 1, m, 0, slot, theta_mode == 1 ? 1 : 0, theta, thq, max_spans, 0, 0, nullptr,
+                                         /*release=*/false, st, /*tables=*/false, 0));
+  else
+    LTRI_CUDA(ctx, launch_segment(d, 0, 0, 1, m, 0, slot, theta_mode == 1 ? 1 : 0, theta, thq, max_spans, 0, 0, nullptr, st));
   int cnt = 0;
   int rc = copy_back(ctx, &cnt, d.pend_cnt + slot, sizeof(int), st);
   if (rc) return rc;
