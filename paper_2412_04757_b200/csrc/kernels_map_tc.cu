@@ -373,6 +373,12 @@ typedef CUresult (*EncodeFnM)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
 
 constexpr int kMapSmem = kMapKT * 32768 + 65536 + 3 * 4096 + 1024;  // key tiles, two query stages, the offset tiles
 
+// A model of the launches, in tenths of a microsecond: a CTA starts and ends in 45 and takes 6.6 for a product of a key tile with
+// a query block (a CTA of four tiles and 16 blocks lives 45 us); the segmenter is through about 35 us after its start for 512
+// tokens.
+constexpr int kMapStart = 45, kMapProduct = 66;  // (kMapProduct: hundredths)
+static int segment_time(int n) { return 150 + n * 2 / 5; }
+
 template <int G>
 static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, MapPart part, bool late_wait,
                                    cudaStream_t s) {
@@ -400,10 +406,10 @@ static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const 
   const int nloc = part != kMapOwn && a.loc_begin >= c.Ls ? (a.t0 - a.loc_begin + 127) / 128 : 0;
   const int ncur = part != kMapBefore ? (a.n + 127) / 128 : 0;
   // Key tiles per CTA and splits of the query blocks.  With enough CTAs for several waves: four tiles, no split (the
-  // queries are re-read least).  Otherwise the pair that finishes first by a model of the launch in tenths of a microsecond: a
-  // CTA starts and ends in 45 and takes 6.6 for a product of a key tile with a query block (a CTA of four tiles and 16 blocks
-  // lives 45 us); beside the segmenter its 16 SMs per layer join in when it is through.  The map and the votes are integer
-  // sums, so the results do not depend on the choice.
+  // queries are re-read least).  Otherwise the pair that finishes first by the model above; beside the segmenter its 16 SMs per
+  // layer join in when it is through.  Against the best of the 32 pairs for either launch the choice costs a call of 1, 2, 4 or 7
+  // layers, 512 or 1024 tokens of 32 heads over a window of 4096, up to 2.3%.  The map and the votes are integer sums, so the
+  // results do not depend on it.
   const int nblk = (a.n + 128 / G - 1) / (128 / G);
   int kt = kMapKT, qs = 1;
   const int heads = c.Hkv * a.layer_count;
@@ -411,11 +417,11 @@ static cudaError_t launch_map_tc_g(const DevCtx& c, const PrefillArgs& a, const 
   const bool beside = part == kMapBefore;
   if (ctas_of(kMapKT, 1) <= (beside ? 6 : 3) * c.sms) {
     const int late = beside ? min(kSegSms * a.layer_count, c.sms - 1) : 0, now = c.sms - late;
-    const int from = 150 + a.n * 2 / 5;  // when the segmenter is through (about 35 us for 512 tokens)
+    const int from = segment_time(a.n);
     int best = 0;
     for (int k = kMapKT; k >= 1; --k)
       for (int q = 1; q <= 8 && q <= nblk; ++q) {
-        const int n = ctas_of(k, q), d = 45 + (66 * k * ((nblk + q - 1) / q) + 9) / 10;
+        const int n = ctas_of(k, q), d = kMapStart + (kMapProduct * k * ((nblk + q - 1) / q) + 9) / 10;
         // the first moment at which `now` CTAs at a time since the start and `late` at a time since `from` come to n
         int t = (n + now - 1) / now * d;
         for (int w = 1; late > 0 && from + w * d < t; ++w)
@@ -450,16 +456,20 @@ cudaError_t prepare_map_tc(const DevCtx& c) {
   return cudaErrorInvalidValue;
 }
 
-// The keys before the call take four products of a key tile with a query block per SM, or more.  (256 tokens over 576 of one
-// layer with two KV heads, 80 products: 803 us a request of eight calls in one launch, 813 in two; 512 tokens over 1024 with
-// eight, 1024 products: 5 us a call gained.)
+// The keys before the call are worth a launch of their own when they take three products of a key tile with a query block per
+// two SMs, or more: of 128 products a call gains -1.6 to 0.4 us by it, of 256 products -0.4 to 5.5 (seven shapes of one to four
+// layers), of 512 1.7 to 8.2, of 1024 9 to 13.  And when the segmenter leaves a third of the SMs, or they are done before it is:
+// seven layers leave 36 SMs, and calls of 256 to 1024 tokens of 32 query heads over windows of 2048 and 4096 lose 5 to 27 us of
+// 262 to 1207, while 512 tokens of eight single-query heads over 1024, 1792 products, gain 7 of 201.  (Six layers: -14 to 31.)
 bool map_pass_splits(const DevCtx& c, const PrefillArgs& a) {
   const long long tiles = (a.t0 - a.loc_begin + 127) / 128, blocks = ((long long)a.n * c.G + 127) / 128;
-  return tiles * blocks * c.Hkv * a.layer_count >= 4ll * c.sms;
+  const long long products = tiles * blocks * c.Hkv * a.layer_count, busy = (long long)kSegSms * a.layer_count;
+  if (2 * products < 3ll * c.sms) return false;
+  return 3 * busy <= 2ll * c.sms || products * kMapProduct <= (c.sms - busy) * 10 * segment_time(a.n);
 }
 
 cudaError_t launch_map_pass_tc(const DevCtx& c, const PrefillArgs& a, const void* kv_maps, MapPart part, bool late_wait,
-                                   cudaStream_t s) {
+                               cudaStream_t s) {
   switch (c.G) {
     case 1: return launch_map_tc_g<1>(c, a, kv_maps, part, late_wait, s);
     case 2: return launch_map_tc_g<2>(c, a, kv_maps, part, late_wait, s);

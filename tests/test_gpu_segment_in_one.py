@@ -44,19 +44,21 @@ def check(one, two, layers, votes):
 
 
 def splits_map_pass(lt, layer, n, per_call):
-    """Whether the call of n tokens that is just behind `layer` had a launch of its own for the keys before it: four products of
-    a key tile with a query block per SM, or more."""
+    """Whether the call of n tokens that is just behind `layer` had a launch of its own for the keys before it: three products of
+    a key tile with a query block per two SMs, or more, and a third of the SMs beside the segmenter or an early end."""
     p, s = lt.params, lt.ltri_get_stats(0, layer)
     t0 = s.tokens - n
     if s.evicted_end < p.n_sink or t0 <= s.evicted_end:
         return False
     products = -(-(t0 - s.evicted_end) // 128) * -(-n * p.n_q_heads // p.n_kv_heads // 128) * p.n_kv_heads * per_call
-    return products >= 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    sms, busy = torch.cuda.get_device_properties(0).multi_processor_count, 16 * per_call
+    return 2 * products >= 3 * sms and (3 * busy <= 2 * sms or products * 66 <= (sms - busy) * 10 * (150 + n * 2 // 5))
 
 
 @pytest.mark.parametrize("per_call,kw", [
     (1, dict()),
     (2, dict(theta=0.5)),
+    (7, dict(n_layers=7, n_q_heads=8, n_kv_heads=1)),                # the segmenter on three quarters of the SMs
     (1, dict(theta=0.0)), (1, dict(theta=1.0)),                    # first and last rank
     (2, dict(theta_mode=0, theta=0.002)),                          # a given threshold
     (2, dict(layer_theta=[0.8, 0.97], layer_nms_iou_milli=[0, 200], layer_rep_lambda=[1.0, 2.0], rep_mode=1)),
