@@ -623,9 +623,9 @@ __device__ __forceinline__ void spans_and_reps(const DevCtx& c, const NmsArgs& a
   // candidates, keeps it, and lets every thread strike out its own candidates that the new span suppresses (or whose
   // unit is full).  At most max_spans rounds instead of sorting up to 2047 keys.
   // Candidate of anti-diagonal cd: key = (S << 10) | (1023 - len) > 0; x = (cd - len) / 2, y = x + len.
-  // The rounds run in the first 8 warps, one barrier each (three where units fill up): the warps' best meet in one of two arrays that the rounds use in
-  // turn.  A key is held as its upper 32 significant bits (of the largest key) and the rest, so that one warp-wide maximum
-  // nearly always names the winner.  (Bound: latency of the chain suppress - warp maximum - barrier - maximum.  With three
+  // The rounds run in the first 8 warps, one barrier each (three where units fill up): the warps' best meet in one of two arrays
+  // that the rounds use in turn.  A key is held as its upper 32 significant bits (of the largest key) and the rest, so that one
+  // warp-wide maximum nearly always names the winner.  (Bound: latency of the chain suppress - warp maximum - barrier - maximum.  With three
   // warp-wide reductions per maximum and a branch per candidate a round took 1300 cycles, now 750.)
   constexpr int NT = 256, NW = NT / 32;
   __shared__ uint4 s_wbest[2][NW];

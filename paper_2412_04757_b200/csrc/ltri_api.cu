@@ -900,9 +900,9 @@ int ltri_prefill_chunk_host(ltri_ctx* ctx, int seq, int layer_begin, int layer_c
     if (rc != LTRI_OK) return rc;
     LTRI_CUDA(ctx, cudaEventRecord(ctx->ev_run[set][s.g], st));
     // Down, not before the next group's inputs are up.  The bus is what bounds this entry, and it moves least when a copy down
-    // starts in the middle of the copies up: 8 layers of 512 tokens, 16 calls, the copies alone, take 17.0 to 22.0 ms depending on
-    // how long after its inputs a group's output leaves, 18.1 at any such time when it waits (32 layers, 8 calls: 34.4 to 38.7
-    // and 35.0).  An 8K prompt of 8 layers: 20.4 -> 17.6 ms.
+    // starts in the middle of the copies up: 8 layers of 512 tokens, 16 calls, the copies alone, take 17.0 to 22.0 ms depending
+    // on how long after its inputs a group's output leaves, 18.1 at any such time when it waits (32 layers, 8 calls: 34.4 to
+    // 38.7 and 35.0).  An 8K prompt of 8 layers: 20.4 -> 17.6 ms.
     LTRI_CUDA(ctx, cudaStreamWaitEvent(ctx->s_down, ctx->ev_run[set][s.g], 0));
     if (i + 1 < ns) LTRI_CUDA(ctx, cudaStreamWaitEvent(ctx->s_down, ctx->ev_up[set][sl[i + 1].g], 0));
     LTRI_CUDA(ctx, cudaMemcpyAsync(static_cast<char*>(out_host) + s.qh, so + s.qs, s.qn, cudaMemcpyDeviceToHost, ctx->s_down));
